@@ -225,7 +225,7 @@ int run_filter(ctf_texture tex, const float *uv, const float *jac, const uint8_t
     } else if (tex->mode == CTF_EVAL_BLOCK) {
         e = ctf::launch_exact_filter(p, (int)alg, ro.tile_w, ro.mask_dim, stream);
     } else {
-        e = ctf::launch_mlp_filter(p, ctf::mlp_device_view(tex), (int)alg, ro.tile_w, ro.mask_dim, err, stream);
+        e = ctf::launch_mlp_filter(p, ctf::mlp_device_view(tex), tex->epi, (int)alg, ro.tile_w, ro.mask_dim, err, stream);
     }
     if (e != cudaSuccess) return cuda_fail(e, "filter launch");
     return CTF_OK;

@@ -363,6 +363,7 @@ bool aligned(const void *p, size_t a) { return (reinterpret_cast<uintptr_t>(p) %
 // their own, and, per kind, the other views' indices and item prefix.
 struct Plan {
     std::vector<BatchViewDev> views;
+    std::vector<const MlpEpilogue *> epi;  // of the views' textures (learned ones)
     std::vector<int> solo;
     std::vector<int> index[2];           // [0] block views, [1] learned views
     std::vector<long long> begin[2];
@@ -373,6 +374,7 @@ int make_plan(const ctf_view *views, int nviews, ctf_algorithm alg, uint64_t see
     if (!views || nviews < 1 || nviews > kMaxViews) return report(CTF_ERR_ARG, "nviews %d outside [1, %d]", nviews, kMaxViews);
     if ((int)alg < CTF_ALG_4TAP || (int)alg > CTF_ALG_MASK) return report(CTF_ERR_ARG, "unknown algorithm %d", (int)alg);
     plan->views.resize(nviews);
+    plan->epi.resize(nviews);
     for (int i = 0; i < nviews; ++i) {
         const ctf_view &v = views[i];
         if (!v.tex) return report(CTF_ERR_ARG, "view %d has no texture", i);
@@ -382,6 +384,7 @@ int make_plan(const ctf_view *views, int nviews, ctf_algorithm alg, uint64_t see
         if (np && (!v.uv || !v.jac || !v.out_rgba)) return report(CTF_ERR_ARG, "view %d: uv, jac and out_rgba needed", i);
         if (np && (!aligned(v.uv, 8) || !aligned(v.jac, 16) || !aligned(v.out_rgba, 16)))
             return report(CTF_ERR_ALIGN, "view %d: uv 8-byte, jac and out_rgba 16-byte alignment needed", i);
+        plan->epi[i] = &v.tex->epi;
         BatchViewDev &d = plan->views[i];
         std::memset(&d, 0, sizeof(d));
         ExactParams &p = d.p;
@@ -489,7 +492,7 @@ cudaError_t launch_plan(const Plan &plan, const DevPlan &dp, int alg, const Reso
         ExactParams p = plan.views[i].p;
         p.stats = stats;
         const cudaError_t le = plan.views[i].learned
-                                   ? launch_mlp_filter(p, plan.views[i].m, alg, r.tile_w, r.mask_dim, err, s)
+                                   ? launch_mlp_filter(p, plan.views[i].m, *plan.epi[i], alg, r.tile_w, r.mask_dim, err, s)
                                    : launch_exact_filter(p, alg, r.tile_w, r.mask_dim, s);
         if (le != cudaSuccess) return le;
     }
@@ -514,7 +517,8 @@ cudaError_t launch_plan(const Plan &plan, const DevPlan &dp, int alg, const Reso
         if (k == 1 && mlp_batch_pf_applies(alg, r.group_dedup)) {
             // learned views on the packed-group kernel (one group per fetch)
             e = launch_mlp_batch_pf(dp.views, (int)plan.views.size(), dp.index[1], dp.begin[1], b.nkind, b.total_items,
-                                    b.counter, stats, err, plan.views[plan.index[1][0]].m, alg, r.tile_w, r.mask_dim, s);
+                                    b.counter, stats, err, plan.views[plan.index[1][0]].m, *plan.epi[plan.index[1][0]], alg, r.tile_w,
+                                    r.mask_dim, s);
             if (e != cudaSuccess) return e;
             continue;
         }

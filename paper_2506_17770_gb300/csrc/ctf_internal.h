@@ -50,6 +50,7 @@ struct ctf_texture_s {
     __half *lat[2] = {nullptr, nullptr};  // device latent grids [gh][gw][8]
     int gw[2] = {0, 0}, gh[2] = {0, 0};
     void *img = nullptr;                  // device operand image (kImgBytes)
+    ctf::MlpEpilogue epi{};               // its biases and output scales, for kernel parameters
     // stored (quantised) parameters as floats, for ctf_mlp_export
     std::vector<float> s_lat[2], s_w1, s_b1, s_w2, s_b2, s_w3, s_b3, s_wscale[3], s_ascale[3];
 };
@@ -129,8 +130,8 @@ cudaError_t launch_bounded_wait_selftest(uint32_t polls, int *err, cudaStream_t 
 cudaError_t launch_bounds_selftest(int index, int *err, cudaStream_t stream);
 // Name of a BoundsSite (ctf_debug.cuh) for error messages.
 const char *bounds_site_name(int site);
-cudaError_t launch_mlp_filter(const ExactParams &p, const MlpDevice &m, int alg, int tile_w, int mask_dim, int *err,
-                              cudaStream_t stream);
+cudaError_t launch_mlp_filter(const ExactParams &p, const MlpDevice &m, const MlpEpilogue &ep, int alg, int tile_w,
+                              int mask_dim, int *err, cudaStream_t stream);
 MlpDevice mlp_device_view(const ctf_texture_s *t);
 // Uploads a learned texture's stored (already quantised) parameters: the
 // FP16 latent grids and the operand image (ctf_mlp_host.cu).  On failure the
@@ -164,8 +165,8 @@ bool mlp_filter_ext_applies(const ExactParams &p, int alg);
 cudaError_t prepare_mlp_filter_ext(int alg, int tile_w, int mask_dim);
 cudaError_t launch_mlp_filter_ext(const ExactParams &p, const MlpDevice &m, int alg, int tile_w, int mask_dim,
                                   int *err, cudaStream_t stream);
-cudaError_t launch_mlp_filter_pf(const ExactParams &p, const MlpDevice &m, int alg, int tile_w, int mask_dim,
-                                 int *err, cudaStream_t stream);
+cudaError_t launch_mlp_filter_pf(const ExactParams &p, const MlpDevice &m, const MlpEpilogue &ep, int alg, int tile_w,
+                                 int mask_dim, int *err, cudaStream_t stream);
 cudaError_t prepare_mlp_filter_ws(int alg, int tile_w, int mask_dim);
 cudaError_t launch_mlp_filter_ws(const ExactParams &p, const MlpDevice &m, int alg, int tile_w, int mask_dim,
                                  int *err, cudaStream_t stream);
@@ -182,13 +183,14 @@ static_assert(sizeof(ExactParams) % 16 == 0 && sizeof(ExactParams) <= 32 * 16, "
 // The learned views of a batch (other than per-pixel 4-tap and group_dedup)
 // on the packed-group kernel (ctf_mlp_ws2.cu): the views index[0..nkind)
 // of the table of nviews views, whose items (groups of 8 tiles) are numbered from
-// item_begin[k]; the CTAs take items from *counter (zero at launch).  m0 is
-// the first view's network, which the CTAs load first.
+// item_begin[k]; the CTAs take items from *counter (zero at launch).  m0 and
+// ep0 are the first view's network, which the CTAs load first.
 bool mlp_batch_pf_applies(int alg, int group_dedup);
 cudaError_t prepare_mlp_batch_pf(int alg, int tile_w, int mask_dim);
 cudaError_t launch_mlp_batch_pf(const BatchViewDev *views, int nviews, const int *index, const long long *item_begin,
                                 int nkind, long long total_items, unsigned long long *counter, unsigned long long *stats,
-                                int *err, const MlpDevice &m0, int alg, int tile_w, int mask_dim, cudaStream_t s);
+                                int *err, const MlpDevice &m0, const MlpEpilogue &ep0, int alg, int tile_w, int mask_dim,
+                                cudaStream_t s);
 
 // Error reporting shared by the C ABI translation units (ctf_api.cu).
 int report(int status, const char *fmt, ...);

@@ -56,4 +56,14 @@ struct MlpDevice {
     int *err;              // device error word (index checks of the debug build)
 };
 
+// What the hidden and output epilogues add and multiply, as in the operand
+// image (FP8: biases and output scales of layers 1 and 2 times the next
+// layer's inverse activation scale).  Passed to kernels as a parameter: an
+// epilogue then takes every value as a constant-bank operand of its packed
+// add, with no load.
+struct __align__(16) MlpEpilogue {
+    float b1[kMlpHidden], b2[kMlpHidden], b3[kMlpOut];
+    float s1[kMlpHidden], s2[kMlpHidden], s3[kMlpOut];
+};
+
 }  // namespace ctf

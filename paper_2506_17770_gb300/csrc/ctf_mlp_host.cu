@@ -6,6 +6,7 @@
 #include <cstdint>
 #include <cstring>
 #include <new>
+#include <utility>
 #include <vector>
 
 #include <cuda_fp16.h>
@@ -85,6 +86,10 @@ int upload_mlp_texture(ctf_texture_s *t) {
             }
         }
     }
+    const std::pair<float *, int> fields[6] = {{t->epi.b1, kImgB1}, {t->epi.b2, kImgB2}, {t->epi.b3, kImgB3},
+                                               {t->epi.s1, kImgS1}, {t->epi.s2, kImgS2}, {t->epi.s3, kImgS3}};
+    for (int i = 0; i < 6; ++i)
+        std::memcpy(fields[i].first, img.data() + fields[i].second, 4 * (i % 3 == 2 ? kMlpOut : kMlpHidden));
     cudaError_t e = ctf::dev_malloc(&t->img, kImgBytes);
     if (e == cudaSuccess) e = cudaMemcpy(t->img, img.data(), kImgBytes, cudaMemcpyHostToDevice);
     if (e != cudaSuccess) return report_cuda(e, "operand image upload");

@@ -15,9 +15,9 @@
 //     the output epilogue into the row values; then it gathers, filters and
 //     stores the group's pixels from the row values (warp w the tiles w and
 //     4 + w).
-// One consumer thread issues the MMAs and polls their barrier; the other
-// consumer threads wait at a named barrier (no polling).  Warps whose 32
-// rows all lie past the group's last row skip their epilogues.  The hidden
+// One consumer thread issues the MMAs; every consumer thread polls their
+// barrier.  Warps whose 32 rows all lie past the group's last row skip their
+// epilogues.  The hidden
 // activations stay in tensor memory: each epilogue writes them next to the
 // accumulator, and the next layer's MMAs read their A operand from there.
 // Three stages of group buffers (operand rows, whose first 4 KB the row
@@ -153,11 +153,15 @@ __device__ __forceinline__ bool bar_or(bool v) {
 // Hidden epilogue of a warp's 32 rows: TMEM columns [taddr, taddr + 64) of
 // this thread's row -> bias, ReLU -> the next layer's A operand, written to
 // TMEM columns from hcol on (FP16 pairs, or E4M3 quadruples, per 32-bit
-// column in K order).
-__device__ __forceinline__ void p_hidden_epilogue(uint32_t hcol, uint32_t taddr, const float *bias,
-                                                  const float *oscale, bool fp8) {
-    const float4 *b4 = reinterpret_cast<const float4 *>(bias);
-    const float4 *o4 = reinterpret_cast<const float4 *>(oscale);
+// column in K order).  `bias` and `oscale` point into the kernel's parameters
+// (every address is a compile-time offset there, so the packed adds take
+// them as constant-bank operands) or, in a batch whose group has another
+// network, into the operand image in shared memory.  From shared memory the
+// epilogue takes about 490 clocks with four CTAs on the SM, from the
+// parameters 270.
+template <typename F>
+__device__ __forceinline__ void p_hidden_epilogue(uint32_t hcol, uint32_t taddr, const F *bias, const F *oscale,
+                                                  bool fp8) {
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
         float d[16];
@@ -167,24 +171,21 @@ __device__ __forceinline__ void p_hidden_epilogue(uint32_t hcol, uint32_t taddr,
         if (!fp8) {
             uint32_t w[8];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const int k = 4 * i;
-                const float4 b = b4[(16 * q + k) / 4];
-                const float2 t0 = __fadd2_rn(make_float2(d[k], d[k + 1]), make_float2(b.x, b.y));
-                const float2 t1 = __fadd2_rn(make_float2(d[k + 2], d[k + 3]), make_float2(b.z, b.w));
-                w[2 * i] = relu_half2(t0.x, t0.y);
-                w[2 * i + 1] = relu_half2(t1.x, t1.y);
+            for (int i = 0; i < 8; ++i) {
+                const int k = 2 * i, c = 16 * q + k;
+                const float2 t = __fadd2_rn(make_float2(d[k], d[k + 1]), make_float2(bias[c], bias[c + 1]));
+                w[i] = relu_half2(t.x, t.y);
             }
             tc::tmem_st8(hcol + 8 * q, w);
         } else {
             uint32_t w[4];
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-                const int k = 4 * i;
-                const float4 b = b4[(16 * q + k) / 4], o = o4[(16 * q + k) / 4];
-                const float2 t0 = __ffma2_rn(make_float2(d[k], d[k + 1]), make_float2(o.x, o.y), make_float2(b.x, b.y));
-                const float2 t1 =
-                    __ffma2_rn(make_float2(d[k + 2], d[k + 3]), make_float2(o.z, o.w), make_float2(b.z, b.w));
+                const int k = 4 * i, c = 16 * q + k;
+                const float2 t0 = __ffma2_rn(make_float2(d[k], d[k + 1]), make_float2(oscale[c], oscale[c + 1]),
+                                             make_float2(bias[c], bias[c + 1]));
+                const float2 t1 = __ffma2_rn(make_float2(d[k + 2], d[k + 3]), make_float2(oscale[c + 2], oscale[c + 3]),
+                                             make_float2(bias[c + 2], bias[c + 3]));
                 w[i] = (uint32_t)relu_e4m3x2(t0.x, t0.y) | ((uint32_t)relu_e4m3x2(t1.x, t1.y) << 16);
             }
             tc::tmem_st4(hcol + 4 * q, w);
@@ -193,29 +194,33 @@ __device__ __forceinline__ void p_hidden_epilogue(uint32_t hcol, uint32_t taddr,
     tc::tmem_wait_st();
 }
 
-// One MMA layer's completion: thread 0 polls the barrier, the other
-// consumer threads wait at the consumer barrier, which also carries the
-// outcome to all of them.  Returns false (for every consumer thread alike)
-// if the MMAs did not complete within the bound.
-__device__ __forceinline__ bool p_layer_done(uint64_t *bar, uint32_t &phase, int *err) {
-    bool ok = true;
-    if (threadIdx.x == 0) ok = tc::mbar_wait(bar, phase, kMaxTries);
+// The end of one MMA layer, for one thread: every consumer thread polls the
+// MMA barrier itself.  (One polling thread and a named barrier for the others
+// took about 240 clocks longer per layer: 2700 instead of 2130 clocks for a
+// chain with four CTAs on the SM.)  Returns false if the MMAs did not
+// complete within the bound; the caller goes on and the threads agree on it
+// at their next barrier.
+__device__ __forceinline__ bool p_layer_wait(uint64_t *bar, uint32_t &phase) {
+    const bool ok = tc::mbar_wait(bar, phase, kMaxTries);
     phase ^= 1u;
-    __syncwarp();  // the barrier below is .aligned: warp 0 reconverges first
-    if (bar_or<1, kRows>(!ok)) {
-        if (threadIdx.x == 0) atomicExch(err, CTF_ERR_TIMEOUT);
-        return false;
-    }
+    __syncwarp();  // the TMEM accesses that follow are .aligned
     tc::fence_after_sync();
-    return true;
+    return ok;
 }
 
 // The three layers for the 128 rows of chain c of a stage (layer-1 operand
 // at sX).  TMEM columns: D (every layer's accumulator) at [0, 64), the
 // hidden activations H at [64, 96).  `live`: this warp has rows below the
-// group's row count (else it skips its epilogues).  Consumer threads only.
+// group's row count (else it skips its epilogues).  kParam: the network's
+// biases and scales are in ep (a kernel parameter), else in the operand
+// image.  Consumer threads only.  Returns false (for every consumer thread
+// alike) if layer 1 or 2 did not complete within the wait bound; `bad` is
+// set in the threads that gave up on layer 3, which the caller's next
+// barrier has to collect.
+template <bool kParam>
 __device__ __forceinline__ bool p_chain(unsigned char *sm, uint32_t tmem, uint64_t *bar, uint32_t &phase,
-                                        uint32_t sX, bool fp8, bool live, float4 &out, int *err) {
+                                        uint32_t sX, bool fp8, bool live, const MlpEpilogue &ep, float4 &out,
+                                        bool &bad, int *err) {
     const int tid = threadIdx.x, warp = tid >> 5;
     const float *b1 = reinterpret_cast<const float *>(sm + kImgB1);
     const float *b2 = reinterpret_cast<const float *>(sm + kImgB2);
@@ -242,10 +247,16 @@ __device__ __forceinline__ bool p_chain(unsigned char *sm, uint32_t tmem, uint64
         else tc::mma_f16(tmem, a, b, id64, false);
         tc::commit(bar);
     }
-    if (!p_layer_done(bar, phase, err)) return false;
-    if (live) p_hidden_epilogue(lane_base + 64, lane_base + 0, b1, s1, fp8);
+    bad |= !p_layer_wait(bar, phase);
+    if (live) {
+        if (kParam) p_hidden_epilogue(lane_base + 64, lane_base + 0, ep.b1, ep.s1, fp8);
+        else p_hidden_epilogue(lane_base + 64, lane_base + 0, b1, s1, fp8);
+    }
     tc::fence_before_sync();
-    cons_bar();
+    if (bar_or<1, kRows>(bad)) {
+        if (tid == 0) atomicExch(err, CTF_ERR_TIMEOUT);
+        return false;
+    }
     // ---- layer 2: D = H1 W2^T (D1 has been read)
     if (tid == 0) {
         tc::fence_after_sync();
@@ -256,11 +267,17 @@ __device__ __forceinline__ bool p_chain(unsigned char *sm, uint32_t tmem, uint64
         }
         tc::commit(bar);
     }
-    if (!p_layer_done(bar, phase, err)) return false;
+    bad |= !p_layer_wait(bar, phase);
     // the layer-2 MMAs have read H1, so H2 may overwrite it
-    if (live) p_hidden_epilogue(lane_base + 64, lane_base + 0, b2, s2, fp8);
+    if (live) {
+        if (kParam) p_hidden_epilogue(lane_base + 64, lane_base + 0, ep.b2, ep.s2, fp8);
+        else p_hidden_epilogue(lane_base + 64, lane_base + 0, b2, s2, fp8);
+    }
     tc::fence_before_sync();
-    cons_bar();
+    if (bar_or<1, kRows>(bad)) {
+        if (tid == 0) atomicExch(err, CTF_ERR_TIMEOUT);
+        return false;
+    }
     // ---- layer 3: D[0..16) = H2 W3^T
     if (tid == 0) {
         tc::fence_after_sync();
@@ -271,7 +288,7 @@ __device__ __forceinline__ bool p_chain(unsigned char *sm, uint32_t tmem, uint64
         }
         tc::commit(bar);
     }
-    if (!p_layer_done(bar, phase, err)) return false;
+    bad |= !p_layer_wait(bar, phase);
     if (live) {
         uint32_t r[4];
         tc::tmem_ld4(lane_base + 0, r);
@@ -281,7 +298,8 @@ __device__ __forceinline__ bool p_chain(unsigned char *sm, uint32_t tmem, uint64
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
             const float d = __uint_as_float(r[c]);
-            const float v = fp8 ? __fmaf_rn(d, s3[c], b3[c]) : __fadd_rn(d, b3[c]);
+            const float s = kParam ? ep.s3[c] : s3[c], b = kParam ? ep.b3[c] : b3[c];
+            const float v = fp8 ? __fmaf_rn(d, s, b) : __fadd_rn(d, b);
             o[c] = fminf(fmaxf(v, 0.f), 1.f);
         }
         out = make_float4(o[0], o[1], o[2], o[3]);
@@ -462,7 +480,8 @@ __device__ __forceinline__ void p_gather(const ExactParams &p, const TilePos &tp
 }
 
 template <int ALG, int TW, int MD, bool kStats, bool kFb, bool kTwo>
-__global__ void __launch_bounds__(kPThreads, kPCtasPerSm) mlp_filter_pf_kernel(const ExactParams p, const MlpDevice m, int *err) {
+__global__ void __launch_bounds__(kPThreads, kPCtasPerSm)
+    mlp_filter_pf_kernel(const ExactParams p, const MlpDevice m, const __grid_constant__ MlpEpilogue ep, int *err) {
     static_assert(!(kFb && kTwo), "fallbacks with two texels per lane run on the extension kernel");
     constexpr bool kList = ALG == ALG_LIST;
     constexpr int kPStages = PLayout<kFb, kList>::kStages;
@@ -527,8 +546,7 @@ __global__ void __launch_bounds__(kPThreads, kPCtasPerSm) mlp_filter_pf_kernel(c
             const int s = (int)(j % kPStages);
             const uint32_t par = (uint32_t)((j / kPStages) & 1);
             unsigned char *st = p_stage<kFb, kList>(sm, s);
-            bool ok = true;
-            if (tid == 0) ok = tc::mbar_wait(p_full(sm, s), par, kMaxTries);
+            bool ok = tc::mbar_wait(p_full(sm, s), par, kMaxTries);
             __syncwarp();
             if (bar_or<1, kRows>(!ok)) {
                 if (tid == 0) atomicExch(err, CTF_ERR_TIMEOUT);
@@ -541,12 +559,15 @@ __global__ void __launch_bounds__(kPThreads, kPCtasPerSm) mlp_filter_pf_kernel(c
             for (int c = 0; c < passes && ok; ++c) {
                 const bool live = kRows * c + 32 * warp < R;
                 float4 v;
-                ok = p_chain(sm, tmem, mma_bar, phase, sX + 4096u * (uint32_t)c, fp8, live, v, err);
+                bool bad = false;
+                ok = p_chain<true>(sm, tmem, mma_bar, phase, sX + 4096u * (uint32_t)c, fp8, live, ep, v, bad, err);
+                if (!ok) break;
                 // chain c's outputs overwrite operand rows of chain 0, which its
                 // layer-1 MMA has read; chain 1's operand rows (bytes 4096 on)
                 // are untouched
-                if (ok && live) outrow[ck(kRows * c + tid, 2 * kRows, p.err, kBndRow)] = v;
-                cons_bar();
+                if (live) outrow[ck(kRows * c + tid, 2 * kRows, p.err, kBndRow)] = v;
+                ok = !bar_or<1, kRows>(bad);
+                if (!ok && tid == 0) atomicExch(err, CTF_ERR_TIMEOUT);
             }
             if (!ok) break;
             {
@@ -576,17 +597,19 @@ __global__ void __launch_bounds__(kPThreads, kPCtasPerSm) mlp_filter_pf_kernel(c
                 unsigned char *st = p_stage<kFb, kList>(sm, s);
                 if (j >= kPStages) {
                     // the consumer has gathered group j - kPStages from this stage
-                    bool okd = true;
-                    if (lane == 0) okd = tc::mbar_wait(p_done(sm, s), (uint32_t)(((j - kPStages) / kPStages) & 1), kMaxTries);
+                    const bool okd = tc::mbar_wait(p_done(sm, s), (uint32_t)(((j - kPStages) / kPStages) & 1), kMaxTries);
                     __syncwarp();
+                    // (this barrier also says that every producer warp has read
+                    // the texel lists of group j - 1)
                     if (bar_or<2, kPProducerThreads>(!okd)) {
                         if (threadIdx.x == 128) atomicExch(err, CTF_ERR_TIMEOUT);
                         break;
                     }
+                } else {
+                    // every producer warp has read the texel lists of group j - 1
+                    __syncwarp();
+                    prod_bar();
                 }
-                // every producer warp has read the texel lists of group j - 1
-                __syncwarp();
-                prod_bar();
                 const long long first = grp * kGT;
                 const TilePos tp = tile_pos0(p, first);
 #pragma unroll 1
@@ -685,7 +708,8 @@ struct PfBatch {
 };
 
 template <int ALG, int TW, int MD, bool kStats>
-__global__ void __launch_bounds__(kPThreads, kPCtasPerSm) mlp_batch_pf_kernel(const PfBatch b, const MlpDevice m0) {
+__global__ void __launch_bounds__(kPThreads, kPCtasPerSm)
+    mlp_batch_pf_kernel(const PfBatch b, const MlpDevice m0, const __grid_constant__ MlpEpilogue ep0) {
     constexpr bool kList = ALG == ALG_LIST;
     constexpr int kPStages = PLayout<false, kList, true>::kStages;
     extern __shared__ __align__(1024) unsigned char sm[];
@@ -738,8 +762,7 @@ __global__ void __launch_bounds__(kPThreads, kPCtasPerSm) mlp_batch_pf_kernel(co
             const int s = (int)(j % kPStages);
             const uint32_t par = (uint32_t)((j / kPStages) & 1);
             unsigned char *st = p_stage<false, kList, true>(sm, s);
-            bool ok = true;
-            if (tid == 0) ok = tc::mbar_wait(p_full(sm, s), par, kMaxTries);
+            bool ok = tc::mbar_wait(p_full(sm, s), par, kMaxTries);
             __syncwarp();
             if (bar_or<1, kRows>(!ok)) {
                 if (tid == 0) atomicExch(err, CTF_ERR_TIMEOUT);
@@ -767,9 +790,13 @@ __global__ void __launch_bounds__(kPThreads, kPCtasPerSm) mlp_batch_pf_kernel(co
             for (int c = 0; c < passes && ok; ++c) {
                 const bool live = kRows * c + 32 * warp < R;
                 float4 v;
-                ok = p_chain(sm, tmem, mma_bar, phase, sX + 4096u * (uint32_t)c, fp8, live, v, err);
-                if (ok && live) outrow[ck(kRows * c + tid, 2 * kRows, err, kBndRow)] = v;
-                cons_bar();
+                bool bad = false;
+                ok = loaded == m0.img ? p_chain<true>(sm, tmem, mma_bar, phase, sX + 4096u * (uint32_t)c, fp8, live, ep0, v, bad, err)
+                                      : p_chain<false>(sm, tmem, mma_bar, phase, sX + 4096u * (uint32_t)c, fp8, live, ep0, v, bad, err);
+                if (!ok) break;
+                if (live) outrow[ck(kRows * c + tid, 2 * kRows, err, kBndRow)] = v;
+                ok = !bar_or<1, kRows>(bad);
+                if (!ok && tid == 0) atomicExch(err, CTF_ERR_TIMEOUT);
             }
             if (!ok) break;
             {
@@ -794,17 +821,19 @@ __global__ void __launch_bounds__(kPThreads, kPCtasPerSm) mlp_batch_pf_kernel(co
             unsigned char *st = p_stage<false, kList, true>(sm, s);
             if (j >= kPStages) {
                 // the consumer has gathered group j - kPStages from this stage
-                bool okd = true;
-                if (lane == 0) okd = tc::mbar_wait(p_done(sm, s), (uint32_t)(((j - kPStages) / kPStages) & 1), kMaxTries);
+                const bool okd = tc::mbar_wait(p_done(sm, s), (uint32_t)(((j - kPStages) / kPStages) & 1), kMaxTries);
                 __syncwarp();
+                // (this barrier also says that every producer warp has read
+                // the texel lists of the last group)
                 if (bar_or<2, kPProducerThreads>(!okd)) {
                     if (threadIdx.x == 128) atomicExch(err, CTF_ERR_TIMEOUT);
                     break;
                 }
+            } else {
+                // every producer warp has read the texel lists of the last group
+                __syncwarp();
+                prod_bar();
             }
-            // every producer warp has read the texel lists of the last group
-            __syncwarp();
-            prod_bar();
             int *bm = reinterpret_cast<int *>(st + kPBat);
             if (pt == 0) *reinterpret_cast<long long *>(st + kPBat + 8) = (long long)atomicAdd(b.counter, 1ull);
             prod_bar();
@@ -895,7 +924,7 @@ __global__ void __launch_bounds__(kPThreads, kPCtasPerSm) mlp_batch_pf_kernel(co
         atomicAdd(b.stats + threadIdx.x, block_stats[threadIdx.x]);
 }
 
-using PfFn = void (*)(const ExactParams, const MlpDevice, int *);
+using PfFn = void (*)(const ExactParams, const MlpDevice, const MlpEpilogue, int *);
 
 // Variants: kPlain, kFallback (C / C+ on Box and Mask), kTwoTexels (two
 // texels per lane on List Merge, Box and Mask).
@@ -980,8 +1009,8 @@ cudaError_t prepare_mlp_filter_pf(int alg, int tile_w, int mask_dim) {
     return cudaSuccess;
 }
 
-cudaError_t launch_mlp_filter_pf(const ExactParams &p, const MlpDevice &m, int alg, int tile_w, int mask_dim, int *err,
-                                 cudaStream_t stream) {
+cudaError_t launch_mlp_filter_pf(const ExactParams &p, const MlpDevice &m, const MlpEpilogue &ep, int alg, int tile_w,
+                                 int mask_dim, int *err, cudaStream_t stream) {
     const int var = p.fallback != 0 ? kFallback : (p.tpl == 2 ? kTwoTexels : kPlain);
     if (var == kFallback && !mlp_filter_pf_fallback_applies(p, alg)) return cudaErrorInvalidValue;
     if (var == kTwoTexels && !mlp_filter_pf_two_applies(p, alg)) return cudaErrorInvalidValue;
@@ -995,12 +1024,12 @@ cudaError_t launch_mlp_filter_pf(const ExactParams &p, const MlpDevice &m, int a
     const long long groups = (p.n_tiles + gt - 1) / gt;
     const long long cap = (long long)device_sm_count() * kPCtasPerSm;
     const int grid = (int)(groups < cap ? groups : cap);
-    fn<<<grid, kPThreads, pf_smem(var, alg), stream>>>(p, m, err);
+    fn<<<grid, kPThreads, pf_smem(var, alg), stream>>>(p, m, ep, err);
     return cudaGetLastError();
 }
 
 namespace {
-using BatchPfFn = void (*)(const PfBatch, const MlpDevice);
+using BatchPfFn = void (*)(const PfBatch, const MlpDevice, const MlpEpilogue);
 
 template <int TW, bool kStats>
 BatchPfFn batch_pf_pick(int alg, int md) {
@@ -1043,7 +1072,8 @@ cudaError_t prepare_mlp_batch_pf(int alg, int tile_w, int mask_dim) {
 
 cudaError_t launch_mlp_batch_pf(const BatchViewDev *views, int nviews, const int *index, const long long *item_begin,
                                 int nkind, long long total_items, unsigned long long *counter, unsigned long long *stats,
-                                int *err, const MlpDevice &m0, int alg, int tile_w, int mask_dim, cudaStream_t s) {
+                                int *err, const MlpDevice &m0, const MlpEpilogue &ep0, int alg, int tile_w, int mask_dim,
+                                cudaStream_t s) {
     BatchPfFn fn = batch_pf_kernel(alg, tile_w, mask_dim, stats != nullptr);
     if (!fn) return cudaErrorInvalidValue;
     if (total_items <= 0) return cudaSuccess;
@@ -1061,7 +1091,7 @@ cudaError_t launch_mlp_batch_pf(const BatchViewDev *views, int nviews, const int
     b.err = err;
     const long long cap = (long long)device_sm_count() * kPCtasPerSm;
     const int grid = (int)(total_items < cap ? total_items : cap);
-    fn<<<grid, kPThreads, batch_pf_smem(alg), s>>>(b, m0);
+    fn<<<grid, kPThreads, batch_pf_smem(alg), s>>>(b, m0, ep0);
     return cudaGetLastError();
 }
 
