@@ -335,7 +335,6 @@ const char *bounds_site_name(int site) {
     case kBndBlock: return "the texture's blocks";
     case kBndDecodeTable: return "the decode tables";
     case kBndRanks: return "a warp's rank slots";
-    case kBndListTable: return "a warp's List Merge table";
     case kBndFbTable: return "a warp's fallback table";
     case kBndLatent: return "a latent grid";
     case kBndTexList: return "a group's texel lists";

@@ -94,7 +94,6 @@ __global__ void __launch_bounds__(kBlockWarps * 32, batch_min_blocks<ALG>()) bat
     __shared__ unsigned long long block_stats[kNumStats];
     __shared__ int s_begin[kSmViews];
     __shared__ __align__(16) ExactParams s_params[kBlockWarps];  // each warp's current view
-    extern __shared__ __align__(16) unsigned char dyn_smem[];
     load_decode_tables(&tabs, b.tables);
     if (threadIdx.x < kNumStats) block_stats[threadIdx.x] = 0;
     const bool cached = b.nkind <= kSmViews && b.total_items < 0x7fffffffLL;
@@ -102,11 +101,6 @@ __global__ void __launch_bounds__(kBlockWarps * 32, batch_min_blocks<ALG>()) bat
         for (int i = threadIdx.x; i < b.nkind; i += blockDim.x) s_begin[i] = (int)__ldg(b.item_begin + i);
     const int *sb = cached ? s_begin : nullptr;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    ListTable *T = ALG == ALG_LIST ? reinterpret_cast<ListTable *>(dyn_smem) + warp : nullptr;
-    if (ALG == ALG_LIST) {
-#pragma unroll
-        for (int s = 0; s < 8; ++s) T->keys[lane * 8 + s] = kEmpty;
-    }
     if (kFb) fb_clear(&fb_tab[warp], lane);  // the fallback's texel table starts empty
     __syncthreads();
     const int tx = lane % TW, ty = lane / TW;
@@ -157,7 +151,7 @@ __global__ void __launch_bounds__(kBlockWarps * 32, batch_min_blocks<ALG>()) bat
             const uint32_t nidx = nby * (TH * W) + nbx * TW + lane_off;
             const Inputs nxt = load_inputs_any<kJac>(p, ninside, nidx);
             filter_tile<ALG, TW, MD, true, kFb ? kExtFallback | kExtTwo : 0>(p, cur, (int)(bx * TW) + tx, (int)(by * TH) + ty, inside, idx, lane, lt,
-                                           &tabs, T, rank_slots[warp], &fb_tab[warp], cnt);
+                                           &tabs, rank_slots[warp], &fb_tab[warp], cnt);
             bx = nbx;
             by = nby;
             inside = ninside;
@@ -194,11 +188,6 @@ __global__ void __launch_bounds__(kRows, 4) batch_mlp_kernel(const BatchParams b
     chain_setup(ch, sm, m0);
     if (threadIdx.x < kNumStats) block_stats[threadIdx.x] = 0;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    ListTable *T = reinterpret_cast<ListTable *>(sm + kSmList) + warp;
-    if (ALG == ALG_LIST) {
-#pragma unroll
-        for (int s = 0; s < 8; ++s) T->keys[lane * 8 + s] = kEmpty;
-    }
     const float *inv_a1 = reinterpret_cast<const float *>(sm + kImgA1);
     const uint32_t lt = lanemask_lt();
     Counters cnt;
@@ -245,9 +234,9 @@ __global__ void __launch_bounds__(kRows, 4) batch_mlp_kernel(const BatchParams b
                 __syncthreads();
             }
             if (ALG == ALG_4TAP)
-                ok = mlp_warp_tile<ALG, TW, MD>(V.p, V.m, ch, local * 4 + warp, lane, lt, T, cnt, inv_a1, b.err);
+                ok = mlp_warp_tile<ALG, TW, MD>(V.p, V.m, ch, local * 4 + warp, lane, lt, cnt, inv_a1, b.err);
             else
-                ok = mlp_group<ALG, TW, MD>(V.p, V.m, ch, local * kGroupTiles, lane, lt, T, cnt, inv_a1, b.err);
+                ok = mlp_group<ALG, TW, MD>(V.p, V.m, ch, local * kGroupTiles, lane, lt, cnt, inv_a1, b.err);
         }
     }
     if (b.stats && lane == 0) {
@@ -530,15 +519,14 @@ cudaError_t launch_plan(const Plan &plan, const DevPlan &dp, int alg, const Reso
             if (grid > useful) grid = useful;
             fn<<<(int)grid, kRows, kSmRequest, s>>>(b);
         } else {
-            const size_t smem = alg == ALG_LIST ? sizeof(ListTable) * kBlockWarps : 0;
             int per_sm = 0;
-            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kBlockWarps * 32, smem) != cudaSuccess ||
+            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kBlockWarps * 32, 0) != cudaSuccess ||
                 per_sm < 1)
                 per_sm = 1;
             long long grid = (long long)device_sm_count() * per_sm;
             const long long useful = (plan.items[k] + kBlockWarps - 1) / kBlockWarps;
             if (grid > useful) grid = useful;
-            fn<<<(int)grid, kBlockWarps * 32, smem, s>>>(b);
+            fn<<<(int)grid, kBlockWarps * 32, 0, s>>>(b);
         }
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;

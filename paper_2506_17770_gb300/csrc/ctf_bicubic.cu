@@ -76,6 +76,37 @@ __device__ __forceinline__ uint32_t block_bits(int t00, int bw, int w) {
     return m;
 }
 
+// List Merge of a tile whose bounding box is larger than 16 x 16 texels:
+// list_union of ctf_select.cuh for the 16 taps of the 4x4 footprint at
+// (ox, oy).  Returns the number of distinct texels (budget + 1 when there are
+// more); src[k] is the list index of tap k, (qx, qy) texel `lane` of the list.
+__device__ __forceinline__ int list_union16(bool active, int ox, int oy, int budget, int lane, int src[16], int &qx,
+                                            int &qy) {
+    uint32_t left = active ? 0xFFFFu : 0u;
+    int n = 0;
+#pragma unroll
+    for (int k = 0; k < 16; ++k) src[k] = 0;
+    while (true) {  // at most budget + 1 <= 33 iterations
+        const uint32_t any = __ballot_sync(FULL, left != 0);
+        if (any == 0) return n;
+        if (n == budget) return budget + 1;
+        const int from = __ffs(any) - 1, k = __ffs(left) - 1;
+        const int x = __shfl_sync(FULL, ox + (k & 3), from), y = __shfl_sync(FULL, oy + ((k >> 2) & 3), from);
+#pragma unroll
+        for (int t = 0; t < 16; ++t) {
+            if (((left >> t) & 1u) && ox + (t & 3) == x && oy + (t >> 2) == y) {
+                src[t] = n;
+                left &= ~(1u << t);
+            }
+        }
+        if (lane == n) {
+            qx = x;
+            qy = y;
+        }
+        ++n;
+    }
+}
+
 template <int ALG, int TW, int MD, int FILT, bool kStats>
 __global__ void __launch_bounds__(kThreads) bicubic_filter_kernel(const ExactParams p) {
     constexpr int TH = 32 / TW;
@@ -84,15 +115,9 @@ __global__ void __launch_bounds__(kThreads) bicubic_filter_kernel(const ExactPar
     __shared__ DecodeTables tabs;
     __shared__ int rank_slots[kWarps][32];
     __shared__ unsigned long long block_stats[kNumStats];
-    extern __shared__ __align__(16) unsigned char dyn_smem[];
 
     if (threadIdx.x < kNumStats) block_stats[threadIdx.x] = 0;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    ListTable *T = ALG == ALG_LIST ? reinterpret_cast<ListTable *>(dyn_smem) + warp : nullptr;
-    if (ALG == ALG_LIST) {
-#pragma unroll
-        for (int s = 0; s < 8; ++s) T->keys[lane * 8 + s] = kEmpty;
-    }
     load_decode_tables(&tabs, p.tables);
     __syncthreads();
     int *ranks = rank_slots[warp];
@@ -161,6 +186,7 @@ __global__ void __launch_bounds__(kThreads) bicubic_filter_kernel(const ExactPar
         int n = 0, minx = 0, miny = 0, bw = 0, mcls = 0;
         uint32_t Bw[NW];
         int pre[NW];
+        int lsrc[16], qlx = 0, qly = 0;  // List Merge with a larger box: list indices of the taps, texel `lane`
         if (ALG >= ALG_LIST) {
             mini = __any_sync(FULL, ps.active && is_minified(in.jac, fW, fH));
             if (!mini) {
@@ -176,7 +202,9 @@ __global__ void __launch_bounds__(kThreads) bicubic_filter_kernel(const ExactPar
                         n = bw * bh;
                         fits = true;
                     }
-                } else if (ALG == ALG_MASK) {
+                } else {
+                    // Mask Sampling, and List Merge with a box of at most 16 x 16
+                    // (the same set; larger boxes: one distinct texel at a time)
                     if (bw <= MD && bh <= MD) {
                         const int area = bw * bh;
                         mcls = area <= 32 ? 1 : 3;
@@ -193,48 +221,11 @@ __global__ void __launch_bounds__(kThreads) bicubic_filter_kernel(const ExactPar
                             }
                         }
                         fits = n <= p.budget;
+                    } else if (ALG == ALG_LIST) {
+                        mcls = 4;
+                        n = list_union16(ps.active, ox, oy, p.budget, lane, lsrc, qlx, qly);
+                        fits = n <= p.budget;
                     }
-                } else {  // List Merge: the 16 taps of every pixel into the warp's hash table
-                    int base = 0;
-                    bool over = false;
-#pragma unroll 1
-                    for (int k = 0; k < 16; ++k) {
-                        const unsigned long long key =
-                            ps.active ? (((unsigned long long)(uint32_t)(oy + (k >> 2) - miny) << 32) |
-                                         (uint32_t)(ox + (k & 3) - minx))
-                                      : (kEmpty - 1ull - (unsigned long long)lane);
-                        const uint32_t grp = __match_any_sync(FULL, key);
-                        const bool leader = ps.active && (__ffs(grp) - 1) == lane;
-                        bool inserted = false;
-                        unsigned slot = 0;
-                        if (leader) {
-                            unsigned h = hash_key(key) & 255u;
-                            for (int probe = 0; probe < 256; ++probe) {
-                                const unsigned long long old = atomicCAS(&T->keys[h], kEmpty, key);
-                                if (old == kEmpty) {
-                                    inserted = true;
-                                    slot = h;
-                                    break;
-                                }
-                                if (old == key) break;
-                                h = (h + 1) & 255u;
-                            }
-                        }
-                        const uint32_t newm = __ballot_sync(FULL, inserted);
-                        if (inserted) {
-                            const int index = base + __popc(newm & lt);
-                            T->index[ck(slot, 256, p.err, kBndListTable)] = (unsigned char)index;
-                            if (index < 64) T->list[ck(index, 64, p.err, kBndListTable)] = key;
-                        }
-                        base += __popc(newm);
-                        __syncwarp();
-                        if (base > p.budget) {
-                            over = true;
-                            break;
-                        }
-                    }
-                    n = base;
-                    fits = !over;
                 }
                 if (fits) {
                     if (p.edge_remap) {
@@ -271,12 +262,6 @@ __global__ void __launch_bounds__(kThreads) bicubic_filter_kernel(const ExactPar
                 count = 1;
             }
             if (inside) store_pixel(p, idx, res, (uint8_t)count);
-            if (ALG == ALG_LIST) {
-                __syncwarp();
-#pragma unroll
-                for (int s = 0; s < 8; ++s) T->keys[lane * 8 + s] = kEmpty;
-                __syncwarp();
-            }
             continue;
         }
 
@@ -292,7 +277,7 @@ __global__ void __launch_bounds__(kThreads) bicubic_filter_kernel(const ExactPar
         const int dx0 = ox - minx, dy0 = oy - miny, t00 = dy0 * bw + dx0;
         int qx = ps.ulx, qy = ps.uly;  // the texel this lane decodes
         int src[16];                   // lane holding tap k
-        if (ALG == ALG_BOX || (ALG == ALG_MASK && mcls == 1)) {
+        if (ALG == ALG_BOX || mcls == 1) {
             // a box of at most 32 texels: lane L decodes box position L
             const bool in_set = ALG == ALG_BOX ? lane < n : ((Bw[0] >> lane) & 1u) != 0;
             if (in_set) {
@@ -303,7 +288,7 @@ __global__ void __launch_bounds__(kThreads) bicubic_filter_kernel(const ExactPar
 #pragma unroll
             for (int k = 0; k < 16; ++k) src[k] = t00 + (k >> 2) * bw + (k & 3);
         } else {
-            if (ALG == ALG_MASK) {
+            if (ALG == ALG_MASK || mcls == 3) {
                 // ranks of the 16 taps; the pixels file each rank's position
 #pragma unroll
                 for (int k = 0; k < 16; ++k) {
@@ -320,29 +305,12 @@ __global__ void __launch_bounds__(kThreads) bicubic_filter_kernel(const ExactPar
                 }
                 __syncwarp();
             } else {
-#pragma unroll 1
-                for (int k = 0; k < 16; ++k) {
-                    int jk = 0;
-                    if (ps.active) {
-                        const unsigned long long key =
-                            ((unsigned long long)(uint32_t)(dy0 + (k >> 2)) << 32) | (uint32_t)(dx0 + (k & 3));
-                        unsigned h = hash_key(key) & 255u;
-                        for (int probe = 0; probe < 256; ++probe) {
-                            const unsigned long long kk = T->keys[h];
-                            if (kk == key) {
-                                jk = ck((int)T->index[h], 64, p.err, kBndListTable);
-                                break;
-                            }
-                            if (kk == kEmpty) break;
-                            h = (h + 1) & 255u;
-                        }
-                    }
-                    src[k] = jk;
-                }
+#pragma unroll
+                for (int k = 0; k < 16; ++k) src[k] = lsrc[k];
+                const int lx = __shfl_sync(FULL, qlx, my_i & 31), ly = __shfl_sync(FULL, qly, my_i & 31);
                 if (my_i < n) {
-                    const unsigned long long key = T->list[ck(my_i, 64, p.err, kBndListTable)];
-                    qx = minx + (int)(uint32_t)key;
-                    qy = miny + (int)(uint32_t)(key >> 32);
+                    qx = lx;
+                    qy = ly;
                 }
             }
             if (!full && p.edge_remap) {
@@ -367,12 +335,6 @@ __global__ void __launch_bounds__(kThreads) bicubic_filter_kernel(const ExactPar
         if (ps.active) res = acc;
         else count = 0;
         if (inside) store_pixel(p, idx, res, (uint8_t)count);
-        if (ALG == ALG_LIST) {
-            __syncwarp();
-#pragma unroll
-            for (int s = 0; s < 8; ++s) T->keys[lane * 8 + s] = kEmpty;
-            __syncwarp();
-        }
     }
 
     if (kStats) {
@@ -431,14 +393,13 @@ cudaError_t launch_bicubic_filter(const ExactParams &p, int alg, int tile_w, int
     if (!fn) return cudaErrorInvalidValue;
     if (p.n_tiles == 0) return cudaSuccess;
     if (p.n_tiles > 0x7fffffffLL) return cudaErrorInvalidValue;
-    const size_t smem = alg == ALG_LIST ? sizeof(ListTable) * kWarps : 0;
     int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kThreads, smem) != cudaSuccess || per_sm < 1)
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kThreads, 0) != cudaSuccess || per_sm < 1)
         per_sm = 1;
     const long long want = (p.n_tiles + kWarps - 1) / kWarps;
     const long long cap = (long long)device_sm_count() * per_sm;
     const int grid = (int)(want < cap ? want : cap);
-    fn<<<grid, kThreads, smem, stream>>>(p);
+    fn<<<grid, kThreads, 0, stream>>>(p);
     return cudaGetLastError();
 }
 

@@ -22,7 +22,6 @@ enum BoundsSite {
     kBndBlock,         // 8-byte block of a block texture (n = Wt/4 x Ht/4)
     kBndDecodeTable,   // the block decode tables in shared memory
     kBndRanks,         // a warp's rank slots (Mask Sampling)
-    kBndListTable,     // a warp's List Merge table and texel list
     kBndFbTable,       // a warp's fallback C / C+ texel table
     kBndLatent,        // a cell of a latent grid (n = gw x gh)
     kBndTexList,       // a group's texel lists (8 tiles x 32 entries)

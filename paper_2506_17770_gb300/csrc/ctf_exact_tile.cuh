@@ -375,7 +375,7 @@ constexpr int kExtFallback = 1, kExtTwo = 2;
 template <int ALG, int TW, int MD, bool kStats, int kExt = 0>
 __device__ __forceinline__ void filter_tile(const ExactParams &p, const Inputs &in, int px, int py, bool inside,
                                             uint32_t idx, int lane, uint32_t lt, const DecodeTables *tabs,
-                                            ListTable *T, int *ranks, FbTable *fbtab, Counters &cnt) {
+                                            int *ranks, FbTable *fbtab, Counters &cnt) {
     PixelSetup ps;
     ps.active = in.covered;
     setup_coords(in.uv, (float)p.Wt, (float)p.Ht, ps);
@@ -412,7 +412,7 @@ __device__ __forceinline__ void filter_tile(const ExactParams &p, const Inputs &
         }
     } else {
         const Selection sel =
-            select_tile<ALG, MD, kStats, true, (kExt & kExtTwo) != 0>(p, ps, in.jac, px, py, lane, lt, T, ranks, cnt);
+            select_tile<ALG, MD, kStats, true, (kExt & kExtTwo) != 0>(p, ps, in.jac, px, py, lane, lt, ranks, cnt);
         if ((kExt & kExtFallback) && ALG >= ALG_LIST && p.fallback != 0 && sel.path == PATH_FALLBACK_BUDGET) {
             // fallback C or C+ in place of one-tap STF
             FallbackArgs fa;

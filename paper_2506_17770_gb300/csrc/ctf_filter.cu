@@ -43,15 +43,9 @@ __global__ void __launch_bounds__(kThreads, kExt ? 4 : min_blocks<ALG>()) exact_
     __shared__ int rank_slots[kWarps][64];
     __shared__ FbTable fb_tab[kWarps];  // fallback C / C+ texel lookups
     __shared__ unsigned long long block_stats[kNumStats];
-    extern __shared__ __align__(16) unsigned char dyn_smem[];
 
     if (threadIdx.x < kNumStats) block_stats[threadIdx.x] = 0;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    ListTable *T = ALG == ALG_LIST ? reinterpret_cast<ListTable *>(dyn_smem) + warp : nullptr;
-    if (ALG == ALG_LIST) {
-#pragma unroll
-        for (int s = 0; s < 8; ++s) T->keys[lane * 8 + s] = kEmpty;
-    }
     if (kExt & kExtFallback) fb_clear(&fb_tab[warp], lane);  // the fallback's texel table starts empty
 
     const int tx = lane % TW, ty = lane / TW;
@@ -94,7 +88,7 @@ __global__ void __launch_bounds__(kThreads, kExt ? 4 : min_blocks<ALG>()) exact_
         const Inputs nxt = load_inputs_any<kJac>(p, ninside, nidx);
 
         filter_tile<ALG, TW, MD, kStats, kExt>(p, cur, (int)(bx * TW) + tx, (int)(by * TH) + ty, inside, idx, lane, lt,
-                                         &tabs, T, rank_slots[warp], &fb_tab[warp], cnt);
+                                         &tabs, rank_slots[warp], &fb_tab[warp], cnt);
 
         bx = nbx;
         by = nby;
@@ -183,14 +177,13 @@ cudaError_t launch_exact_filter(const ExactParams &p, int alg, int tile_w, int m
     if (!fn) return cudaErrorInvalidValue;
     if (p.n_tiles == 0) return cudaSuccess;
     if (p.n_tiles > 0x7fffffffLL) return cudaErrorInvalidValue;
-    const size_t smem = alg == ALG_LIST ? sizeof(ListTable) * kWarps : 0;
     int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kThreads, smem) != cudaSuccess || per_sm < 1)
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kThreads, 0) != cudaSuccess || per_sm < 1)
         per_sm = 1;
     const long long want = (p.n_tiles + kWarps - 1) / kWarps;
     const long long cap = (long long)device_sm_count() * per_sm;
     const int grid = (int)(want < cap ? want : cap);
-    fn<<<grid, kThreads, smem, stream>>>(p);
+    fn<<<grid, kThreads, 0, stream>>>(p);
     return cudaGetLastError();
 }
 

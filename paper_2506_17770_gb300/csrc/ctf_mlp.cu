@@ -84,11 +84,6 @@ __global__ void __launch_bounds__(kRows, 4) mlp_filter_kernel(const ExactParams 
     chain_setup(ch, sm, m);
     const float *inv_a1 = reinterpret_cast<const float *>(sm + kImgA1);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    ListTable *T = reinterpret_cast<ListTable *>(sm + kSmList) + warp;
-    if (ALG == ALG_LIST) {
-#pragma unroll
-        for (int s = 0; s < 8; ++s) T->keys[lane * 8 + s] = kEmpty;
-    }
     if (threadIdx.x < kNumStats) block_stats[threadIdx.x] = 0;
     __syncthreads();
     const uint32_t lt = lanemask_lt();
@@ -99,8 +94,8 @@ __global__ void __launch_bounds__(kRows, 4) mlp_filter_kernel(const ExactParams 
     const long long n_iter = (p.n_tiles + kTiles - 1) / kTiles;
     bool ok = true;
     for (long long it = blockIdx.x; it < n_iter && ok; it += gridDim.x) {
-        if (ALG == ALG_4TAP) ok = mlp_warp_tile<ALG, TW, MD>(p, m, ch, it * kTiles + warp, lane, lt, T, cnt, inv_a1, err);
-        else ok = mlp_group<ALG, TW, MD>(p, m, ch, it * kTiles, lane, lt, T, cnt, inv_a1, err);
+        if (ALG == ALG_4TAP) ok = mlp_warp_tile<ALG, TW, MD>(p, m, ch, it * kTiles + warp, lane, lt, cnt, inv_a1, err);
+        else ok = mlp_group<ALG, TW, MD>(p, m, ch, it * kTiles, lane, lt, cnt, inv_a1, err);
     }
     if (p.stats) {
         if (lane == 0) {

@@ -26,8 +26,7 @@ constexpr int kSmX = 14080;              // A operand of layer 1: 128 x 32 B
 constexpr int kSmH = kSmX + 4096;        // A operand of layers 2 and 3: 128 x 128 B
 constexpr int kSmBar = kSmH + 16384;     // mbarrier (8 B)
 constexpr int kSmTmem = kSmBar + 8;      // TMEM base address (4 B)
-constexpr int kSmList = kSmBar + 64;     // List Merge tables (4 x ListTable)
-constexpr int kSmRanks = kSmList + 4 * (int)sizeof(ListTable);  // Mask rank slots (4 x 32 ints)
+constexpr int kSmRanks = kSmBar + 64;    // rank slots of the larger masks (4 x 32 ints)
 // Packed groups of 8 tiles (collaborative algorithms and STF): per pixel the
 // fractions (s, t) and a packed word, the texel value of every list row, the
 // texels per tile; the texel lists themselves sit in the X buffer until the
@@ -390,7 +389,7 @@ __device__ __forceinline__ void chain_teardown(const Chain &ch) {
 // gather and filter, the store.  Returns false if the chain gave up.
 template <int ALG, int TW, int MD>
 __device__ __forceinline__ bool mlp_warp_tile(const ExactParams &p, const MlpDevice &m, Chain &ch, long long tile,
-                                              int lane, uint32_t lt, ListTable *T, Counters &cnt,
+                                              int lane, uint32_t lt, Counters &cnt,
                                               const float *inv_a1, int *err) {
     constexpr int TH = 32 / TW;
     unsigned char *sm = ch.sm;
@@ -464,7 +463,7 @@ __device__ __forceinline__ bool mlp_warp_tile(const ExactParams &p, const MlpDev
     } else {
         Selection sel;
         if (valid) {
-            sel = select_tile<ALG, MD, true>(p, ps, jac, px, py, lane, lt, T,
+            sel = select_tile<ALG, MD, true>(p, ps, jac, px, py, lane, lt,
                                           reinterpret_cast<int *>(sm + kSmRanks) + 32 * (threadIdx.x >> 5), cnt);
         } else {
             sel.path = PATH_EMPTY;
@@ -531,7 +530,7 @@ __device__ __forceinline__ bool mlp_warp_tile(const ExactParams &p, const MlpDev
 // independent.  Returns false (for every thread alike) if a chain gave up.
 template <int ALG, int TW, int MD>
 __device__ __forceinline__ bool mlp_group(const ExactParams &p, const MlpDevice &m, Chain &ch, long long first,
-                                          int lane, uint32_t lt, ListTable *T, Counters &cnt, const float *inv_a1,
+                                          int lane, uint32_t lt, Counters &cnt, const float *inv_a1,
                                           int *err) {
     constexpr int TH = 32 / TW;
     unsigned char *sm = ch.sm;
@@ -573,7 +572,7 @@ __device__ __forceinline__ bool mlp_group(const ExactParams &p, const MlpDevice 
         setup_coords(uv, fW, fH, ps);
         Selection sel;
         if (valid) {
-            sel = select_tile<ALG, MD, true, false>(p, ps, jac, px, py, lane, lt, T, ranks, cnt);
+            sel = select_tile<ALG, MD, true, false>(p, ps, jac, px, py, lane, lt, ranks, cnt);
         } else {
             sel.path = PATH_EMPTY;
             sel.A = 0;

@@ -50,7 +50,7 @@ static_assert(kSmExtRanks % 16 == 0 && kSmExtRanks + 4 * 64 * 4 <= kSmCount,
 
 template <int ALG, int TW, int MD>
 __device__ __forceinline__ bool ext_warp_tile(const ExactParams &p, const MlpDevice &m, Chain &ch, long long tile,
-                                              int lane, uint32_t lt, ListTable *T, FbTable *fbt, int *ranks,
+                                              int lane, uint32_t lt, FbTable *fbt, int *ranks,
                                               Counters &cnt, const float *inv_a1, int *err) {
     constexpr int TH = 32 / TW;
     unsigned char *sm = ch.sm;
@@ -75,7 +75,7 @@ __device__ __forceinline__ bool ext_warp_tile(const ExactParams &p, const MlpDev
     setup_coords(uv, (float)p.Wt, (float)p.Ht, ps);
     Selection sel;
     if (valid) {
-        sel = select_tile<ALG, MD, true, true, true>(p, ps, jac, px, py, lane, lt, T, ranks, cnt);
+        sel = select_tile<ALG, MD, true, true, true>(p, ps, jac, px, py, lane, lt, ranks, cnt);
     } else {
         sel.path = PATH_EMPTY;
         sel.A = 0;
@@ -174,13 +174,8 @@ __global__ void __launch_bounds__(kRows, 3) mlp_filter_ext_kernel(const ExactPar
     chain_setup(ch, sm, m);
     const float *inv_a1 = reinterpret_cast<const float *>(sm + kImgA1);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    ListTable *T = reinterpret_cast<ListTable *>(sm + kSmList) + warp;
     FbTable *fbt = reinterpret_cast<FbTable *>(sm + kSmFb) + warp;
     int *ranks = reinterpret_cast<int *>(sm + kSmExtRanks) + 64 * warp;
-    if (ALG == ALG_LIST) {
-#pragma unroll
-        for (int s = 0; s < 8; ++s) T->keys[lane * 8 + s] = kEmpty;
-    }
     fb_clear(fbt, lane);  // the fallback's texel table starts empty
     if (threadIdx.x < kNumStats) block_stats[threadIdx.x] = 0;
     __syncthreads();
@@ -191,7 +186,7 @@ __global__ void __launch_bounds__(kRows, 3) mlp_filter_ext_kernel(const ExactPar
     const long long n_iter = (p.n_tiles + 3) / 4;
     bool ok = true;
     for (long long it = blockIdx.x; it < n_iter && ok; it += gridDim.x)
-        ok = ext_warp_tile<ALG, TW, MD>(p, m, ch, it * 4 + warp, lane, lt, T, fbt, ranks, cnt, inv_a1, err);
+        ok = ext_warp_tile<ALG, TW, MD>(p, m, ch, it * 4 + warp, lane, lt, fbt, ranks, cnt, inv_a1, err);
     if (p.stats && lane == 0) {
 #pragma unroll
         for (int i = 0; i < kNumStats; ++i)

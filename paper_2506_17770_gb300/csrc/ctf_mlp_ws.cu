@@ -49,9 +49,9 @@ static_assert(128 * kWsConsumerRegs + 32 * kWsProducerWarps * kWsProducerRegs ==
 constexpr int kWsSlotsPerProducer = kGroupTiles / kWsProducerWarps;  // pixel tiles of the group per producer warp
 
 // Shared memory: the chain's operand image, X, H, MMA barrier and TMEM slot
-// (ctf_mlp_chain.cuh offsets below kSmList), then the producers' Mask rank
+// (ctf_mlp_chain.cuh offsets below kSmRanks), then the producers' Mask rank
 // slots, two stages of group buffers and the hand-over barriers.
-constexpr int kWsRanks = kSmList;                            // producer warps x 32 ints
+constexpr int kWsRanks = kSmRanks;                           // producer warps x 32 ints
 constexpr int kWsStage0 = kWsRanks + kWsProducerWarps * 32 * 4;
 constexpr int kWsTex = 0;                                    // 256 x int2 texel lists (slot g at 32 g)
 constexpr int kWsST = kWsTex + 256 * 8;                      // 256 x float2 (s, t)
@@ -283,7 +283,7 @@ __device__ __forceinline__ void ws_step1(const ExactParams &p, long long first, 
     setup_coords(uv, (float)p.Wt, (float)p.Ht, ps);
     Selection sel;
     if (valid) {
-        sel = select_tile<ALG, MD, true, false>(p, ps, jac, px, py, lane, lt, nullptr, ranks, cnt);
+        sel = select_tile<ALG, MD, true, false>(p, ps, jac, px, py, lane, lt, ranks, cnt);
     } else {
         sel.path = PATH_EMPTY;
         sel.A = 0;

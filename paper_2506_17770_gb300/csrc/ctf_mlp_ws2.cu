@@ -92,21 +92,17 @@ constexpr int kPQ = kPRows + 16;                 // fallback variant: 256 x int2
 constexpr int kPUL = kPQ + 2048;                 // fallback variant: 256 x int2 upper-left texel of the footprint
 
 // kFb: the variant with fallbacks C / C+ (two stages, to make room for the
-// texel tables and the per-pixel texels the blend of eq. 1 needs); kList:
-// List Merge (two stages and a List Merge table per producer warp, at the
-// place of the fallback tables).
+// texel tables and the per-pixel texels the blend of eq. 1 needs).
 // kBatch: the persistent batch kernel, whose stages also carry the group's
 // view (at kPBat: its slot, the group's first tile, copies of its
 // parameters and network).
 constexpr int kPBat = kPRows + 16;
 constexpr int kPBatBytes = 16 + (int)sizeof(ExactParams) + (((int)sizeof(MlpDevice) + 15) & ~15);
-template <bool kFb, bool kList = false, bool kBatch = false>
+template <bool kFb, bool kBatch = false>
 struct PLayout {
-    static_assert(!(kFb && kList), "List Merge with fallbacks runs on the extension kernel");
     static_assert(!(kFb && kBatch), "batches take no fallbacks on learned views");
-    static constexpr int kStages = (kFb || kList) ? 2 : 3;
-    static constexpr int kStage0 = kFb ? kPFbTab + 8 * (int)sizeof(FbTable)
-                                       : (kList ? kPFbTab + kPProducerWarps * (int)sizeof(ListTable) : kPFbTab);
+    static constexpr int kStages = kFb ? 2 : 3;
+    static constexpr int kStage0 = kFb ? kPFbTab + 8 * (int)sizeof(FbTable) : kPFbTab;
     static constexpr int kStageBytes = kFb ? kPUL + 2048 : kPRows + 16 + (kBatch ? kPBatBytes : 0);
     static constexpr int kBytes = kStage0 + kStages * kStageBytes;
     static_assert(kStage0 % 16 == 0 && kStageBytes % 16 == 0 && kPFbTab % 16 == 0, "16-byte operand buffers");
@@ -115,9 +111,9 @@ struct PLayout {
 };
 static_assert(65536 / (kPThreads * kPLaunchRegs) <= 4, "at most four CTAs share an SM's TMEM");
 
-template <bool kFb, bool kList, bool kBatch = false>
+template <bool kFb, bool kBatch = false>
 __device__ __forceinline__ unsigned char *p_stage(unsigned char *sm, int s) {
-    return sm + PLayout<kFb, kList, kBatch>::kStage0 + s * PLayout<kFb, kList, kBatch>::kStageBytes;
+    return sm + PLayout<kFb, kBatch>::kStage0 + s * PLayout<kFb, kBatch>::kStageBytes;
 }
 __device__ __forceinline__ uint64_t *p_full(unsigned char *sm, int s) {
     return reinterpret_cast<uint64_t *>(sm + kPHand) + s;
@@ -327,7 +323,7 @@ __device__ __forceinline__ bool p_chain(unsigned char *sm, uint32_t tmem, uint64
 template <int ALG, int TW, int MD, bool kStats, bool kFb, bool kTwo = false>
 __device__ __forceinline__ void p_step1(const ExactParams &p, const TilePos &tp, long long first, int g,
                                         unsigned char *st, int2 *list, int lane, uint32_t lt, int *ranks,
-                                        Counters &cnt, FbTable *fbt, ListTable *T) {
+                                        Counters &cnt, FbTable *fbt) {
     constexpr int TH = 32 / TW;
     const int tx = lane % TW, ty = lane / TW;
     float2 *pix_st = reinterpret_cast<float2 *>(st + kPST);
@@ -353,7 +349,7 @@ __device__ __forceinline__ void p_step1(const ExactParams &p, const TilePos &tp,
     setup_coords(uv, (float)p.Wt, (float)p.Ht, ps);
     Selection sel;
     if (valid) {
-        sel = select_tile<ALG, MD, kStats, false, kTwo>(p, ps, jac, px, py, lane, lt, T, ranks, cnt);
+        sel = select_tile<ALG, MD, kStats, false, kTwo>(p, ps, jac, px, py, lane, lt, ranks, cnt);
     } else {
         sel.path = PATH_EMPTY;
         sel.A = 0;
@@ -483,8 +479,7 @@ template <int ALG, int TW, int MD, bool kStats, bool kFb, bool kTwo>
 __global__ void __launch_bounds__(kPThreads, kPCtasPerSm)
     mlp_filter_pf_kernel(const ExactParams p, const MlpDevice m, const __grid_constant__ MlpEpilogue ep, int *err) {
     static_assert(!(kFb && kTwo), "fallbacks with two texels per lane run on the extension kernel");
-    constexpr bool kList = ALG == ALG_LIST;
-    constexpr int kPStages = PLayout<kFb, kList>::kStages;
+    constexpr int kPStages = PLayout<kFb>::kStages;
     // tiles per group: two texels per lane may need 64 rows a tile
     constexpr int kGT = kTwo ? kGroupTiles / 2 : kGroupTiles;
     constexpr int kSlots = kGT / kPProducerWarps;
@@ -494,12 +489,6 @@ __global__ void __launch_bounds__(kPThreads, kPCtasPerSm)
     // fallback variant: warp w's texel table (empty between tiles)
     FbTable *fbt = kFb ? reinterpret_cast<FbTable *>(sm + kPFbTab) + warp : nullptr;
     if (kFb) fb_clear(fbt, lane);
-    // List Merge: producer warp w - 4's table (empty between tiles)
-    ListTable *T = kList && warp >= 4 ? reinterpret_cast<ListTable *>(sm + kPFbTab) + (warp - 4) : nullptr;
-    if (kList && warp >= 4) {
-#pragma unroll
-        for (int q = 0; q < 8; ++q) T->keys[lane * 8 + q] = kEmpty;
-    }
     uint64_t *mma_bar = reinterpret_cast<uint64_t *>(sm + kPBar);
     uint32_t *tslot = reinterpret_cast<uint32_t *>(sm + kPTmem);
     if (threadIdx.x < kNumStats) block_stats[threadIdx.x] = 0;
@@ -545,7 +534,7 @@ __global__ void __launch_bounds__(kPThreads, kPCtasPerSm)
             if (grp >= n_groups) break;
             const int s = (int)(j % kPStages);
             const uint32_t par = (uint32_t)((j / kPStages) & 1);
-            unsigned char *st = p_stage<kFb, kList>(sm, s);
+            unsigned char *st = p_stage<kFb>(sm, s);
             bool ok = tc::mbar_wait(p_full(sm, s), par, kMaxTries);
             __syncwarp();
             if (bar_or<1, kRows>(!ok)) {
@@ -594,7 +583,7 @@ __global__ void __launch_bounds__(kPThreads, kPCtasPerSm)
             if (!have) break;
             {
                 const int s = (int)(j % kPStages);
-                unsigned char *st = p_stage<kFb, kList>(sm, s);
+                unsigned char *st = p_stage<kFb>(sm, s);
                 if (j >= kPStages) {
                     // the consumer has gathered group j - kPStages from this stage
                     const bool okd = tc::mbar_wait(p_done(sm, s), (uint32_t)(((j - kPStages) / kPStages) & 1), kMaxTries);
@@ -615,7 +604,7 @@ __global__ void __launch_bounds__(kPThreads, kPCtasPerSm)
 #pragma unroll 1
                 for (int k = 0; k < kSlots; ++k)
                     p_step1<ALG, TW, MD, kStats, kFb, kTwo>(p, tp, first, kSlots * pw + k, st, list, lane, lt, ranks,
-                                                            cnt, fbt, T);
+                                                            cnt, fbt);
                 __syncwarp();
                 prod_bar();  // every slot's list and count is in place
                 // rows: slot g owns [start_g, start_g + count_g) in slot order;
@@ -710,16 +699,10 @@ struct PfBatch {
 template <int ALG, int TW, int MD, bool kStats>
 __global__ void __launch_bounds__(kPThreads, kPCtasPerSm)
     mlp_batch_pf_kernel(const PfBatch b, const MlpDevice m0, const __grid_constant__ MlpEpilogue ep0) {
-    constexpr bool kList = ALG == ALG_LIST;
-    constexpr int kPStages = PLayout<false, kList, true>::kStages;
+    constexpr int kPStages = PLayout<false, true>::kStages;
     extern __shared__ __align__(1024) unsigned char sm[];
     __shared__ unsigned long long block_stats[kNumStats];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    ListTable *T = kList && warp >= 4 ? reinterpret_cast<ListTable *>(sm + kPFbTab) + (warp - 4) : nullptr;
-    if (kList && warp >= 4) {
-#pragma unroll
-        for (int q = 0; q < 8; ++q) T->keys[lane * 8 + q] = kEmpty;
-    }
     uint64_t *mma_bar = reinterpret_cast<uint64_t *>(sm + kPBar);
     uint32_t *tslot = reinterpret_cast<uint32_t *>(sm + kPTmem);
     if (threadIdx.x < kNumStats) block_stats[threadIdx.x] = 0;
@@ -761,7 +744,7 @@ __global__ void __launch_bounds__(kPThreads, kPCtasPerSm)
         for (long long j = 0;; ++j) {
             const int s = (int)(j % kPStages);
             const uint32_t par = (uint32_t)((j / kPStages) & 1);
-            unsigned char *st = p_stage<false, kList, true>(sm, s);
+            unsigned char *st = p_stage<false, true>(sm, s);
             bool ok = tc::mbar_wait(p_full(sm, s), par, kMaxTries);
             __syncwarp();
             if (bar_or<1, kRows>(!ok)) {
@@ -818,7 +801,7 @@ __global__ void __launch_bounds__(kPThreads, kPCtasPerSm)
         const int pt = threadIdx.x - kRows;  // producer thread
         for (long long j = 0;; ++j) {
             const int s = (int)(j % kPStages);
-            unsigned char *st = p_stage<false, kList, true>(sm, s);
+            unsigned char *st = p_stage<false, true>(sm, s);
             if (j >= kPStages) {
                 // the consumer has gathered group j - kPStages from this stage
                 const bool okd = tc::mbar_wait(p_done(sm, s), (uint32_t)(((j - kPStages) / kPStages) & 1), kMaxTries);
@@ -869,7 +852,7 @@ __global__ void __launch_bounds__(kPThreads, kPCtasPerSm)
 #pragma unroll 1
             for (int k = 0; k < kPSlots; ++k)
                 p_step1<ALG, TW, MD, kStats, false>(p, tp, first, kPSlots * pw + k, st, list, lane, lt, ranks, cnt,
-                                                    nullptr, T);
+                                                    nullptr);
             __syncwarp();
             prod_bar();  // every slot's list and count is in place
             const int *count = reinterpret_cast<const int *>(st + kPCount);
@@ -982,10 +965,7 @@ cudaError_t pf_prepare(PfFn fn, int smem_bytes) {
     return e;
 }
 
-int pf_smem(int var, int alg) {
-    return var == kFallback ? PLayout<true>::kBytes
-                            : (alg == ALG_LIST ? PLayout<false, true>::kBytes : PLayout<false>::kBytes);
-}
+int pf_smem(int var) { return var == kFallback ? PLayout<true>::kBytes : PLayout<false>::kBytes; }
 
 }  // namespace
 
@@ -1002,7 +982,7 @@ cudaError_t prepare_mlp_filter_pf(int alg, int tile_w, int mask_dim) {
         for (int st = 0; st < 2; ++st) {
             PfFn fn = pf_kernel(alg, tile_w, mask_dim, st != 0, var);
             if (!fn) continue;  // no such variant for this algorithm
-            const cudaError_t e = pf_prepare(fn, pf_smem(var, alg));
+            const cudaError_t e = pf_prepare(fn, pf_smem(var));
             if (e != cudaSuccess) return e;
         }
     }
@@ -1018,13 +998,13 @@ cudaError_t launch_mlp_filter_pf(const ExactParams &p, const MlpDevice &m, const
     if (!fn) return cudaErrorInvalidValue;
     if (p.n_tiles == 0) return cudaSuccess;
     if (p.n_tiles > 0x7fffffffLL) return cudaErrorInvalidValue;  // tile positions use 32-bit arithmetic
-    cudaError_t e = pf_prepare(fn, pf_smem(var, alg));
+    cudaError_t e = pf_prepare(fn, pf_smem(var));
     if (e != cudaSuccess) return e;
     const int gt = var == kTwoTexels ? kGroupTiles / 2 : kGroupTiles;
     const long long groups = (p.n_tiles + gt - 1) / gt;
     const long long cap = (long long)device_sm_count() * kPCtasPerSm;
     const int grid = (int)(groups < cap ? groups : cap);
-    fn<<<grid, kPThreads, pf_smem(var, alg), stream>>>(p, m, ep, err);
+    fn<<<grid, kPThreads, pf_smem(var), stream>>>(p, m, ep, err);
     return cudaGetLastError();
 }
 
@@ -1051,9 +1031,7 @@ BatchPfFn batch_pf_kernel(int alg, int tile_w, int md, bool st) {
     }
 }
 
-int batch_pf_smem(int alg) {
-    return alg == ALG_LIST ? PLayout<false, true, true>::kBytes : PLayout<false, false, true>::kBytes;
-}
+constexpr int kBatchPfSmem = PLayout<false, true>::kBytes;
 }  // namespace
 
 bool mlp_batch_pf_applies(int alg, int group_dedup) {
@@ -1064,7 +1042,7 @@ cudaError_t prepare_mlp_batch_pf(int alg, int tile_w, int mask_dim) {
     for (int st = 0; st < 2; ++st) {
         BatchPfFn fn = batch_pf_kernel(alg, tile_w, mask_dim, st != 0);
         if (!fn) return cudaErrorInvalidValue;
-        const cudaError_t e = pf_prepare(reinterpret_cast<PfFn>(fn), batch_pf_smem(alg));
+        const cudaError_t e = pf_prepare(reinterpret_cast<PfFn>(fn), kBatchPfSmem);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
@@ -1077,7 +1055,7 @@ cudaError_t launch_mlp_batch_pf(const BatchViewDev *views, int nviews, const int
     BatchPfFn fn = batch_pf_kernel(alg, tile_w, mask_dim, stats != nullptr);
     if (!fn) return cudaErrorInvalidValue;
     if (total_items <= 0) return cudaSuccess;
-    cudaError_t e = pf_prepare(reinterpret_cast<PfFn>(fn), batch_pf_smem(alg));
+    cudaError_t e = pf_prepare(reinterpret_cast<PfFn>(fn), kBatchPfSmem);
     if (e != cudaSuccess) return e;
     PfBatch b;
     b.views = views;
@@ -1091,7 +1069,7 @@ cudaError_t launch_mlp_batch_pf(const BatchViewDev *views, int nviews, const int
     b.err = err;
     const long long cap = (long long)device_sm_count() * kPCtasPerSm;
     const int grid = (int)(total_items < cap ? total_items : cap);
-    fn<<<grid, kPThreads, batch_pf_smem(alg), s>>>(b, m0, ep0);
+    fn<<<grid, kPThreads, kBatchPfSmem, s>>>(b, m0, ep0);
     return cudaGetLastError();
 }
 
