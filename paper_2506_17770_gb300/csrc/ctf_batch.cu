@@ -411,7 +411,9 @@ int make_plan(const ctf_view *views, int nviews, ctf_algorithm alg, uint64_t see
             continue;
         }
         const int kind = d.learned ? 1 : 0;
-        const long long per_item = d.learned ? mlp_group_tiles((int)alg) : kBlockItemTiles;
+        const long long per_item = !d.learned ? kBlockItemTiles
+                                   : mlp_batch_pf_applies((int)alg, r.group_dedup) ? mlp_batch_pf_tiles()
+                                                                                   : mlp_group_tiles((int)alg);
         plan->index[kind].push_back(i);
         plan->begin[kind].push_back(plan->items[kind]);
         plan->items[kind] += (p.n_tiles + per_item - 1) / per_item;

@@ -186,6 +186,7 @@ static_assert(sizeof(ExactParams) % 16 == 0 && sizeof(ExactParams) <= 32 * 16, "
 // item_begin[k]; the CTAs take items from *counter (zero at launch).  m0 and
 // ep0 are the first view's network, which the CTAs load first.
 bool mlp_batch_pf_applies(int alg, int group_dedup);
+int mlp_batch_pf_tiles();  // tiles of an item
 cudaError_t prepare_mlp_batch_pf(int alg, int tile_w, int mask_dim);
 cudaError_t launch_mlp_batch_pf(const BatchViewDev *views, int nviews, const int *index, const long long *item_begin,
                                 int nkind, long long total_items, unsigned long long *counter, unsigned long long *stats,

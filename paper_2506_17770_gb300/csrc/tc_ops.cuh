@@ -43,6 +43,19 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, uint32
     return false;
 }
 
+// One thread of a converged warp (the same one every time): the form in which
+// tcgen05.mma and tcgen05.commit are issued, inside a warp-uniform branch, so
+// that the compiler knows that a single thread of a whole warp gets there.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t leader;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "elect.sync _|p, 0xffffffff;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(leader)::"memory");
+    return leader != 0;
+}
+
 // ---------------------------------------------------------------------------
 // Tensor memory
 // ---------------------------------------------------------------------------
