@@ -116,9 +116,14 @@ int device_sm_count();
 // recorded error if that failed).
 const DecodeTables *device_decode_tables();
 
-// Learned decode (ctf_mlp.cu).
-cudaError_t launch_mlp_decode(const MlpDevice &m, int Wt, int Ht, const int2 *xy, int n, float4 *out, int *err,
-                              cudaStream_t stream);
+// Decode of a list of texels, and the learned per-pixel 4-tap filter
+// (ctf_mlp_dense.cu).
+cudaError_t launch_mlp_decode(const MlpDevice &m, const MlpEpilogue &ep, int Wt, int Ht, const int2 *xy, int n,
+                              float4 *out, int *err, cudaStream_t stream);
+cudaError_t prepare_mlp_4tap(int tile_w);
+cudaError_t launch_mlp_4tap(const ExactParams &p, const MlpDevice &m, const MlpEpilogue &ep, int tile_w, int *err,
+                            cudaStream_t stream);
+// Learned filter (ctf_mlp.cu).
 // Sets the learned filter kernel's attributes without launching it (needed
 // before a stream capture records a launch of it).
 cudaError_t prepare_mlp_filter(int alg, int tile_w, int mask_dim);

@@ -17,15 +17,15 @@
 // tracked with an mbarrier whose waits are bounded: a wait that gives up sets
 // the library's error word and every thread of the CTA leaves together.
 //
-// Two kernels here use the chain: a decode of an explicit list of texels, and
-// the learned-decode filter for per-pixel 4-tap and List Merge.  Per-pixel
-// 4-tap gives each warp one pixel tile (its lane's row per tap, four chains
-// per iteration); List Merge gives each warp two tiles of a group of 8, packs
-// the group's texel lists into consecutive rows (one or two chains) and
-// gathers every pixel's taps from the rows (ctf_mlp_chain.cuh, mlp_group;
-// the persistent batch kernel runs the same for every algorithm).  STF, Box
-// and Mask Sampling on single views run in the kernel whose warps are
-// specialised by role (ctf_mlp_ws.cu), which gives the same outputs.
+// The kernel here runs List Merge with group_dedup: each warp takes two tiles
+// of a group of 8, the group's distinct texels are packed into consecutive
+// rows (one or two chains), and every pixel gathers its taps from the rows
+// (ctf_mlp_chain.cuh, mlp_group; the persistent batch kernel runs the same
+// for every algorithm with group_dedup).  Everything else runs in kernels
+// whose warps are specialised by role, which give the same outputs:
+// ctf_mlp_ws2.cuh (STF, List Merge, Box and Mask Sampling), ctf_mlp_ws.cu (STF,
+// Box and Mask with group_dedup), ctf_mlp_ext.cu (combined extensions) and
+// ctf_mlp_dense.cu (per-pixel 4-tap, decode of a list).
 #include <cstdint>
 #include <mutex>
 #include <set>
@@ -45,36 +45,8 @@ namespace ctf {
 namespace {
 
 // ---------------------------------------------------------------------------
-// Decode an explicit list of texels.
-// ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(kRows) mlp_decode_kernel(const MlpDevice m, int Wt, int Ht, const int2 *xy, int n,
-                                                           float4 *out, int *err) {
-    extern __shared__ __align__(1024) unsigned char sm[];
-    Chain ch;
-    chain_setup(ch, sm, m);
-    const float *inv_a1 = reinterpret_cast<const float *>(sm + kImgA1);
-    const int ntiles = (n + kRows - 1) / kRows;
-    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-        const int row = tile * kRows + threadIdx.x;
-        if (row < n) {
-            const int2 c = xy[row];
-            const int x = min(max(c.x, 0), Wt - 1), y = min(max(c.y, 0), Ht - 1);
-            float f[kMlpIn];
-            texel_features(m, x, y, f);
-            store_x_row(sm, threadIdx.x, f, m.fp8, inv_a1);
-        } else {
-            store_zero_x_row(sm, threadIdx.x);
-        }
-        float4 v;
-        if (!mlp_chain(ch, m.fp8, v, err)) break;
-        if (row < n) out[row] = v;
-    }
-    chain_teardown(ch);
-}
-
-// ---------------------------------------------------------------------------
-// Learned-decode filter for per-pixel 4-tap and List Merge: 4 warps; a group
-// of 8 pixel tiles (4 for per-pixel 4-tap) per CTA iteration.
+// Learned-decode filter for List Merge with group_dedup: 4 warps; a group of
+// 8 pixel tiles per CTA iteration.
 // ---------------------------------------------------------------------------
 template <int ALG, int TW, int MD>
 __global__ void __launch_bounds__(kRows, 4) mlp_filter_kernel(const ExactParams p, const MlpDevice m, int *err) {
@@ -83,7 +55,7 @@ __global__ void __launch_bounds__(kRows, 4) mlp_filter_kernel(const ExactParams 
     Chain ch;
     chain_setup(ch, sm, m);
     const float *inv_a1 = reinterpret_cast<const float *>(sm + kImgA1);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31;
     if (threadIdx.x < kNumStats) block_stats[threadIdx.x] = 0;
     __syncthreads();
     const uint32_t lt = lanemask_lt();
@@ -94,8 +66,7 @@ __global__ void __launch_bounds__(kRows, 4) mlp_filter_kernel(const ExactParams 
     const long long n_iter = (p.n_tiles + kTiles - 1) / kTiles;
     bool ok = true;
     for (long long it = blockIdx.x; it < n_iter && ok; it += gridDim.x) {
-        if (ALG == ALG_4TAP) ok = mlp_warp_tile<ALG, TW, MD>(p, m, ch, it * kTiles + warp, lane, lt, cnt, inv_a1, err);
-        else ok = mlp_group<ALG, TW, MD>(p, m, ch, it * kTiles, lane, lt, cnt, inv_a1, err);
+        ok = mlp_group<ALG, TW, MD>(p, m, ch, it * kTiles, lane, lt, cnt, inv_a1, err);
     }
     if (p.stats) {
         if (lane == 0) {
@@ -125,21 +96,11 @@ __global__ void bounded_wait_selftest_kernel(uint32_t polls, int *err) {
 
 using FilterFn = void (*)(const ExactParams, const MlpDevice, int *);
 
-template <int ALG, int TW>
-FilterFn pick_mask(int md) {
-    if constexpr (ALG == ALG_MASK) {
-        return md == 11 ? mlp_filter_kernel<ALG, TW, 11> : mlp_filter_kernel<ALG, TW, 16>;
-    } else {
-        return mlp_filter_kernel<ALG, TW, 16>;
-    }
-}
-
-// (STF, Box and Mask Sampling run in mlp_filter_ws_kernel.)
-template <int TW>
-FilterFn pick_alg(int alg, int md) {
-    switch (alg) {
-    case ALG_4TAP: return pick_mask<ALG_4TAP, TW>(md);
-    case ALG_LIST: return pick_mask<ALG_LIST, TW>(md);
+FilterFn pick_list(int tile_w) {
+    switch (tile_w) {
+    case 8: return mlp_filter_kernel<ALG_LIST, 8, 16>;
+    case 4: return mlp_filter_kernel<ALG_LIST, 4, 16>;
+    case 16: return mlp_filter_kernel<ALG_LIST, 16, 16>;
     default: return nullptr;
     }
 }
@@ -161,18 +122,8 @@ cudaError_t prepare(F fn) {
 
 }  // namespace
 
-cudaError_t launch_mlp_decode(const MlpDevice &m, int Wt, int Ht, const int2 *xy, int n, float4 *out, int *err,
-                              cudaStream_t stream) {
-    if (n <= 0) return cudaSuccess;
-    cudaError_t e = prepare(mlp_decode_kernel);
-    if (e != cudaSuccess) return e;
-    const int ntiles = (n + kRows - 1) / kRows;
-    const int cap = device_sm_count() * 4;
-    mlp_decode_kernel<<<ntiles < cap ? ntiles : cap, kRows, kSmRequest, stream>>>(m, Wt, Ht, xy, n, out, err);
-    return cudaGetLastError();
-}
-
 cudaError_t prepare_mlp_filter(int alg, int tile_w, int mask_dim) {
+    if (alg == ALG_4TAP) return prepare_mlp_4tap(tile_w);
     if (alg == ALG_LIST) {
         cudaError_t e = prepare_mlp_filter_pf(alg, tile_w, mask_dim);
         if (e != cudaSuccess) return e;
@@ -181,13 +132,7 @@ cudaError_t prepare_mlp_filter(int alg, int tile_w, int mask_dim) {
         cudaError_t e = prepare_mlp_filter_pf(alg, tile_w, mask_dim);
         return e == cudaSuccess ? prepare_mlp_filter_ws(alg, tile_w, mask_dim) : e;
     }
-    FilterFn fn = nullptr;
-    switch (tile_w) {
-    case 8: fn = pick_alg<8>(alg, mask_dim); break;
-    case 4: fn = pick_alg<4>(alg, mask_dim); break;
-    case 16: fn = pick_alg<16>(alg, mask_dim); break;
-    default: return cudaErrorInvalidValue;
-    }
+    FilterFn fn = alg == ALG_LIST ? pick_list(tile_w) : nullptr;
     return fn ? prepare(fn) : cudaErrorInvalidValue;
 }
 
@@ -198,6 +143,7 @@ cudaError_t launch_bounded_wait_selftest(uint32_t polls, int *err, cudaStream_t 
 
 cudaError_t launch_mlp_filter(const ExactParams &p, const MlpDevice &m, const MlpEpilogue &ep, int alg, int tile_w,
                               int mask_dim, int *err, cudaStream_t stream) {
+    if (alg == ALG_4TAP) return launch_mlp_4tap(p, m, ep, tile_w, err, stream);
     // fallbacks C / C+ with one texel per lane on Box and Mask: the packed-group kernel's fallback variant
     if (mlp_filter_pf_fallback_applies(p, alg) || mlp_filter_pf_two_applies(p, alg))
         return launch_mlp_filter_pf(p, m, ep, alg, tile_w, mask_dim, err, stream);
@@ -208,13 +154,7 @@ cudaError_t launch_mlp_filter(const ExactParams &p, const MlpDevice &m, const Ml
     if (mlp_filter_ws_applies(p, alg))
         return p.group_dedup ? launch_mlp_filter_ws(p, m, alg, tile_w, mask_dim, err, stream)
                              : launch_mlp_filter_pf(p, m, ep, alg, tile_w, mask_dim, err, stream);
-    FilterFn fn = nullptr;
-    switch (tile_w) {
-    case 8: fn = pick_alg<8>(alg, mask_dim); break;
-    case 4: fn = pick_alg<4>(alg, mask_dim); break;
-    case 16: fn = pick_alg<16>(alg, mask_dim); break;
-    default: return cudaErrorInvalidValue;
-    }
+    FilterFn fn = alg == ALG_LIST ? pick_list(tile_w) : nullptr;
     if (!fn) return cudaErrorInvalidValue;
     if (p.n_tiles == 0) return cudaSuccess;
     if (p.n_tiles > 0x7fffffffLL) return cudaErrorInvalidValue;  // tile positions use 32-bit arithmetic

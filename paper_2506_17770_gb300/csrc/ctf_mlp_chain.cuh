@@ -88,6 +88,30 @@ __device__ __forceinline__ void tile_pos(const TilePos &t, int g, int &bx, int &
     by = (int)y;
 }
 
+// Bilinear blend of the 8 channels of four latent cells at (fx, fy).
+__device__ __forceinline__ void blend_latents(const uint4 &q00, const uint4 &q10, const uint4 &q01, const uint4 &q11,
+                                              float fx, float fy, float f[8]) {
+    const float ofx = __fsub_rn(1.f, fx), ofy = __fsub_rn(1.f, fy);
+    const float w00 = __fmul_rn(ofx, ofy), w10 = __fmul_rn(fx, ofy), w01 = __fmul_rn(ofx, fy), w11 = __fmul_rn(fx, fy);
+    const __half2 *h00 = reinterpret_cast<const __half2 *>(&q00);
+    const __half2 *h10 = reinterpret_cast<const __half2 *>(&q10);
+    const __half2 *h01 = reinterpret_cast<const __half2 *>(&q01);
+    const __half2 *h11 = reinterpret_cast<const __half2 *>(&q11);
+    // channels 2c and 2c+1 together: packed multiply and FMAs round each
+    // component like their scalar forms
+    const float2 v00 = make_float2(w00, w00), v10 = make_float2(w10, w10), v01 = make_float2(w01, w01),
+                 v11 = make_float2(w11, w11);
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        float2 acc = __fmul2_rn(v00, __half22float2(h00[c]));
+        acc = __ffma2_rn(v10, __half22float2(h10[c]), acc);
+        acc = __ffma2_rn(v01, __half22float2(h01[c]), acc);
+        acc = __ffma2_rn(v11, __half22float2(h11[c]), acc);
+        f[2 * c] = acc.x;
+        f[2 * c + 1] = acc.y;
+    }
+}
+
 // Features of texel (x, y) (inside the texture) in FP32.
 __device__ __forceinline__ void texel_features(const MlpDevice &m, int x, int y, float f[kMlpIn]) {
 #pragma unroll
@@ -105,26 +129,7 @@ __device__ __forceinline__ void texel_features(const MlpDevice &m, int x, int y,
         const uint4 q10 = __ldg(L + ck((size_t)ya * m.gw[g] + xb, cells, m.err, kBndLatent));
         const uint4 q01 = __ldg(L + ck((size_t)yb * m.gw[g] + xa, cells, m.err, kBndLatent));
         const uint4 q11 = __ldg(L + ck((size_t)yb * m.gw[g] + xb, cells, m.err, kBndLatent));
-        const float ofx = __fsub_rn(1.f, fx), ofy = __fsub_rn(1.f, fy);
-        const float w00 = __fmul_rn(ofx, ofy), w10 = __fmul_rn(fx, ofy), w01 = __fmul_rn(ofx, fy),
-                    w11 = __fmul_rn(fx, fy);
-        const __half2 *h00 = reinterpret_cast<const __half2 *>(&q00);
-        const __half2 *h10 = reinterpret_cast<const __half2 *>(&q10);
-        const __half2 *h01 = reinterpret_cast<const __half2 *>(&q01);
-        const __half2 *h11 = reinterpret_cast<const __half2 *>(&q11);
-        // channels 2c and 2c+1 together: packed multiply and FMAs round each
-        // component like their scalar forms
-        const float2 v00 = make_float2(w00, w00), v10 = make_float2(w10, w10), v01 = make_float2(w01, w01),
-                     v11 = make_float2(w11, w11);
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            float2 acc = __fmul2_rn(v00, __half22float2(h00[c]));
-            acc = __ffma2_rn(v10, __half22float2(h10[c]), acc);
-            acc = __ffma2_rn(v01, __half22float2(h01[c]), acc);
-            acc = __ffma2_rn(v11, __half22float2(h11[c]), acc);
-            f[g * 8 + 2 * c] = acc.x;
-            f[g * 8 + 2 * c + 1] = acc.y;
-        }
+        blend_latents(q00, q10, q01, q11, fx, fy, f + 8 * g);
     }
 }
 

@@ -245,7 +245,7 @@ int ctf_mlp_decode(ctf_texture t, const int32_t *xy, int n, float *out_rgba, voi
     int *err = nullptr;
     int rc = device_error_word(&err);
     if (rc) return rc;
-    cudaError_t e = launch_mlp_decode(mlp_device_view(t), t->width, t->height, reinterpret_cast<const int2 *>(xy), n,
+    cudaError_t e = launch_mlp_decode(mlp_device_view(t), t->epi, t->width, t->height, reinterpret_cast<const int2 *>(xy), n,
                                       reinterpret_cast<float4 *>(out_rgba), err, static_cast<cudaStream_t>(stream));
     if (e != cudaSuccess) return report_cuda(e, "decode launch");
     return CTF_OK;

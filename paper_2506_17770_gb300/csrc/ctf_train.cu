@@ -1276,7 +1276,7 @@ int ctf_texture_compare(ctf_texture ref, ctf_texture learned, double *mse_rgb, d
         const int n = (int)std::min<long long>(chunk, total - st);
         linear_xy_kernel<<<1024, 256, 0, s>>>(xy, st, n, ref->width);
         e = cudaGetLastError();
-        if (e == cudaSuccess) e = launch_mlp_decode(m, learned->width, learned->height, xy, n, dec, err, s);
+        if (e == cudaSuccess) e = launch_mlp_decode(m, learned->epi, learned->width, learned->height, xy, n, dec, err, s);
         if (e == cudaSuccess) {
             compare_kernel<<<1024, 256, 0, s>>>(static_cast<const uint2 *>(ref->blocks), ref->width / 4, ref->width,
                                                 ref->height, dec, st, n, sse, mx);
