@@ -364,18 +364,25 @@ constexpr bool p_tap_pairs() { return ALG == ALG_BOX || ALG == ALG_MASK; }
 // texels): the pixel's word holds the 6-bit list indices of its taps (bits
 // 0-23, or of its own texel), its count (24-25), active (26), inside (27)
 // and success (28).
+// The inputs of the lane's pixel of the tile at (bx, by).  Every lane loads
+// (lanes outside the frame pixel 0, which exists), so that the loads carry no
+// predicates.
+template <int ALG, int TW>
+__device__ __forceinline__ Inputs p_load(const ExactParams &p, const LanePlace<TW> &lp, uint32_t bx, uint32_t by) {
+    constexpr uint32_t TH = 32 / TW;
+    return load_inputs_any<(ALG >= ALG_LIST)>(p, bx < lp.lim_x && by < lp.lim_y,
+                                              by * (TH * (uint32_t)p.W) + bx * TW + lp.off);
+}
+
 template <int ALG, int TW, int MD, bool kStats, bool kFb, bool kTwo = false>
-__device__ __forceinline__ void p_step1(const ExactParams &p, const LanePlace<TW> &lp, uint32_t bx, uint32_t by, int g,
-                                        unsigned char *st, int2 *list, int lane, uint32_t lt, int *ranks,
+__device__ __forceinline__ void p_step1(const ExactParams &p, const LanePlace<TW> &lp, uint32_t bx, uint32_t by,
+                                        const Inputs &in, int g, unsigned char *st, int2 *list, int lane, uint32_t lt, int *ranks,
                                         Counters &cnt, FbTable *fbt) {
     using S = typename PLayout<kFb>::S;
     constexpr uint32_t TH = 32 / TW;
     const bool inside = bx < lp.lim_x && by < lp.lim_y;
     const int px = (int)(bx * TW + lp.tx), py = (int)(by * TH + lp.ty);
     const uint32_t pixel = by * (TH * (uint32_t)p.W) + bx * TW;
-    // every lane loads (lanes outside pixel 0, which exists), so that the
-    // loads carry no predicates
-    const Inputs in = load_inputs_any<(ALG >= ALG_LIST)>(p, inside, pixel + lp.off);
     PixelSetup ps;
     ps.active = in.covered;
     setup_coords(in.uv, (float)p.Wt, (float)p.Ht, ps);
@@ -603,11 +610,13 @@ __global__ void __launch_bounds__(kPThreads, kPCtasPerSm)
         int2 *list = reinterpret_cast<int2 *>(sm + kPList);
         const int pt = threadIdx.x - kRows;  // producer thread
         const LanePlace<TW> lp(p, lane);
-        // the first tile of the CTA's group, advanced by the grid's stride
-        // without dividing again
+        // the warp's tiles, advanced by the grid's stride without dividing again
         const uint32_t tiles_x = (uint32_t)p.tiles_x;
-        uint32_t gx = (uint32_t)blockIdx.x * kGT % tiles_x, gy = (uint32_t)blockIdx.x * kGT / tiles_x;
+        const uint32_t mine = (uint32_t)blockIdx.x * kGT + (uint32_t)(kSlots * pw);
+        uint32_t gx = mine % tiles_x, gy = mine / tiles_x;  // the warp's first tile of the group
         const uint32_t step = (uint32_t)G * kGT, step_x = step % tiles_x, step_y = step / tiles_x;
+        uint32_t bx = gx, by = gy;
+        Inputs in = p_load<ALG, TW>(p, lp, bx, by);
         for (long long j = 0;; ++j) {
             const long long grp = blockIdx.x + j * G;
             const bool have = grp < n_groups;  // uniform over the CTA
@@ -630,19 +639,29 @@ __global__ void __launch_bounds__(kPThreads, kPCtasPerSm)
                     __syncwarp();
                     prod_bar();
                 }
-                uint32_t bx = gx, by = gy;  // the warp's first tile of the group
-                p_tile(tiles_x, bx, by, (uint32_t)(kSlots * pw));
 #pragma unroll 1
                 for (int k = 0; k < kSlots; ++k) {
-                    p_step1<ALG, TW, MD, kStats, kFb, kTwo>(p, lp, bx, by, kSlots * pw + k, st, list, lane, lt, ranks,
-                                                            cnt, fbt);
-                    p_tile(tiles_x, bx, by, 1u);
-                }
-                gx += step_x;  // the CTA's next group
-                gy += step_y;
-                if (gx >= tiles_x) {
-                    gx -= tiles_x;
-                    ++gy;
+                    // the inputs of the warp's next tile come in while this one
+                    // is in step 1 (or the group's features are computed)
+                    uint32_t nx = bx, ny = by;
+                    if (k + 1 < kSlots) {
+                        p_tile(tiles_x, nx, ny, 1u);
+                    } else {  // first slot of the CTA's next group
+                        gx += step_x;
+                        gy += step_y;
+                        if (gx >= tiles_x) {
+                            gx -= tiles_x;
+                            ++gy;
+                        }
+                        nx = gx;
+                        ny = gy;
+                    }
+                    const Inputs next = p_load<ALG, TW>(p, lp, nx, ny);
+                    p_step1<ALG, TW, MD, kStats, kFb, kTwo>(p, lp, bx, by, in, kSlots * pw + k, st, list, lane, lt,
+                                                            ranks, cnt, fbt);
+                    bx = nx;
+                    by = ny;
+                    in = next;
                 }
                 // the next group's stage starts with no rows given out (the last
                 // group that used it has its row count in kRowsOff)
@@ -871,8 +890,9 @@ __global__ void __launch_bounds__(kPThreads, kPCtasPerSm)
             uint32_t bx = mine % tiles_x, by = mine / tiles_x;
 #pragma unroll 1
             for (int k = 0; k < kPSlots; ++k) {
-                p_step1<ALG, TW, MD, kStats, false>(p, lp, bx, by, kPSlots * pw + k, st, list, lane, lt, ranks, cnt,
-                                                    nullptr);
+                const Inputs in = p_load<ALG, TW>(p, lp, bx, by);
+                p_step1<ALG, TW, MD, kStats, false>(p, lp, bx, by, in, kPSlots * pw + k, st, list, lane, lt, ranks,
+                                                    cnt, nullptr);
                 p_tile(tiles_x, bx, by, 1u);
             }
             // (as in the single-view kernel)
