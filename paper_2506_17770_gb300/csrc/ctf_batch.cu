@@ -84,7 +84,10 @@ constexpr int batch_min_blocks() {
     return ALG >= ALG_LIST ? 4 : 1;
 }
 
-template <int ALG, int TW, int MD, bool kFb>
+// kStats: the variant that keeps the outcome counters (its registers spill;
+// 256 views of 64..512^2, half of them blocks: 163 us with, for every call
+// before, see below for without).
+template <int ALG, int TW, int MD, bool kFb, bool kStats>
 __global__ void __launch_bounds__(kBlockWarps * 32, batch_min_blocks<ALG>()) batch_block_kernel(const BatchParams b) {
     constexpr int TH = 32 / TW;
     constexpr bool kJac = ALG >= ALG_LIST;
@@ -150,7 +153,7 @@ __global__ void __launch_bounds__(kBlockWarps * 32, batch_min_blocks<ALG>()) bat
             const bool ninside = i + 1u < n_item && nbx < lim_x && nby < lim_y;
             const uint32_t nidx = nby * (TH * W) + nbx * TW + lane_off;
             const Inputs nxt = load_inputs_any<kJac>(p, ninside, nidx);
-            filter_tile<ALG, TW, MD, true, kFb ? kExtFallback | kExtTwo : 0>(p, cur, (int)(bx * TW) + tx, (int)(by * TH) + ty, inside, idx, lane, lt,
+            filter_tile<ALG, TW, MD, kStats, kFb ? kExtFallback | kExtTwo : 0>(p, cur, (int)(bx * TW) + tx, (int)(by * TH) + ty, inside, idx, lane, lt,
                                            &tabs, rank_slots[warp], &fb_tab[warp], cnt);
             bx = nbx;
             by = nby;
@@ -159,7 +162,7 @@ __global__ void __launch_bounds__(kBlockWarps * 32, batch_min_blocks<ALG>()) bat
             cur = nxt;
         }
     }
-    if (b.stats) {
+    if (kStats && b.stats) {
         if (lane == 0) {
 #pragma unroll
             for (int i = 0; i < kNumStats; ++i)
@@ -254,42 +257,43 @@ using BatchFn = void (*)(const BatchParams);
 // Learned views never take fallbacks C / C+ (the plan refuses them); block
 // views of the collaborative algorithms have a variant that does.
 template <bool kMlp, int ALG, int TW, int MD>
-BatchFn kernel_of(bool fb) {
+BatchFn kernel_of(bool fb, bool stats) {
     if constexpr (kMlp) {
         return batch_mlp_kernel<ALG, TW, MD>;
     } else if constexpr (ALG >= ALG_LIST) {
-        return fb ? batch_block_kernel<ALG, TW, MD, true> : batch_block_kernel<ALG, TW, MD, false>;
+        if (fb) return batch_block_kernel<ALG, TW, MD, true, true>;
+        return stats ? batch_block_kernel<ALG, TW, MD, false, true> : batch_block_kernel<ALG, TW, MD, false, false>;
     } else {
-        return batch_block_kernel<ALG, TW, MD, false>;
+        return stats ? batch_block_kernel<ALG, TW, MD, false, true> : batch_block_kernel<ALG, TW, MD, false, false>;
     }
 }
 
 template <bool kMlp, int ALG, int TW>
-BatchFn pick_mask(int md, bool fb) {
+BatchFn pick_mask(int md, bool fb, bool st) {
     if constexpr (ALG == ALG_MASK) {
-        return md == 11 ? kernel_of<kMlp, ALG, TW, 11>(fb) : kernel_of<kMlp, ALG, TW, 16>(fb);
+        return md == 11 ? kernel_of<kMlp, ALG, TW, 11>(fb, st) : kernel_of<kMlp, ALG, TW, 16>(fb, st);
     } else {
-        return kernel_of<kMlp, ALG, TW, 16>(fb);
+        return kernel_of<kMlp, ALG, TW, 16>(fb, st);
     }
 }
 
 template <bool kMlp, int TW>
-BatchFn pick_alg(int alg, int md, bool fb) {
+BatchFn pick_alg(int alg, int md, bool fb, bool st) {
     switch (alg) {
-    case ALG_4TAP: return pick_mask<kMlp, ALG_4TAP, TW>(md, fb);
-    case ALG_STF: return pick_mask<kMlp, ALG_STF, TW>(md, fb);
-    case ALG_LIST: return pick_mask<kMlp, ALG_LIST, TW>(md, fb);
-    case ALG_BOX: return pick_mask<kMlp, ALG_BOX, TW>(md, fb);
-    case ALG_MASK: return pick_mask<kMlp, ALG_MASK, TW>(md, fb);
+    case ALG_4TAP: return pick_mask<kMlp, ALG_4TAP, TW>(md, fb, st);
+    case ALG_STF: return pick_mask<kMlp, ALG_STF, TW>(md, fb, st);
+    case ALG_LIST: return pick_mask<kMlp, ALG_LIST, TW>(md, fb, st);
+    case ALG_BOX: return pick_mask<kMlp, ALG_BOX, TW>(md, fb, st);
+    case ALG_MASK: return pick_mask<kMlp, ALG_MASK, TW>(md, fb, st);
     default: return nullptr;
     }
 }
 
-BatchFn pick(bool mlp, int alg, int tile_w, int md, bool fb) {
+BatchFn pick(bool mlp, int alg, int tile_w, int md, bool fb, bool st) {
     switch (tile_w) {
-    case 8: return mlp ? pick_alg<true, 8>(alg, md, fb) : pick_alg<false, 8>(alg, md, fb);
-    case 4: return mlp ? pick_alg<true, 4>(alg, md, fb) : pick_alg<false, 4>(alg, md, fb);
-    case 16: return mlp ? pick_alg<true, 16>(alg, md, fb) : pick_alg<false, 16>(alg, md, fb);
+    case 8: return mlp ? pick_alg<true, 8>(alg, md, fb, st) : pick_alg<false, 8>(alg, md, fb, st);
+    case 4: return mlp ? pick_alg<true, 4>(alg, md, fb, st) : pick_alg<false, 4>(alg, md, fb, st);
+    case 16: return mlp ? pick_alg<true, 16>(alg, md, fb, st) : pick_alg<false, 16>(alg, md, fb, st);
     default: return nullptr;
     }
 }
@@ -491,7 +495,7 @@ cudaError_t launch_plan(const Plan &plan, const DevPlan &dp, int alg, const Reso
     if (e != cudaSuccess) return e;
     for (int k = 0; k < 2; ++k) {
         if (plan.items[k] == 0) continue;
-        BatchFn fn = pick(k == 1, alg, r.tile_w, r.mask_dim, r.fallback != 0 || r.tpl == 2);
+        BatchFn fn = pick(k == 1, alg, r.tile_w, r.mask_dim, r.fallback != 0 || r.tpl == 2, stats != nullptr);
         if (!fn) return cudaErrorInvalidValue;
         BatchParams b;
         b.views = dp.views;
@@ -507,8 +511,8 @@ cudaError_t launch_plan(const Plan &plan, const DevPlan &dp, int alg, const Reso
         b.tables = k == 0 ? plan.views[plan.index[0][0]].p.tables : nullptr;
         if (k == 1 && mlp_batch_pf_applies(alg, r.group_dedup)) {
             // learned views on the packed-group kernel (one group per fetch)
-            e = launch_mlp_batch_pf(dp.views, (int)plan.views.size(), dp.index[1], dp.begin[1], b.nkind, b.total_items,
-                                    b.counter, stats, err, plan.views[plan.index[1][0]].m, *plan.epi[plan.index[1][0]], alg, r.tile_w,
+            e = launch_mlp_batch_pf(dp.views, (int)plan.views.size(), dp.index[1], dp.begin[1], b.nkind, b.total_items, stats,
+                                    err, plan.views[plan.index[1][0]].m, *plan.epi[plan.index[1][0]], alg, r.tile_w,
                                     r.mask_dim, s);
             if (e != cudaSuccess) return e;
             continue;
@@ -614,7 +618,7 @@ int ctf_batch_graph_create(const ctf_view *views, int nviews, ctf_algorithm alg,
     if (e == cudaSuccess) e = upload_plan(plan, &g->plan, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     // the kernel attributes must be set before capture
-    if (e == cudaSuccess && plan.items[1]) e = prepare_batch(pick(true, (int)alg, r.tile_w, r.mask_dim, false));
+    if (e == cudaSuccess && plan.items[1]) e = prepare_batch(pick(true, (int)alg, r.tile_w, r.mask_dim, false, false));
     if (e == cudaSuccess && plan.items[1] && mlp_batch_pf_applies((int)alg, r.group_dedup))
         e = prepare_mlp_batch_pf((int)alg, r.tile_w, r.mask_dim);
     for (int i : plan.solo)

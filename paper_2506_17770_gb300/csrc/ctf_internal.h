@@ -188,14 +188,13 @@ static_assert(sizeof(ExactParams) % 16 == 0 && sizeof(ExactParams) <= 32 * 16, "
 // The learned views of a batch (other than per-pixel 4-tap and group_dedup)
 // on the packed-group kernel (ctf_mlp_ws2.cu): the views index[0..nkind)
 // of the table of nviews views, whose items (groups of 8 tiles) are numbered from
-// item_begin[k]; the CTAs take items from *counter (zero at launch).  m0 and
-// ep0 are the first view's network, which the CTAs load first.
+// item_begin[k] (nkind + 1 of them); CTA c takes items c, c + grid, ...  m0
+// and ep0 are the first view's network, which the CTAs load first.
 bool mlp_batch_pf_applies(int alg, int group_dedup);
 int mlp_batch_pf_tiles();  // tiles of an item
 cudaError_t prepare_mlp_batch_pf(int alg, int tile_w, int mask_dim);
 cudaError_t launch_mlp_batch_pf(const BatchViewDev *views, int nviews, const int *index, const long long *item_begin,
-                                int nkind, long long total_items, unsigned long long *counter, unsigned long long *stats,
-                                int *err, const MlpDevice &m0, const MlpEpilogue &ep0, int alg, int tile_w, int mask_dim,
+                                int nkind, long long total_items, unsigned long long *stats, int *err, const MlpDevice &m0, const MlpEpilogue &ep0, int alg, int tile_w, int mask_dim,
                                 cudaStream_t s);
 
 // Error reporting shared by the C ABI translation units (ctf_api.cu).

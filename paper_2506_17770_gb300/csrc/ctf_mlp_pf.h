@@ -16,7 +16,6 @@ struct PfBatch {
     const long long *item_begin;
     int nkind, nviews;
     long long total_items;
-    unsigned long long *counter;
     unsigned long long *stats;
     int *err;
 };

@@ -101,16 +101,16 @@ struct PStage {
 // kFb: the variant with fallbacks C / C+ (two stages, to make room for the
 // texel tables and the per-pixel texels the blend of eq. 1 needs).
 // kBatch: the persistent batch kernel, whose stages also carry the group's
-// view (after the other fields: its slot, the group's first tile, copies of
-// its parameters and network).
-constexpr int kPBatBytes = 16 + (int)sizeof(ExactParams) + (((int)sizeof(MlpDevice) + 15) & ~15);
+// view (copies of its parameters and network) and whose producer warps keep
+// two copies of their own.
+constexpr int kPViewBytes = (int)sizeof(ExactParams) + (((int)sizeof(MlpDevice) + 15) & ~15);
 template <bool kFb, bool kBatch = false>
 struct PLayout {
     static_assert(!(kFb && kBatch), "batches take no fallbacks on learned views");
     using S = PStage<kPTiles>;
     static constexpr int kStages = kFb ? 2 : 3;
-    static constexpr int kStage0 = kFb ? kPListEnd + (4 + kPProducerWarps) * (int)sizeof(FbTable) : kPListEnd;
-    static constexpr int kStageBytes = kFb ? S::kFbEnd : S::kEnd + (kBatch ? kPBatBytes : 0);
+    static constexpr int kStage0 = kPListEnd + (kFb ? (4 + kPProducerWarps) * (int)sizeof(FbTable) : kBatch ? 2 * kPProducerWarps * kPViewBytes : 0);
+    static constexpr int kStageBytes = kFb ? S::kFbEnd : S::kEnd + (kBatch ? kPViewBytes : 0);
     static constexpr int kBytes = kStage0 + kStages * kStageBytes;
     static_assert(kStage0 % 16 == 0 && kStageBytes % 16 == 0 && kPListEnd % 16 == 0, "16-byte operand buffers");
     // kPCtasPerSm CTAs per SM fit, and no more than four (4 x 128 TMEM columns)
@@ -705,26 +705,44 @@ __global__ void __launch_bounds__(kPThreads, kPCtasPerSm)
         atomicAdd(p.stats + threadIdx.x, block_stats[threadIdx.x]);
 }
 
-// Last view whose first item is <= item (views without items share the
-// next view's first item, so they are skipped).
-__device__ __forceinline__ int find_batch_view(const long long *begin, int nviews, long long item) {
-    int lo = 0, hi = nviews - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (__ldg(begin + mid) <= item) lo = mid;
-        else hi = mid - 1;
+// A producer warp's place in the items of a batch: the view of its current
+// item and that view's items [begin, end).
+struct BatchPlace {
+    int view;
+    long long begin, end;
+};
+
+// The view of `item`: the last one whose first item is <= item (views without
+// items share the next view's first item, so they are skipped).  Items only
+// grow, so the search starts at the current view, 32 views at a time.
+// Warp-collective.
+__device__ __forceinline__ BatchPlace find_batch_view(const long long *begin, int nviews, long long item, int from,
+                                                      int lane) {
+    int k = from;  // begin[k] <= item
+    while (true) {
+        const int i = k + 1 + lane;
+        const bool le = i < nviews && __ldg(begin + i) <= item;
+        const int n = __popc(__ballot_sync(FULL, le));  // (begin is sorted: the first n)
+        k += n;
+        if (n < 32) break;
     }
-    return lo;
+    BatchPlace b;
+    b.view = k;
+    b.begin = __ldg(begin + k);
+    b.end = __ldg(begin + k + 1);
+    return b;
 }
 
-// The learned views of a batch: the packed-group kernel made persistent.
-// The producers take groups (items of 8 tiles) from a global counter, find
-// the group's view, copy its parameters and network into the stage and run
-// step 1 and the features as for one view; the consumer runs the chains and
-// the gather with the stage's copies, and reloads the operand image when a
+// The learned views of a batch: the packed-group kernel made persistent.  CTA
+// c takes the groups (items of 8 tiles) c, c + G, ... of all views, so that
+// every producer warp knows its next group and has its next tile's inputs in
+// flight, as in the single-view kernel (groups from a global counter, a view
+// lookup and a parameter copy between barriers took 579 us for 256 views, of
+// which the learned half was 415).  Each producer warp keeps copies of the
+// parameters and network of its current and its next group's view; the stage
+// carries a copy for the consumer, which reloads the operand image when a
 // group's network is not the one in shared memory (between chains, when no
-// MMA is in flight).  A stage whose view slot is -1 ends the CTA's work.
-
+// MMA is in flight).
 template <int ALG, int TW, int MD, bool kStats>
 __global__ void __launch_bounds__(kPThreads, kPCtasPerSm)
     mlp_batch_pf_kernel(const PfBatch b, const MlpDevice m0, const __grid_constant__ MlpEpilogue ep0) {
@@ -774,7 +792,7 @@ __global__ void __launch_bounds__(kPThreads, kPCtasPerSm)
         const int tid = threadIdx.x;
         uint32_t phase = 0;
         const uint4 *loaded = m0.img;
-        for (long long j = 0;; ++j) {
+        for (long long j = 0; blockIdx.x + j * (long long)gridDim.x < b.total_items; ++j) {
             const int s = (int)(j % kPStages);
             const uint32_t par = (uint32_t)((j / kPStages) & 1);
             unsigned char *st = p_stage<false, true>(sm, s);
@@ -784,10 +802,8 @@ __global__ void __launch_bounds__(kPThreads, kPCtasPerSm)
                 if (tid == 0) atomicExch(err, CTF_ERR_TIMEOUT);
                 break;
             }
-            const int *bm = reinterpret_cast<const int *>(st + kPBat);
-            if (bm[0] < 0) break;  // no more groups
-            const ExactParams &p = *reinterpret_cast<const ExactParams *>(st + kPBat + 16);
-            const MlpDevice &m = *reinterpret_cast<const MlpDevice *>(st + kPBat + 16 + sizeof(ExactParams));
+            const ExactParams &p = *reinterpret_cast<const ExactParams *>(st + kPBat);
+            const MlpDevice &m = *reinterpret_cast<const MlpDevice *>(st + kPBat + sizeof(ExactParams));
             if (m.img != loaded) {
                 // another network: its operand image (every MMA of the last chain is done)
                 const uint4 *src = m.img;
@@ -835,9 +851,49 @@ __global__ void __launch_bounds__(kPThreads, kPCtasPerSm)
         int *ranks = reinterpret_cast<int *>(sm + kPRanks) + 64 * pw;
         int2 *list = reinterpret_cast<int2 *>(sm + kPList);
         const int pt = threadIdx.x - kRows;  // producer thread
-        for (long long j = 0;; ++j) {
+        // this warp's copies of its current and its next group's view
+        unsigned char *own = sm + kPListEnd + 2 * pw * kPViewBytes;
+        auto params = [&](int c) -> const ExactParams & {
+            return *reinterpret_cast<const ExactParams *>(own + c * kPViewBytes);
+        };
+        auto locate = [&](long long it, BatchPlace &at, int c) {
+            at = find_batch_view(b.item_begin, b.nkind, it, at.view, lane);
+            const BatchViewDev *V =
+                b.views + ck(__ldg(b.index + ck(at.view, b.nkind, err, kBndBatch)), b.nviews, err, kBndBatch);
+            __syncwarp();
+            const uint4 *src = reinterpret_cast<const uint4 *>(&V->p);
+            uint4 *dst = reinterpret_cast<uint4 *>(own + c * kPViewBytes);
+            if (lane < (int)(sizeof(ExactParams) / 16)) dst[lane] = __ldg(src + lane);
+            const uint2 *msrc = reinterpret_cast<const uint2 *>(&V->m);
+            uint2 *mdst = reinterpret_cast<uint2 *>(own + c * kPViewBytes + sizeof(ExactParams));
+            if (lane < (int)(sizeof(MlpDevice) / 8)) mdst[lane] = __ldg(msrc + lane);
+            __syncwarp();
+        };
+        auto first_tile = [&](long long it, const BatchPlace &at, int c, uint32_t &x, uint32_t &y) {
+            const uint32_t t = (uint32_t)((it - at.begin) * kPTiles) + (uint32_t)(kPSlots * pw);
+            const uint32_t tiles_x = (uint32_t)params(c).tiles_x;
+            x = t % tiles_x;
+            y = t / tiles_x;
+        };
+        BatchPlace at;
+        at.view = 0;
+        long long item = blockIdx.x;  // (the grid has at most one CTA per item)
+        int cur = 0;
+        locate(item, at, cur);
+        uint32_t bx, by;
+        first_tile(item, at, cur, bx, by);
+        Inputs in = p_load<ALG, TW>(params(cur), LanePlace<TW>(params(cur), lane), bx, by);
+        for (long long j = 0; item < b.total_items; ++j) {
             const int s = (int)(j % kPStages);
             unsigned char *st = p_stage<false, true>(sm, s);
+            // the next group's view (a copy into the other slot when it changes)
+            const long long next_item = item + gridDim.x;
+            const bool more = next_item < b.total_items;
+            int nxt = cur;
+            if (more && next_item >= at.end) {
+                nxt = cur ^ 1;
+                locate(next_item, at, nxt);
+            }
             if (j >= kPStages) {
                 // the consumer has gathered group j - kPStages from this stage
                 const bool okd = tc::mbar_wait(p_done(sm, s), (uint32_t)(((j - kPStages) / kPStages) & 1), kMaxTries);
@@ -853,47 +909,33 @@ __global__ void __launch_bounds__(kPThreads, kPCtasPerSm)
                 __syncwarp();
                 prod_bar();
             }
-            int *bm = reinterpret_cast<int *>(st + kPBat);
-            if (pt == 0) *reinterpret_cast<long long *>(st + kPBat + 8) = (long long)atomicAdd(b.counter, 1ull);
-            prod_bar();
-            const long long item = *reinterpret_cast<volatile long long *>(st + kPBat + 8);
-            if (item >= b.total_items) {
-                if (pt == 0) bm[0] = -1;
-                __syncwarp();
-                if (lane == 0) p_arrive(p_full(sm, s));
-                break;
+            const ExactParams &p = params(cur);
+            const MlpDevice &m = *reinterpret_cast<const MlpDevice *>(own + cur * kPViewBytes + sizeof(ExactParams));
+            if (pw == 0) {  // the view for the consumer
+                const uint4 *src = reinterpret_cast<const uint4 *>(own + cur * kPViewBytes);
+                if (lane < kPViewBytes / 16) reinterpret_cast<uint4 *>(st + kPBat)[lane] = src[lane];
             }
-            const int vk = ck(find_batch_view(b.item_begin, b.nkind, item), b.nkind, err, kBndBatch);
-            const BatchViewDev *V = b.views + ck(__ldg(b.index + vk), b.nviews, err, kBndBatch);
-            {
-                // the view's parameters and network into the stage
-                const uint4 *src = reinterpret_cast<const uint4 *>(&V->p);
-                uint4 *dst = reinterpret_cast<uint4 *>(st + kPBat + 16);
-                if (pt < (int)(sizeof(ExactParams) / 16)) dst[pt] = __ldg(src + pt);
-                const uint2 *msrc = reinterpret_cast<const uint2 *>(&V->m);
-                uint2 *mdst = reinterpret_cast<uint2 *>(st + kPBat + 16 + sizeof(ExactParams));
-                if (pt < (int)(sizeof(MlpDevice) / 8)) mdst[pt] = __ldg(msrc + pt);
-            }
-            const long long first = (item - __ldg(b.item_begin + vk)) * kPTiles;
-            prod_bar();  // the copies are in place
-            if (pt == 0) {
-                bm[0] = vk;
-                *reinterpret_cast<long long *>(st + kPBat + 8) = first;
-            }
-            const ExactParams &p = *reinterpret_cast<const ExactParams *>(st + kPBat + 16);
-            const MlpDevice &m = *reinterpret_cast<const MlpDevice *>(st + kPBat + 16 + sizeof(ExactParams));
             const bool fp8 = m.fp8 != 0;
             const float *inv_a1 = reinterpret_cast<const float *>(reinterpret_cast<const unsigned char *>(m.img) + kImgA1);
             const LanePlace<TW> lp(p, lane);
             const uint32_t tiles_x = (uint32_t)p.tiles_x;
-            const uint32_t mine = (uint32_t)first + (uint32_t)(kPSlots * pw);
-            uint32_t bx = mine % tiles_x, by = mine / tiles_x;
 #pragma unroll 1
             for (int k = 0; k < kPSlots; ++k) {
-                const Inputs in = p_load<ALG, TW>(p, lp, bx, by);
+                uint32_t nx = bx, ny = by;
+                Inputs next;
+                if (k + 1 < kPSlots) {
+                    p_tile(tiles_x, nx, ny, 1u);
+                    next = p_load<ALG, TW>(p, lp, nx, ny);
+                } else {
+                    // (after the last group: this tile's inputs again, unused)
+                    if (more) first_tile(next_item, at, nxt, nx, ny);
+                    next = p_load<ALG, TW>(params(nxt), LanePlace<TW>(params(nxt), lane), nx, ny);
+                }
                 p_step1<ALG, TW, MD, kStats, false>(p, lp, bx, by, in, kPSlots * pw + k, st, list, lane, lt, ranks,
                                                     cnt, nullptr);
-                p_tile(tiles_x, bx, by, 1u);
+                bx = nx;
+                by = ny;
+                in = next;
             }
             // (as in the single-view kernel)
             if (pt == 0) *reinterpret_cast<int *>(p_stage<false, true>(sm, (int)((j + 1) % kPStages)) + S::kAlloc) = 0;
@@ -914,6 +956,8 @@ __global__ void __launch_bounds__(kPThreads, kPCtasPerSm)
             tc::fence_proxy_async();  // generic-proxy writes -> the MMAs' async proxy
             __syncwarp();
             if (lane == 0) p_arrive(p_full(sm, s));
+            item = next_item;
+            cur = nxt;
         }
     }
 
