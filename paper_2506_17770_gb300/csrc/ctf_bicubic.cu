@@ -136,7 +136,7 @@ __global__ void __launch_bounds__(kThreads) bicubic_filter_kernel(const ExactPar
         const uint32_t idx = inside ? (uint32_t)py * (uint32_t)p.W + (uint32_t)px : 0u;
         const Inputs in = load_inputs_any<kJac>(p, inside, idx);
         PixelSetup ps;
-        ps.active = in.covered;
+        ps.active = inside && in.cov != 0;
         setup_coords(in.uv, fW, fH, ps);
         const int ox = ps.ulx - 1, oy = ps.uly - 1;  // the 4x4 footprint's corner
         float wx[4], wy[4];

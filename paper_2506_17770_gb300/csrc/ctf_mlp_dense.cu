@@ -242,7 +242,7 @@ __global__ void __launch_bounds__(kPThreads, kPCtasPerSm)
                 const uint32_t idx = py * (uint32_t)p.W + px;
                 const Inputs in = load_inputs_any<false>(p, inside, idx);
                 PixelSetup ps;
-                ps.active = in.covered;
+                ps.active = inside && in.cov != 0;
                 setup_coords(in.uv, (float)p.Wt, (float)p.Ht, ps);
                 const uint32_t A = __ballot_sync(FULL, ps.active);
                 if (kStats && tile < (uint32_t)p.n_tiles) {

@@ -384,7 +384,7 @@ __device__ __forceinline__ void p_step1(const ExactParams &p, const LanePlace<TW
     const int px = (int)(bx * TW + lp.tx), py = (int)(by * TH + lp.ty);
     const uint32_t pixel = by * (TH * (uint32_t)p.W) + bx * TW;
     PixelSetup ps;
-    ps.active = in.covered;
+    ps.active = inside && in.cov != 0;
     setup_coords(in.uv, (float)p.Wt, (float)p.Ht, ps);
     Selection sel;
     if (!kStats || by * TH < (uint32_t)p.H) {
