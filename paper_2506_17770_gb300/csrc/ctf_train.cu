@@ -9,11 +9,11 @@
 // backward pass as tcgen05 MMAs over them (FP16 operands in shared memory,
 // FP32 accumulation in TMEM; bias, ReLU and the loss in FP32): the layer
 // products, the input-side gradients and the weight gradients, which it
-// sums over its rounds in TMEM.  It adds those sums, like the latent-grid
-// gradient scatter, to 64-bit fixed-point accumulators (integer atomics are
-// order-independent, so a step is deterministic).  An Adam kernel converts
-// the sums back, updates parameters and moments, and clears the
-// accumulators.
+// sums over its rounds in TMEM and leaves as the CTA's partial sums; the
+// latent-grid gradients go to 64-bit fixed-point accumulators (integer
+// atomics are order-independent, so a step is deterministic).  An update
+// kernel adds the partial sums up, applies Adam to every parameter and clears
+// the accumulators it has read.
 #include <cmath>
 #include <cstdint>
 #include <cstdio>
@@ -28,6 +28,7 @@
 #include "../../include/ctf.h"
 #include "ctf_device.cuh"
 #include "ctf_internal.h"
+#include "tc_ops.cuh"
 
 namespace ctf {
 namespace {
@@ -96,13 +97,17 @@ constexpr int kAHK = 176, kAHGroup = kAHK / 8 * 128;  // channels, bytes per 8-r
 constexpr int kChH2 = 0, kChOnes = 64, kChH1 = 80, kChF = 144, kChOnes2 = 160;
 constexpr int kGAH = kGBias + 640;
 constexpr int kDHGroup = 128 / 8 * 128;
+// after a round's MMAs DH holds the rows' dF (64 B each), then per row and grid
+// the four taps' cells and weights (32 B)
+constexpr int kDHTaps = 128 * 64;
+static_assert(kDHTaps + 128 * 2 * 32 <= 16 * kDHGroup, "inside DH");
 constexpr int kGDH = kGAH + 16 * kAHGroup;
 constexpr int kGDE = kGDH + 16 * kDHGroup;
 constexpr int kGXY = kGDE + 16 * 256;             // int2 [128] texel coordinates
 constexpr int kGBar = kGXY + 128 * 8;             // MMA barrier (8 B), TMEM base (4 B)
 constexpr int kGSlot = kGBar + 8;
-constexpr int kGLoss = kGBar + 16;                // float [128] per-thread squared errors
-constexpr int kGradSmemBytes = kGLoss + 128 * 4;
+constexpr int kGLoss = kGBar + 16;                // float per warp: squared errors
+constexpr int kGradSmemBytes = kGLoss + 16;
 static_assert(kGAH % 16 == 0 && kGDH % 16 == 0 && kGDE % 16 == 0, "16-byte operand buffers");
 static_assert(2 * (kGradSmemBytes + 1024) <= 228 * 1024 && 3 * (kGradSmemBytes + 1024) > 228 * 1024,
               "exactly two CTAs (2 x 256 TMEM columns) per SM");
@@ -132,64 +137,28 @@ __device__ __forceinline__ uint32_t relu_h2(float a, float b) {
 // Offset of element (r, k) in a K-major FP16 operand with K channels.
 __device__ __forceinline__ int kofs(int r, int k, int K) { return (r >> 3) * (K / 8) * 128 + (k >> 3) * 128 + (r & 7) * 16 + (k & 7) * 2; }
 
-// One MMA (FP16 operands, FP32 accumulation), issued by one thread.
-__device__ __forceinline__ void tc_mma(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, bool acc) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d),
-        "l"(a), "l"(b), "r"(idesc), "r"((uint32_t)acc)
-        : "memory");
-}
+__device__ __forceinline__ uint32_t saddr_of(const void *p) { return tc::smem_addr(p); }
 
-__device__ __forceinline__ uint64_t sdesc(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
-    uint64_t d = 0;
-    d |= (uint64_t)((saddr >> 4) & 0x3FFFu);
-    d |= (uint64_t)((lbo >> 4) & 0x3FFFu) << 16;
-    d |= (uint64_t)((sbo >> 4) & 0x3FFFu) << 32;
-    d |= (uint64_t)1 << 46;
-    return d;
-}
-
-__device__ __forceinline__ uint32_t saddr_of(const void *p) { return static_cast<uint32_t>(__cvta_generic_to_shared(p)); }
-
-// The MMAs issued since the last commit: thread 0 commits them to the
-// barrier and polls it; every thread learns the outcome at a CTA barrier.
-// Returns false (for all threads alike) if they did not complete within
-// the bound.
-__device__ __forceinline__ bool tc_sync(uint64_t *bar, uint32_t &phase) {
-    bool ok = true;
-    if (threadIdx.x == 0) {
-        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(saddr_of(bar))
-                     : "memory");
-        ok = false;
-        const uint32_t a = saddr_of(bar);
-        for (uint32_t i = 0; i < kGradTries && !ok; ++i) {
-            uint32_t done;
-            asm volatile(
-                "{\n\t.reg .pred p;\n\t"
-                "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-                "selp.u32 %0, 1, 0, p;\n\t}"
-                : "=r"(done)
-                : "r"(a), "r"(phase)
-                : "memory");
-            ok = done != 0;
-        }
-    }
+// The end of the MMAs committed to `bar`, polled by every thread.  Returns
+// false if they did not complete within the bound; the caller goes on and the
+// threads agree on it at their next barrier.
+__device__ __forceinline__ bool tc_wait(uint64_t *bar, uint32_t &phase) {
+    const bool ok = tc::mbar_wait(bar, phase, kGradTries);
     phase ^= 1u;
-    __syncwarp();
-    const bool bad = __syncthreads_or(!ok);
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    return !bad;
+    __syncwarp();  // the TMEM accesses that follow are .aligned
+    tc::fence_after_sync();
+    return ok;
 }
 
 // Generic-proxy shared-memory writes of every thread made visible to the
-// MMAs that thread 0 issues next.
-__device__ __forceinline__ void tc_publish() {
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+// MMAs issued next.  Returns false (for all threads alike) if a thread gave
+// up a wait.
+__device__ __forceinline__ bool tc_publish(bool bad) {
+    tc::fence_proxy_async();
+    tc::fence_before_sync();
+    const bool any = __syncthreads_or(bad);
+    tc::fence_after_sync();
+    return !any;
 }
 
 __device__ __forceinline__ void tld16(uint32_t taddr, float v[16]) {
@@ -233,10 +202,65 @@ __device__ __forceinline__ void bilinear_taps(const GradParams &g, int grid, int
 }
 
 
-// The gradient kernel's weight image (the first kGAH bytes of its shared
-// memory): W1, W2, W3 (padded) and their transposes as FP16 operands, the
-// biases in FP32, from the current FP32 master parameters.  One thread per
-// parameter of the network.
+// Programmatic dependent launch: wait for the kernels before this one in the
+// stream (at once when it was launched without the attribute), and let the
+// one after it start.
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// Texel i of the step's batch.
+__device__ __forceinline__ void sample_texel(const GradParams &g, uint32_t i, int &x, int &y) {
+    const uint4 rr = philox4x32_10(make_uint4(i, g.step, 0x5A4Du, 0u), g.k0, g.k1);
+    x = (int)(((unsigned long long)rr.x * (unsigned)g.Wt) >> 32);
+    y = (int)(((unsigned long long)rr.y * (unsigned)g.Ht) >> 32);
+}
+
+// A CTA's partial weight-gradient sums, in the order in which its threads
+// hold them (thread m row m of the two products), so that a warp stores 32
+// neighbours: dW2 [input][output], dW1 [input][output], db2, db1, dW3, db3.
+// (In parameter order every lane stored to a sector of its own, 1.6 million
+// sectors a step at batch 8,192.)
+constexpr int kSlotW1 = 4096, kSlotB = 5120, kSlotW3 = 5248, kSlotB3 = 5504;
+
+// The parameter of slot s.
+__device__ __forceinline__ int slot_param(int s) {
+    if (s < kSlotW1) return kOffW2 + (s & 63) * 64 + (s >> 6);
+    if (s < kSlotB) return kOffW1 + (s & 63) * 16 + ((s - kSlotW1) >> 6);
+    if (s < kSlotB + 64) return kOffB2 + s - kSlotB;
+    if (s < kSlotW3) return kOffB1 + s - kSlotB - 64;
+    return s - kSlotW3 + kOffW3;  // dW3 and db3 follow one another in both
+}
+static_assert(kSlotB3 - kSlotW3 == kOffB3 - kOffW3 && kSlotB3 + 4 == kWeights, "one slot per parameter");
+
+// Where parameter e of the network goes in the gradient kernel's weight image
+// (the first kGAH bytes of its shared memory: W1, W2, W3 and their transposes
+// as FP16 operands, the biases in FP32).
+__device__ __forceinline__ void put_weight(unsigned char *img, int e, float v) {
+    const __half w = __float2half_rn(v);
+    if (e < kOffB1) {
+        const int o = e >> 4, k = e & 15;
+        *reinterpret_cast<__half *>(img + kGW1 + kofs(o, k, 16)) = w;
+        *reinterpret_cast<__half *>(img + kGW1T + kofs(k, o, 64)) = w;
+    } else if (e < kOffW2) {
+        reinterpret_cast<float *>(img + kGBias)[e - kOffB1] = v;
+    } else if (e < kOffB2) {
+        const int j = e - kOffW2, o = j >> 6, k = j & 63;
+        *reinterpret_cast<__half *>(img + kGW2 + kofs(o, k, 64)) = w;
+        *reinterpret_cast<__half *>(img + kGW2T + kofs(k, o, 64)) = w;
+    } else if (e < kOffW3) {
+        reinterpret_cast<float *>(img + kGBias)[64 + e - kOffB2] = v;
+    } else if (e < kOffB3) {
+        const int j = e - kOffW3, c = j >> 6, k = j & 63;
+        *reinterpret_cast<__half *>(img + kGW3 + kofs(c, k, 64)) = w;
+        *reinterpret_cast<__half *>(img + kGW3T + kofs(k, c, 16)) = w;
+    } else {
+        reinterpret_cast<float *>(img + kGBias)[128 + e - kOffB3] = v;
+    }
+}
+
+// Before the first step of a call: the weight image from the current FP32
+// master parameters (the updates keep it current from then on).  One thread
+// per element.
 __global__ void pack_kernel(const float *params, unsigned char *img) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < 1024) {
@@ -280,18 +304,13 @@ static_assert(kGBias + 160 * 4 == kGAH, "the image ends where the activations be
 __global__ void __launch_bounds__(kT, 2) grad_kernel(const GradParams g) {
     extern __shared__ __align__(1024) unsigned char sm[];
     const int tid = threadIdx.x;
+    const int warp = __shfl_sync(FULL, tid >> 5, 0);  // uniform, and known to be
     uint64_t *bar = reinterpret_cast<uint64_t *>(sm + kGBar);
     uint32_t *slot = reinterpret_cast<uint32_t *>(sm + kGSlot);
     float *sloss = reinterpret_cast<float *>(sm + kGLoss);
     unsigned char *AH = sm + kGAH, *DH = sm + kGDH, *DE = sm + kGDE;
     const float *P = g.params;  // latents (FP32 master values)
-    // ---- the weights as FP16 operands and the biases (the image that
-    // pack_kernel made from the current parameters), the constant ones blocks
-    {
-        const uint4 *src = reinterpret_cast<const uint4 *>(g.wimg);
-        uint4 *dst = reinterpret_cast<uint4 *>(sm);
-        for (int i = tid; i < kGAH / 16; i += kT) dst[i] = __ldg(src + i);
-    }
+    // ---- the constant ones blocks, and zero features in rows that no round uses
     const float *B = reinterpret_cast<const float *>(sm + kGBias);
     {
         // the ones blocks of every row: channels 64 and 160 are 1, the rest of
@@ -301,20 +320,21 @@ __global__ void __launch_bounds__(kT, 2) grad_kernel(const GradParams g) {
         *reinterpret_cast<uint4 *>(AH + kofs(tid, kChOnes + 8, kAHK)) = zero;
         *reinterpret_cast<uint4 *>(AH + kofs(tid, kChOnes2, kAHK)) = one;
         *reinterpret_cast<uint4 *>(AH + kofs(tid, kChOnes2 + 8, kAHK)) = zero;
+        *reinterpret_cast<uint4 *>(AH + kofs(tid, kChF, kAHK)) = zero;
+        *reinterpret_cast<uint4 *>(AH + kofs(tid, kChF + 8, kAHK)) = zero;
     }
     if (tid == 0) {
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(saddr_of(bar)) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (tid < 32) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(saddr_of(slot)),
-                     "r"(kTcCols)
-                     : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    if (warp == 0) {
+        __syncwarp();  // tcgen05.alloc needs the whole warp
+        tc::tmem_alloc(slot, kTcCols);
+        tc::tmem_relinquish();
     }
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    tc::fence_before_sync();
     __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    tc::fence_after_sync();
     const uint32_t tmem = *slot;
     const uint32_t lane_t = tmem + ((uint32_t)(32 * (tid >> 5)) << 16);  // this thread's TMEM lane
     uint32_t phase = 0;
@@ -325,64 +345,89 @@ __global__ void __launch_bounds__(kT, 2) grad_kernel(const GradParams g) {
     const uint32_t idW1 = idesc_f16_t(128, 96, 1, 1), idW2 = idesc_f16_t(128, 16, 1, 1);
     float loss = 0.f;
 
-#pragma unroll 1
-    for (int r = 0; r < g.rounds && ok; ++r) {
-        const int i0 = (blockIdx.x * g.rounds + r) * g.per_round;
-        const int i = i0 + tid;
-        const bool valid = tid < g.per_round && i < g.n;
-        // ---- the texel of row tid, its features and its target
-        int x, y;
+    // Half rounds (64 texels): two threads share a texel, one latent grid
+    // each, for the features and for the gradient scatter; the rows past the
+    // texels keep zero features.
+    const bool half = g.per_round <= kT / 2;
+    const int row = half ? tid & (kT / 2 - 1) : tid;
+    const int g_lo = half ? tid / (kT / 2) : 0, g_hi = half ? g_lo + 1 : 2;
+    // This thread's texel of round r (`there`; `valid`: it is row tid's) and
+    // its target.
+    int x, y;
+    bool there, valid;
+    float tgt[4];
+    auto pick = [&](int r) {
+        const int i = (blockIdx.x * g.rounds + r) * g.per_round + row;
+        there = row < g.per_round && i < g.n;
+        valid = there && row == tid;
         if (g.xy) {
-            const int2 c = valid ? g.xy[ck(i, g.n, g.err, kBndTrain)] : make_int2(0, 0);
+            const int2 c = there ? g.xy[ck(i, g.n, g.err, kBndTrain)] : make_int2(0, 0);
             x = min(max(c.x, 0), g.Wt - 1);
             y = min(max(c.y, 0), g.Ht - 1);
         } else {
-            const uint4 rr = philox4x32_10(make_uint4((uint32_t)i, g.step, 0x5A4Du, 0u), g.k0, g.k1);
-            x = (int)(((unsigned long long)rr.x * (unsigned)g.Wt) >> 32);
-            y = (int)(((unsigned long long)rr.y * (unsigned)g.Ht) >> 32);
+            sample_texel(g, (uint32_t)i, x, y);
         }
-        {
-            float f[16];
+        const uint32_t px = fetch_block_texel(g.blocks, g.nbx, g.Wt, g.Ht, x, y, g.err);
 #pragma unroll
-            for (int gi = 0; gi < 2; ++gi) {
-                int tap[4];
-                float tw[4];
-                bilinear_taps(g, gi, x, y, tap, tw);
-                const float *lg = P + kOffLat + (gi ? lat1 : 0);
-                float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        for (int c = 0; c < 4; ++c) tgt[c] = __fdiv_rn((float)((px >> (8 * c)) & 0xffu), 255.f);
+    };
+    pick(0);
+    // Launched as the dependent of the previous step's update: what comes
+    // before this line (the first texels and their targets too) overlaps its
+    // end.  The next update may start from here on (it only loads before it
+    // waits for this kernel).
+    grid_wait();
+    grid_trigger();
+    // ---- the weights as FP16 operands and the biases (the image made from
+    // the current parameters): in flight together with the first latents
+    constexpr int kImg16 = kGAH / 16, kImgLoads = (kImg16 + kT - 1) / kT;
+    uint4 img[kImgLoads];
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const float4 v0 = __ldg(reinterpret_cast<const float4 *>(lg + (size_t)tap[k] * 8));
-                    const float4 v1 = __ldg(reinterpret_cast<const float4 *>(lg + (size_t)tap[k] * 8 + 4));
-                    acc[0] = __fmaf_rn(tw[k], v0.x, acc[0]);
-                    acc[1] = __fmaf_rn(tw[k], v0.y, acc[1]);
-                    acc[2] = __fmaf_rn(tw[k], v0.z, acc[2]);
-                    acc[3] = __fmaf_rn(tw[k], v0.w, acc[3]);
-                    acc[4] = __fmaf_rn(tw[k], v1.x, acc[4]);
-                    acc[5] = __fmaf_rn(tw[k], v1.y, acc[5]);
-                    acc[6] = __fmaf_rn(tw[k], v1.z, acc[6]);
-                    acc[7] = __fmaf_rn(tw[k], v1.w, acc[7]);
-                }
+    for (int k = 0; k < kImgLoads; ++k)
+        img[k] = __ldcg(reinterpret_cast<const uint4 *>(g.wimg) + min(tid + k * kT, kImg16 - 1));
+    bool bad = false;
+#pragma unroll 1
+    for (int r = 0; r < g.rounds && ok; ++r) {
+#pragma unroll 1
+        for (int gi = g_lo; gi < g_hi; ++gi) {
+            int tap[4];
+            float tw[4];
+            bilinear_taps(g, gi, x, y, tap, tw);
+            const float *lg = P + kOffLat + (gi ? lat1 : 0);
+            float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+            float4 v0[4], v1[4];
 #pragma unroll
-                for (int c = 0; c < 8; ++c) f[gi * 8 + c] = acc[c];
+            for (int k = 0; k < 4; ++k) {
+                v0[k] = __ldcg(reinterpret_cast<const float4 *>(lg + (size_t)tap[k] * 8));
+                v1[k] = __ldcg(reinterpret_cast<const float4 *>(lg + (size_t)tap[k] * 8 + 4));
             }
-            *reinterpret_cast<uint4 *>(AH + kofs(tid, kChF, kAHK)) =
-                make_uint4(h2pack(f[0], f[1]), h2pack(f[2], f[3]), h2pack(f[4], f[5]), h2pack(f[6], f[7]));
-            *reinterpret_cast<uint4 *>(AH + kofs(tid, kChF + 8, kAHK)) =
-                make_uint4(h2pack(f[8], f[9]), h2pack(f[10], f[11]), h2pack(f[12], f[13]), h2pack(f[14], f[15]));
-        }
-        float tgt[4];
-        {
-            const uint32_t px = fetch_block_texel(g.blocks, g.nbx, g.Wt, g.Ht, x, y, g.err);
+            if (r == 0 && gi == g_lo) {
 #pragma unroll
-            for (int c = 0; c < 4; ++c) tgt[c] = __fdiv_rn((float)((px >> (8 * c)) & 0xffu), 255.f);
+                for (int k = 0; k < kImgLoads; ++k)
+                    if (tid + k * kT < kImg16) reinterpret_cast<uint4 *>(sm)[tid + k * kT] = img[k];
+            }
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                acc[0] = __fmaf_rn(tw[k], v0[k].x, acc[0]);
+                acc[1] = __fmaf_rn(tw[k], v0[k].y, acc[1]);
+                acc[2] = __fmaf_rn(tw[k], v0[k].z, acc[2]);
+                acc[3] = __fmaf_rn(tw[k], v0[k].w, acc[3]);
+                acc[4] = __fmaf_rn(tw[k], v1[k].x, acc[4]);
+                acc[5] = __fmaf_rn(tw[k], v1[k].y, acc[5]);
+                acc[6] = __fmaf_rn(tw[k], v1[k].z, acc[6]);
+                acc[7] = __fmaf_rn(tw[k], v1[k].w, acc[7]);
+            }
+            *reinterpret_cast<uint4 *>(AH + kofs(row, kChF + 8 * gi, kAHK)) =
+                make_uint4(h2pack(acc[0], acc[1]), h2pack(acc[2], acc[3]), h2pack(acc[4], acc[5]), h2pack(acc[6], acc[7]));
         }
-        tc_publish();
+        if (!(ok = tc_publish(bad))) break;
         // ---- H1 = relu(F W1^T + b1)
-        if (tid == 0)
-            tc_mma(tmem + kColA, sdesc(sAH + kChF / 8 * 128, 128, kAHGroup), sdesc(saddr_of(sm + kGW1), 128, 256), id64,
-                   false);
-        if (!(ok = tc_sync(bar, phase))) break;
+        if (warp == 0 && tc::elect_one()) {
+            tc::mma_f16(tmem + kColA, tc::smem_desc(sAH + kChF / 8 * 128, 128, kAHGroup),
+                        tc::smem_desc(saddr_of(sm + kGW1), 128, 256), id64, false);
+            tc::commit(bar);
+        }
+        bad |= !tc_wait(bar, phase);
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             float d[16];
@@ -394,13 +439,16 @@ __global__ void __launch_bounds__(kT, 2) grad_kernel(const GradParams g) {
             *reinterpret_cast<uint4 *>(AH + kofs(tid, kChH1 + 16 * q, kAHK)) = make_uint4(w[0], w[1], w[2], w[3]);
             *reinterpret_cast<uint4 *>(AH + kofs(tid, kChH1 + 16 * q + 8, kAHK)) = make_uint4(w[4], w[5], w[6], w[7]);
         }
-        tc_publish();
+        if (!(ok = tc_publish(bad))) break;
         // ---- H2 = relu(H1 W2^T + b2)
-        if (tid == 0)
+        if (warp == 0 && tc::elect_one()) {
+#pragma unroll
             for (int j = 0; j < 4; ++j)
-                tc_mma(tmem + kColB, sdesc(sAH + kChH1 / 8 * 128 + 256 * j, 128, kAHGroup),
-                       sdesc(saddr_of(sm + kGW2) + 256 * j, 128, 1024), id64, j > 0);
-        if (!(ok = tc_sync(bar, phase))) break;
+                tc::mma_f16(tmem + kColB, tc::smem_desc(sAH + kChH1 / 8 * 128 + 256 * j, 128, kAHGroup),
+                       tc::smem_desc(saddr_of(sm + kGW2) + 256 * j, 128, 1024), id64, j > 0);
+            tc::commit(bar);
+        }
+        bad |= !tc_wait(bar, phase);
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             float d[16];
@@ -413,13 +461,16 @@ __global__ void __launch_bounds__(kT, 2) grad_kernel(const GradParams g) {
             *reinterpret_cast<uint4 *>(AH + kofs(tid, kChH2 + 16 * q, kAHK)) = make_uint4(w[0], w[1], w[2], w[3]);
             *reinterpret_cast<uint4 *>(AH + kofs(tid, kChH2 + 16 * q + 8, kAHK)) = make_uint4(w[4], w[5], w[6], w[7]);
         }
-        tc_publish();
+        if (!(ok = tc_publish(bad))) break;
         // ---- Y = H2 W3^T + b3, e = Y - target (0 past the batch)
-        if (tid == 0)
+        if (warp == 0 && tc::elect_one()) {
+#pragma unroll
             for (int j = 0; j < 4; ++j)
-                tc_mma(tmem + kColC, sdesc(sAH + kChH2 / 8 * 128 + 256 * j, 128, kAHGroup),
-                       sdesc(saddr_of(sm + kGW3) + 256 * j, 128, 1024), id16, j > 0);
-        if (!(ok = tc_sync(bar, phase))) break;
+                tc::mma_f16(tmem + kColC, tc::smem_desc(sAH + kChH2 / 8 * 128 + 256 * j, 128, kAHGroup),
+                       tc::smem_desc(saddr_of(sm + kGW3) + 256 * j, 128, 1024), id16, j > 0);
+            tc::commit(bar);
+        }
+        bad |= !tc_wait(bar, phase);
         {
             float d[16];
             tld16(lane_t + kColC, d);
@@ -432,11 +483,14 @@ __global__ void __launch_bounds__(kT, 2) grad_kernel(const GradParams g) {
             *reinterpret_cast<uint4 *>(DE + kofs(tid, 0, 16)) = make_uint4(h2pack(e[0], e[1]), h2pack(e[2], e[3]), 0u, 0u);
             *reinterpret_cast<uint4 *>(DE + kofs(tid, 8, 16)) = make_uint4(0u, 0u, 0u, 0u);
         }
-        tc_publish();
+        if (!(ok = tc_publish(bad))) break;
         // ---- dH2 = (e W3) masked by H2 > 0
-        if (tid == 0)
-            tc_mma(tmem + kColA, sdesc(sDE, 128, 256), sdesc(saddr_of(sm + kGW3T), 128, 256), id64, false);
-        if (!(ok = tc_sync(bar, phase))) break;
+        if (warp == 0 && tc::elect_one()) {
+            tc::mma_f16(tmem + kColA, tc::smem_desc(sDE, 128, 256), tc::smem_desc(saddr_of(sm + kGW3T), 128, 256), id64,
+                        false);
+            tc::commit(bar);
+        }
+        bad |= !tc_wait(bar, phase);
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             float d[16];
@@ -453,13 +507,17 @@ __global__ void __launch_bounds__(kT, 2) grad_kernel(const GradParams g) {
             *reinterpret_cast<uint4 *>(DH + kofs(tid, 16 * q, 128)) = make_uint4(w[0], w[1], w[2], w[3]);
             *reinterpret_cast<uint4 *>(DH + kofs(tid, 16 * q + 8, 128)) = make_uint4(w[4], w[5], w[6], w[7]);
         }
-        tc_publish();
+        if (!(ok = tc_publish(bad))) break;
         // ---- dH1 = (dH2 W2) masked by H1 > 0
-        if (tid == 0)
+        if (warp == 0 && tc::elect_one()) {
+#pragma unroll
             for (int j = 0; j < 4; ++j)
-                tc_mma(tmem + kColB, sdesc(sDH + 256 * j, 128, kDHGroup), sdesc(saddr_of(sm + kGW2T) + 256 * j, 128, 1024),
+                tc::mma_f16(tmem + kColB, tc::smem_desc(sDH + 256 * j, 128, kDHGroup),
+                            tc::smem_desc(saddr_of(sm + kGW2T) + 256 * j, 128, 1024),
                        id64, j > 0);
-        if (!(ok = tc_sync(bar, phase))) break;
+            tc::commit(bar);
+        }
+        bad |= !tc_wait(bar, phase);
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             float d[16];
@@ -476,49 +534,69 @@ __global__ void __launch_bounds__(kT, 2) grad_kernel(const GradParams g) {
             *reinterpret_cast<uint4 *>(DH + kofs(tid, 64 + 16 * q, 128)) = make_uint4(w[0], w[1], w[2], w[3]);
             *reinterpret_cast<uint4 *>(DH + kofs(tid, 64 + 16 * q + 8, 128)) = make_uint4(w[4], w[5], w[6], w[7]);
         }
-        tc_publish();
+        if (!(ok = tc_publish(bad))) break;
         // ---- dF = dH1 W1; the weight gradients of the round (texels as the
         // reduction index, both operands read MN-major)
-        if (tid == 0) {
+        if (warp == 0 && tc::elect_one()) {
+#pragma unroll
             for (int j = 0; j < 4; ++j)
-                tc_mma(tmem + kColC, sdesc(sDH + 64 / 8 * 128 + 256 * j, 128, kDHGroup),
-                       sdesc(saddr_of(sm + kGW1T) + 256 * j, 128, 1024), id16, j > 0);
+                tc::mma_f16(tmem + kColC, tc::smem_desc(sDH + 64 / 8 * 128 + 256 * j, 128, kDHGroup),
+                       tc::smem_desc(saddr_of(sm + kGW1T) + 256 * j, 128, 1024), id16, j > 0);
             for (int s = 0; s < kT / 16; ++s) {
                 const bool acc = r > 0 || s > 0;
                 // [dH2 dH1]^T [H1 F 1]: A = DH (channels along MN), B = AH channels 80..175
-                tc_mma(tmem + kColWG1, sdesc(sDH + 2 * kDHGroup * s, kDHGroup, 128),
-                       sdesc(sAH + kChH1 / 8 * 128 + 2 * kAHGroup * s, kAHGroup, 128), idW1, acc);
+                tc::mma_f16(tmem + kColWG1, tc::smem_desc(sDH + 2 * kDHGroup * s, kDHGroup, 128),
+                       tc::smem_desc(sAH + kChH1 / 8 * 128 + 2 * kAHGroup * s, kAHGroup, 128), idW1, acc);
                 // [H2 1 H1]^T e: A = AH channels 0..127, B = DE
-                tc_mma(tmem + kColWG2, sdesc(sAH + 2 * kAHGroup * s, kAHGroup, 128), sdesc(sDE + 512 * s, 256, 128),
+                tc::mma_f16(tmem + kColWG2, tc::smem_desc(sAH + 2 * kAHGroup * s, kAHGroup, 128), tc::smem_desc(sDE + 512 * s, 256, 128),
                        idW2, acc);
             }
+            tc::commit(bar);
         }
-        if (!(ok = tc_sync(bar, phase))) break;
-        // ---- the latent-grid gradient of texel row tid
-        float df[16];
-        tld16(lane_t + kColC, df);  // warp-collective: every lane takes it
-        if (valid) {
+        bad |= !tc_wait(bar, phase);
+        // ---- the latent-grid gradient.  The rows' dF, taps and tap weights go
+        // through shared memory (DH, which the MMAs have read), and a warp adds
+        // one texel and grid at a time: 8 lanes a cell, its four cells side by
+        // side, so that a warp's atomics go to 8 sectors and not to 32.
+        {
+            float df[16];
+            tld16(lane_t + kColC, df);  // warp-collective: every lane takes it
 #pragma unroll
-            for (int gi = 0; gi < 2; ++gi) {
+            for (int c = 0; c < 4; ++c)
+                *reinterpret_cast<float4 *>(DH + 64 * tid + 16 * c) =
+                    make_float4(df[4 * c], df[4 * c + 1], df[4 * c + 2], df[4 * c + 3]);
+            for (int gi = g_lo; gi < g_hi; ++gi) {
                 int tap[4];
                 float tw[4];
                 bilinear_taps(g, gi, x, y, tap, tw);
-                unsigned long long *gl = reinterpret_cast<unsigned long long *>(g.grad + kOffLat + (gi ? lat1 : 0));
-                const uint32_t cell0 = gi ? (uint32_t)(lat1 / 8) : 0u;
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const uint32_t cell = cell0 + (uint32_t)tap[k];
-                    atomicOr(g.touched + (cell >> 5), 1u << (cell & 31u));
-                    const float wk = __fmul_rn(tw[k], g.dscale);
-#pragma unroll
-                    for (int ch = 0; ch < 8; ++ch) {
-                        const long long v = to_fix(__fmul_rn(wk, df[gi * 8 + ch]));
-                        if (v) atomicAdd(gl + (size_t)tap[k] * 8 + ch, (unsigned long long)v);
-                    }
+                *reinterpret_cast<int4 *>(DH + kDHTaps + 32 * (2 * row + gi)) = make_int4(tap[0], tap[1], tap[2], tap[3]);
+                *reinterpret_cast<float4 *>(DH + kDHTaps + 32 * (2 * row + gi) + 16) =
+                    make_float4(__fmul_rn(tw[0], g.dscale), __fmul_rn(tw[1], g.dscale), __fmul_rn(tw[2], g.dscale),
+                                __fmul_rn(tw[3], g.dscale));
+            }
+        }
+        if (!(ok = !__syncthreads_or(bad))) break;
+        {
+            const int lane = tid & 31, k = lane >> 3, ch = lane & 7, row0 = row - lane;
+            const int n = __popc(__ballot_sync(FULL, there));  // (the warp's texels are its first n rows)
+            for (int gi = g_lo; gi < g_hi; ++gi) {
+                unsigned long long *gl = reinterpret_cast<unsigned long long *>(g.grad + kOffLat + (gi ? lat1 : 0)) + ch;
+                const uint32_t bit0 = gi ? (uint32_t)(lat1 / 8) : 0u;
+#pragma unroll 4
+                for (int t = 0; t < n; ++t) {
+                    const unsigned char *rec = DH + kDHTaps + 32 * (2 * (row0 + t) + gi) + 4 * k;
+                    const int cell = *reinterpret_cast<const int *>(rec);
+                    const float w = *reinterpret_cast<const float *>(rec + 16);
+                    const float df = *reinterpret_cast<const float *>(DH + 64 * (row0 + t) + 32 * gi + 4 * ch);
+                    if (ch == 0) atomicOr(g.touched + ((bit0 + (uint32_t)cell) >> 5), 1u << ((bit0 + (uint32_t)cell) & 31u));
+                    const long long v = to_fix(__fmul_rn(w, df));
+                    if (v) atomicAdd(gl + (size_t)cell * 8, (unsigned long long)v);
                 }
             }
         }
+        if (r + 1 < g.rounds) pick(r + 1);
     }
+    if (ok) ok = !__syncthreads_or(bad);
     // ---- the CTA's weight-gradient sums, row m = tid of the two products,
     // stored as this CTA's partial sums (reduce_kernel adds the CTAs' up in
     // CTA order: no atomics on the few thousand weight entries)
@@ -532,9 +610,9 @@ __global__ void __launch_bounds__(kT, 2) grad_kernel(const GradParams g) {
 #pragma unroll
             for (int j = 0; j < 16; ++j) {
                 const int n = 16 * q + j;
-                if (m < 64 && n < 64) W[kOffW2 + m * 64 + n] = d[j];                          // dW2
-                else if (m >= 64 && n >= 64 && n < 80) W[kOffW1 + (m - 64) * 16 + (n - 64)] = d[j];  // dW1
-                else if (n == 80) W[m < 64 ? kOffB2 + m : kOffB1 + (m - 64)] = d[j];           // db2, db1
+                if (m < 64 && n < 64) W[n * 64 + m] = d[j];                              // dW2
+                else if (m >= 64 && n >= 64 && n < 80) W[kSlotW1 + (n - 64) * 64 + m - 64] = d[j];  // dW1
+                else if (n == 80) W[kSlotB + m] = d[j];                                  // db2, db1
             }
         }
         {
@@ -542,24 +620,26 @@ __global__ void __launch_bounds__(kT, 2) grad_kernel(const GradParams g) {
             tld16(lane_t + kColWG2, d);
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
-                if (m < 64) W[kOffW3 + c * 64 + m] = d[c];
-                else if (m == 64) W[kOffB3 + c] = d[c];
+                if (m < 64) W[kSlotW3 + c * 64 + m] = d[c];
+                else if (m == 64) W[kSlotB3 + c] = d[c];
             }
         }
-        sloss[tid] = loss;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) loss = __fadd_rn(loss, __shfl_xor_sync(FULL, loss, o));
+        if ((tid & 31) == 0) sloss[warp] = loss;
     }
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    tc::fence_before_sync();
     __syncthreads();
     if (ok && tid == 0) {
         float tot = 0.f;
-        for (int s = 0; s < kT; ++s) tot = __fadd_rn(tot, sloss[s]);
+        for (int s = 0; s < kT / 32; ++s) tot = __fadd_rn(tot, sloss[s]);
         atomicAdd(reinterpret_cast<unsigned long long *>(g.loss), (unsigned long long)__double2ll_rn((double)tot * kLossFix));
     }
     if (!ok && tid == 0 && g.err) atomicExch(g.err, CTF_ERR_TIMEOUT);
-    if (tid < 32) {
-        __syncwarp();
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTcCols) : "memory");
+    if (warp == 0) {
+        __syncwarp();  // tcgen05.dealloc needs the whole warp
+        tc::fence_after_sync();
+        tc::tmem_dealloc(tmem, kTcCols);
     }
 }
 
@@ -569,40 +649,51 @@ __global__ void __launch_bounds__(kT, 2) grad_kernel(const GradParams g) {
 // issued 8 at a time), and the 16 row sums are added in row order, so the
 // result does not depend on timing.
 constexpr int kRedEntries = 16, kRedRows = 16;
+
+// Thread row `row`'s share of slot e: every 16th CTA in order.
+__device__ __forceinline__ double partial_sum(const float *partial, int ctas, int e, int row) {
+    double acc = 0.0;
+    for (int c0 = row; c0 < ctas; c0 += 8 * kRedRows) {
+        float v[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const int c = c0 + j * kRedRows;
+            v[j] = c < ctas ? __ldcg(partial + (size_t)c * kWeights + e) : 0.f;
+        }
+#pragma unroll
+        for (int j = 0; j < 8; ++j) acc += (double)v[j];
+    }
+    return acc;
+}
+
 __global__ void __launch_bounds__(kRedEntries * kRedRows) reduce_kernel(const float *partial, int ctas, double dscale,
                                                                        long long *grad) {
     __shared__ double part[kRedRows][kRedEntries];
     const int e = blockIdx.x * kRedEntries + (threadIdx.x % kRedEntries), row = threadIdx.x / kRedEntries;
-    double acc = 0.0;
-    if (e < kWeights) {
-        for (int c0 = row; c0 < ctas; c0 += 8 * kRedRows) {
-            float v[8];
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                const int c = c0 + j * kRedRows;
-                v[j] = c < ctas ? __ldg(partial + (size_t)c * kWeights + e) : 0.f;
-            }
-#pragma unroll
-            for (int j = 0; j < 8; ++j) acc += (double)v[j];
-        }
-    }
-    part[row][threadIdx.x % kRedEntries] = acc;
+    part[row][threadIdx.x % kRedEntries] = e < kWeights ? partial_sum(partial, ctas, e, row) : 0.0;
     __syncthreads();
     if (row == 0 && e < kWeights) {
         double tot = 0.0;
         for (int r = 0; r < kRedRows; ++r) tot += part[r][threadIdx.x];
-        grad[e] = __double2ll_rn(tot * dscale * kFix);
+        grad[slot_param(e)] = __double2ll_rn(tot * dscale * kFix);
     }
 }
 
 struct AdamParams {
     float *params, *m, *v;
     long long *grad;
-    const uint32_t *touched;  // latent cells with a gradient this step (the others' gradients are zero)
     size_t n;
     float beta1, beta2, eps;
     float step_w, step_lat;  // learning rate / (1 - beta1^t), weights and latents
     float inv_bc2;           // 1 / (1 - beta2^t)
+    const uint32_t *touched;  // latent cells with a gradient this step (the others' gradients are zero)
+    uint32_t *touched_next;   // the next step's, cleared here
+    size_t words;
+    const float *partial;    // the gradient kernel's weight sums, `ctas` of them
+    int ctas;
+    double dscale;           // 2 / batch
+    unsigned char *wimg;     // the weight image, kept current
+    int descending;          // walk the latents from the last one down
 };
 
 __device__ __forceinline__ float sqrt_approx(float x) {
@@ -630,62 +721,119 @@ __device__ __forceinline__ void adam_quad(const AdamParams &a, float step, float
     adam_update(a, g23.y, step, p.w, m.w, v.w);
 }
 
-// Whether quad q has a gradient to read: the weights always, a latent quad
-// (half of a cell's 8 channels) when a texel of the step reached its cell.
-// The gradient of any other latent is exactly zero, so skipping its read and
-// its clearing leaves every update bit for bit the same.
-__device__ __forceinline__ bool quad_has_grad(const AdamParams &a, size_t q) {
-    if (q < (size_t)kOffLat / 4) return true;
-    const size_t cell = (4 * q - kOffLat) >> 3;
-    return (__ldg(a.touched + (cell >> 5)) >> (cell & 31)) & 1u;
-}
-
-// Four parameters per quad, two quads per iteration so that both sets of
-// loads are in flight together.  The buffer length and the start of the
-// latents are multiples of 4; the padding quad (parameters, moments and
-// gradients all zero) stays zero.
-__global__ void adam_kernel(const AdamParams a) {
-    static_assert(kWeights % 4 == 0 && kOffLat == kWeights + 4, "one padding quad");
-    const size_t n4 = a.n / 4, stride = (size_t)gridDim.x * blockDim.x;
-    float4 *__restrict__ P = reinterpret_cast<float4 *>(a.params);
-    float4 *__restrict__ M = reinterpret_cast<float4 *>(a.m);
-    float4 *__restrict__ V = reinterpret_cast<float4 *>(a.v);
-    longlong2 *__restrict__ G = reinterpret_cast<longlong2 *>(a.grad);
+// One step's update, launched as the dependent of the gradient kernel: Adam
+// on the weights (the CTAs' partial sums added in CTA order, as in
+// reduce_kernel), which also refreshes their operand image, and on the
+// latents, reading and clearing the gradients of the cells that a texel
+// reached only (every other gradient is exactly zero, so each update is bit
+// for bit the same).  Bound by the 24 bytes per parameter of parameters and
+// moments.  Each thread loads its first quads before it waits for the
+// gradients, which do not change them.
+// The latents are walked upwards in one step and downwards in the next, so
+// that a step begins with the cells that the last one left in L2 (4096^2
+// texture: 85 us a step with one direction, 71 with both).
+// A 4096^2 step of 8,192 texels took 93 us as seven launches: weight image
+// 4.4, gradients 27.3, weight sums 8.3, Adam 41.4, two memsets and the gaps.
+// Now 17 us of gradients and 47 of update.  Measured and not kept: the
+// untouched cells (nearly all) updated beside the gradient kernel (66-74 us:
+// the moment traffic slows the gradients by as much as it hides), chunks from
+// a counter (72), one, three or four quads in flight or two or four CTAs per
+// SM (70-96), parts of the state kept in L2 by eviction policy (70-73).
+constexpr int kUpThreads = 256, kUpCtasPerSm = 3, kUpQuads = 2;
+__global__ void __launch_bounds__(kUpThreads, kUpCtasPerSm) update_kernel(const AdamParams a) {
+    static_assert(kUpThreads == kRedEntries * kRedRows, "the weight sums' thread layout");
+    __shared__ double part[kRedRows][kRedEntries];
+    float4 *__restrict__ P = reinterpret_cast<float4 *>(a.params + kOffLat);
+    float4 *__restrict__ M = reinterpret_cast<float4 *>(a.m + kOffLat);
+    float4 *__restrict__ V = reinterpret_cast<float4 *>(a.v + kOffLat);
+    longlong2 *__restrict__ G = reinterpret_cast<longlong2 *>(a.grad + kOffLat);
+    const size_t nq = (a.n - kOffLat) / 4, stride = (size_t)gridDim.x * kUpThreads;
+    const size_t t0 = blockIdx.x * (size_t)kUpThreads + threadIdx.x;
     const longlong2 z = make_longlong2(0, 0);
-    for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < n4; q += 2 * stride) {
-        const size_t q2 = q + stride;
-        const bool two = q2 < n4;
-        const bool gq = quad_has_grad(a, q), gq2 = two && quad_has_grad(a, q2);
-        const longlong2 g0 = gq ? G[2 * q] : z, g1 = gq ? G[2 * q + 1] : z;
-        float4 p = P[q], m = M[q], v = V[q];
-        longlong2 h0 = z, h1 = z;
-        float4 p2 = make_float4(0.f, 0.f, 0.f, 0.f), m2 = p2, v2 = p2;
-        if (two) {
-            if (gq2) {
-                h0 = G[2 * q2];
-                h1 = G[2 * q2 + 1];
-            }
-            p2 = P[q2];
-            m2 = M[q2];
-            v2 = V[q2];
+    float4 p[kUpQuads], m[kUpQuads], v[kUpQuads];
+    auto quad_at = [&](size_t i) {  // (past the end: the last quad again, not stored)
+        const size_t c = min(i, nq - 1);
+        return a.descending ? nq - 1 - c : c;
+    };
+    auto load = [&](size_t i) {
+#pragma unroll
+        for (int k = 0; k < kUpQuads; ++k) {
+            const size_t q = quad_at(i + k * stride);
+            p[k] = P[q];
+            m[k] = M[q];
+            v[k] = V[q];
         }
-        adam_quad(a, q < (size_t)kWeights / 4 ? a.step_w : a.step_lat, p, m, v, g0, g1);
-        if (gq) {
-            G[2 * q] = z;
-            G[2 * q + 1] = z;
-        }
-        P[q] = p;
-        M[q] = m;
-        V[q] = v;
-        if (two) {
-            adam_quad(a, q2 < (size_t)kWeights / 4 ? a.step_w : a.step_lat, p2, m2, v2, h0, h1);
-            if (gq2) {
-                G[2 * q2] = z;
-                G[2 * q2 + 1] = z;
+    };
+    load(t0);
+    for (size_t w = t0; w < a.words; w += stride) a.touched_next[w] = 0u;
+    // (the weights' own values too, for the CTAs that have some)
+    const int w0 = blockIdx.x * kRedEntries + threadIdx.x;
+    const bool own = threadIdx.x < kRedEntries && w0 < kWeights;
+    const int wp = own ? slot_param(w0) : 0;
+    float w_p = a.params[wp], w_m = a.m[wp], w_v = a.v[wp];
+
+    grid_wait();  // the gradients
+
+    // ---- the weights: 16 slots per CTA and turn (see reduce_kernel)
+    for (int b = blockIdx.x; b * kRedEntries < kWeights; b += gridDim.x) {
+        const int e = b * kRedEntries + (threadIdx.x % kRedEntries), row = threadIdx.x / kRedEntries;
+        part[row][threadIdx.x % kRedEntries] = e < kWeights ? partial_sum(a.partial, a.ctas, e, row) : 0.0;
+        __syncthreads();
+        if (row == 0 && e < kWeights) {
+            double tot = 0.0;
+            for (int r = 0; r < kRedRows; ++r) tot += part[r][threadIdx.x];
+            const int w = slot_param(e);
+            if (b != (int)blockIdx.x) {
+                w_p = a.params[w];
+                w_m = a.m[w];
+                w_v = a.v[w];
             }
-            P[q2] = p2;
-            M[q2] = m2;
-            V[q2] = v2;
+            adam_update(a, __double2ll_rn(tot * a.dscale * kFix), a.step_w, w_p, w_m, w_v);
+            a.params[w] = w_p;
+            a.m[w] = w_m;
+            a.v[w] = w_v;
+            put_weight(a.wimg, w, w_p);
+        }
+        __syncthreads();
+    }
+
+    // ---- the latents, kUpQuads quads (half a cell each) per iteration, whose
+    // loads are in flight together; the marks are read one iteration ahead, so
+    // that the gradients of the marked cells are too
+    uint32_t mark[kUpQuads];
+    auto load_marks = [&](size_t i) {
+#pragma unroll
+        for (int k = 0; k < kUpQuads; ++k) {
+            const size_t q = quad_at(i + k * stride);
+            mark[k] = (__ldg(a.touched + (q >> 6)) >> ((q >> 1) & 31)) & 1u;
+        }
+    };
+    load_marks(t0);
+    for (size_t i = t0; i < nq; i += kUpQuads * stride) {
+        longlong2 g0[kUpQuads], g1[kUpQuads];
+#pragma unroll
+        for (int k = 0; k < kUpQuads; ++k) {
+            const size_t q = quad_at(i + k * stride);
+            g0[k] = mark[k] ? G[2 * q] : z;
+            g1[k] = mark[k] ? G[2 * q + 1] : z;
+        }
+        if (i != t0) load(i);
+        uint32_t had = 0;
+#pragma unroll
+        for (int k = 0; k < kUpQuads; ++k) had |= mark[k] << k;
+        load_marks(i + kUpQuads * stride);
+#pragma unroll
+        for (int k = 0; k < kUpQuads; ++k) {
+            if (i + k * stride >= nq) break;
+            const size_t q = quad_at(i + k * stride);
+            adam_quad(a, a.step_lat, p[k], m[k], v[k], g0[k], g1[k]);
+            if ((had >> k) & 1u) {
+                G[2 * q] = z;
+                G[2 * q + 1] = z;
+            }
+            P[q] = p[k];
+            M[q] = m[k];
+            V[q] = v[k];
         }
     }
 }
@@ -799,7 +947,7 @@ struct ctf_trainer_s {
     size_t nparams = 0;
     float *params = nullptr, *m = nullptr, *v = nullptr;
     long long *grad = nullptr, *loss = nullptr;
-    uint32_t *touched = nullptr;  // latent cells a step's texels reached (zero between steps)
+    uint32_t *touched = nullptr;  // latent cells that a step's texels reached: two bitmaps, even and odd steps
     unsigned char *wimg = nullptr;  // FP16 weight operands of the gradient kernel
     float *partial = nullptr;       // per-CTA weight-gradient sums of the gradient kernel
     size_t touched_words = 0;
@@ -840,7 +988,40 @@ GradParams grad_params(const ctf_trainer_s *t) {
     return g;
 }
 
-cudaError_t launch_grad(const GradParams &g, cudaStream_t s) {
+// A launch that may begin while the kernel before it in the stream ends (that
+// kernel triggers it early, or not at all); it waits with grid_wait.
+template <typename... Params, typename... Args>
+cudaError_t launch_dependent(void (*fn)(Params...), int grid, int threads, size_t smem, cudaStream_t s, Args... args) {
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, fn, args...);
+}
+
+// The split of a batch over the gradient kernel's CTAs.  Two CTAs fit on an
+// SM (TMEM and shared memory).  Small batches take 64 texels per round (the
+// other 64 rows of the MMAs stay empty) so that more SMs have work; a CTA's
+// fixed costs (weights in, sums out) favour a few rounds each once there are
+// 256 CTAs, and at most kMaxGradCtas CTAs hold partial sums.  The split
+// depends on the batch alone, so a step gives the same sums on any device.
+int split_batch(GradParams &g) {
+    g.per_round = g.n >= 32768 ? kT : kT / 2;
+    int rounds = g.n / (g.per_round * 256);
+    rounds = rounds < 1 ? 1 : (rounds > kMaxRounds ? kMaxRounds : rounds);
+    const int need = (g.n + g.per_round * kMaxGradCtas - 1) / (g.per_round * kMaxGradCtas);
+    g.rounds = rounds > need ? rounds : need;
+    return (g.n + g.per_round * g.rounds - 1) / (g.per_round * g.rounds);
+}
+
+// The gradient kernel, after a kernel that left the weight image.
+cudaError_t launch_grad(const GradParams &g, int ctas, cudaStream_t s) {
     static std::mutex mu;
     static bool attr[64] = {};
     int dev = 0;
@@ -854,28 +1035,11 @@ cudaError_t launch_grad(const GradParams &g, cudaStream_t s) {
             attr[dev] = true;
         }
     }
-    // Two CTAs fit on an SM (TMEM and shared memory).  Small batches take 64
-    // texels per round (the other 64 rows of the MMAs stay empty) so that
-    // more SMs have work; a CTA's fixed costs (weights in, sums out) favour a
-    // few rounds each once there are 256 CTAs, and at most kMaxGradCtas CTAs
-    // hold partial sums.  The split depends on the batch alone, so a step
-    // gives the same sums on any device.
-    GradParams gp = g;
-    gp.per_round = g.n >= 32768 ? kT : kT / 2;
-    int rounds = g.n / (gp.per_round * 256);
-    rounds = rounds < 1 ? 1 : (rounds > kMaxRounds ? kMaxRounds : rounds);
-    const int need = (g.n + gp.per_round * kMaxGradCtas - 1) / (gp.per_round * kMaxGradCtas);
-    gp.rounds = rounds > need ? rounds : need;
-    const int ctas = (g.n + gp.per_round * gp.rounds - 1) / (gp.per_round * gp.rounds);
-    if (ctas == 0) return cudaSuccess;
+    return launch_dependent(grad_kernel, ctas, kT, kGradSmem, s, g);
+}
+
+cudaError_t launch_pack(const GradParams &g, cudaStream_t s) {
     pack_kernel<<<(kPackThreads + 255) / 256, 256, 0, s>>>(g.params, g.wimg);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    grad_kernel<<<ctas, kT, kGradSmem, s>>>(gp);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    reduce_kernel<<<(kWeights + kRedEntries - 1) / kRedEntries, kRedEntries * kRedRows, 0, s>>>(
-        g.partial, ctas, (double)g.dscale, g.grad);
     return cudaGetLastError();
 }
 
@@ -919,8 +1083,7 @@ int alloc_trainer(ctf_texture src, const ctf_train_desc *d, ctf_trainer_s **out)
     t->nparams = kOffLat + t->n_lat[0] + t->n_lat[1];
     t->touched_words = ((t->n_lat[0] + t->n_lat[1]) / 8 + 31) / 32;
     cudaError_t e = ctf::dev_malloc(&t->params, t->nparams * 4);
-    if (e == cudaSuccess) e = ctf::dev_malloc(&t->touched, t->touched_words * 4);
-    if (e == cudaSuccess) e = cudaMemset(t->touched, 0, t->touched_words * 4);
+    if (e == cudaSuccess) e = ctf::dev_malloc(&t->touched, 2 * t->touched_words * 4);
     if (e == cudaSuccess) e = ctf::dev_malloc(&t->m, t->nparams * 4);
     if (e == cudaSuccess) e = ctf::dev_malloc(&t->v, t->nparams * 4);
     if (e == cudaSuccess) e = ctf::dev_malloc(&t->grad, t->nparams * 8);
@@ -1008,21 +1171,32 @@ int ctf_trainer_step(ctf_trainer t, int64_t steps, void *stream) {
     GradParams g = grad_params(t);
     g.n = t->desc.batch;
     g.dscale = 2.0f / (float)t->desc.batch;
+    const int ctas = split_batch(g);
     AdamParams a;
     a.params = t->params;
     a.m = t->m;
     a.v = t->v;
     a.grad = t->grad;
-    a.touched = t->touched;
     a.n = t->nparams;
     a.beta1 = t->desc.beta1;
     a.beta2 = t->desc.beta2;
     a.eps = t->desc.eps;
+    a.words = t->touched_words;
+    a.partial = t->partial;
+    a.ctas = ctas;
+    a.dscale = (double)g.dscale;
+    a.wimg = t->wimg;
+    auto bitmap = [&](int64_t st) { return t->touched + (size_t)(st & 1) * t->touched_words; };
+    if (steps > 0) {
+        cudaError_t e = cudaMemsetAsync(t->touched, 0, 2 * t->touched_words * 4, s);
+        if (e == cudaSuccess) e = launch_pack(g, s);
+        if (e != cudaSuccess) return report_cuda(e, "training step");
+    }
     for (int64_t k = 0; k < steps; ++k) {
         const int64_t st = t->step;
         g.step = (uint32_t)st;
-        cudaError_t e = cudaMemsetAsync(t->loss, 0, 8, s);
-        if (e == cudaSuccess) e = launch_grad(g, s);
+        g.touched = bitmap(st);
+        cudaError_t e = launch_grad(g, ctas, s);
         const double frac = std::fmin(1.0, (double)st / (double)t->desc.total_steps);
         const double sched = 1.0 - (1.0 - t->desc.lr_final_frac) * frac;
         const double bc1 = 1.0 - std::pow((double)t->desc.beta1, (double)(st + 1));
@@ -1030,11 +1204,11 @@ int ctf_trainer_step(ctf_trainer t, int64_t steps, void *stream) {
         a.step_w = (float)(t->desc.lr_weights * sched / bc1);
         a.step_lat = (float)(t->desc.lr_latents * sched / bc1);
         a.inv_bc2 = (float)(1.0 / bc2);
-        if (e == cudaSuccess) {
-            adam_kernel<<<device_sm_count() * 8, 256, 0, s>>>(a);
-            e = cudaGetLastError();
-        }
-        if (e == cudaSuccess) e = cudaMemsetAsync(t->touched, 0, t->touched_words * 4, s);
+        a.touched = bitmap(st);
+        a.touched_next = bitmap(st + 1);
+        a.descending = (int)(st & 1);
+        if (e == cudaSuccess)
+            e = launch_dependent(update_kernel, device_sm_count() * kUpCtasPerSm, kUpThreads, 0, s, a);
         if (e != cudaSuccess) return report_cuda(e, "training step");
         t->step = st + 1;
     }
@@ -1053,8 +1227,15 @@ int ctf_trainer_gradients(ctf_trainer t, const int32_t *xy, int n, double *loss,
     g.n = n;
     g.dscale = 2.0f / (float)n;
     // the accumulators are zero between steps; use them and clear them again
+    const int ctas = split_batch(g);
     cudaError_t e = cudaMemsetAsync(t->loss, 0, 8, s);
-    if (e == cudaSuccess) e = launch_grad(g, s);
+    if (e == cudaSuccess) e = launch_pack(g, s);
+    if (e == cudaSuccess) e = launch_grad(g, ctas, s);
+    if (e == cudaSuccess) {
+        reduce_kernel<<<(kWeights + kRedEntries - 1) / kRedEntries, kRedEntries * kRedRows, 0, s>>>(
+            g.partial, ctas, (double)g.dscale, g.grad);
+        e = cudaGetLastError();
+    }
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return report_cuda(e, "gradient kernel");
     std::vector<long long> h(t->nparams);
@@ -1062,7 +1243,6 @@ int ctf_trainer_gradients(ctf_trainer t, const int32_t *xy, int n, double *loss,
     e = cudaMemcpy(h.data(), t->grad, t->nparams * 8, cudaMemcpyDeviceToHost);
     if (e == cudaSuccess) e = cudaMemcpy(&hl, t->loss, 8, cudaMemcpyDeviceToHost);
     if (e == cudaSuccess) e = cudaMemset(t->grad, 0, t->nparams * 8);
-    if (e == cudaSuccess) e = cudaMemset(t->touched, 0, t->touched_words * 4);
     if (e != cudaSuccess) return report_cuda(e, "reading gradients");
     if (loss) *loss = (double)hl / kLossFix / (double)n;
     if (grads) {
