@@ -97,8 +97,14 @@ __global__ void __launch_bounds__(kBlockWarps * 32, batch_min_blocks<ALG>()) bat
     __shared__ unsigned long long block_stats[kNumStats];
     __shared__ int s_begin[kSmViews];
     __shared__ __align__(16) ExactParams s_params[kBlockWarps];  // each warp's current view
-    load_decode_tables(&tabs, b.tables);
+    {
+        DecodeTableLoad<kBlockWarps * 32> tl;
+        tl.load(b.tables);
+        tl.store(&tabs);
+    }
     if (threadIdx.x < kNumStats) block_stats[threadIdx.x] = 0;
+    grid_wait();  // (the plan's arrays too)
+    grid_trigger();
     const bool cached = b.nkind <= kSmViews && b.total_items < 0x7fffffffLL;
     if (cached)
         for (int i = threadIdx.x; i < b.nkind; i += blockDim.x) s_begin[i] = (int)__ldg(b.item_begin + i);
@@ -524,6 +530,8 @@ cudaError_t launch_plan(const Plan &plan, const DevPlan &dp, int alg, const Reso
             const long long useful = (plan.items[k] + r.items_per_fetch - 1) / r.items_per_fetch;
             if (grid > useful) grid = useful;
             fn<<<(int)grid, kRows, kSmRequest, s>>>(b);
+            e = cudaGetLastError();
+            if (e != cudaSuccess) return e;
         } else {
             int per_sm = 0;
             if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kBlockWarps * 32, 0) != cudaSuccess ||
@@ -532,10 +540,9 @@ cudaError_t launch_plan(const Plan &plan, const DevPlan &dp, int alg, const Reso
             long long grid = (long long)device_sm_count() * per_sm;
             const long long useful = (plan.items[k] + kBlockWarps - 1) / kBlockWarps;
             if (grid > useful) grid = useful;
-            fn<<<(int)grid, kBlockWarps * 32, 0, s>>>(b);
+            e = launch_dependent(fn, (int)grid, kBlockWarps * 32, 0, s, b);
+            if (e != cudaSuccess) return e;
         }
-        e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
 }

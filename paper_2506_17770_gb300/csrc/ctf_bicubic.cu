@@ -118,8 +118,14 @@ __global__ void __launch_bounds__(kThreads) bicubic_filter_kernel(const ExactPar
 
     if (threadIdx.x < kNumStats) block_stats[threadIdx.x] = 0;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    load_decode_tables(&tabs, p.tables);
+    {
+        DecodeTableLoad<kThreads> tl;
+        tl.load(p.tables);
+        tl.store(&tabs);
+    }
     __syncthreads();
+    grid_wait();
+    grid_trigger();
     int *ranks = rank_slots[warp];
     const int tx = lane % TW, ty = lane / TW;
     const uint32_t lt = lanemask_lt();
@@ -399,8 +405,7 @@ cudaError_t launch_bicubic_filter(const ExactParams &p, int alg, int tile_w, int
     const long long want = (p.n_tiles + kWarps - 1) / kWarps;
     const long long cap = (long long)device_sm_count() * per_sm;
     const int grid = (int)(want < cap ? want : cap);
-    fn<<<grid, kThreads, 0, stream>>>(p);
-    return cudaGetLastError();
+    return launch_dependent(fn, grid, kThreads, 0, stream, p);
 }
 
 }  // namespace ctf

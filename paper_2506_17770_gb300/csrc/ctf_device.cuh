@@ -144,6 +144,15 @@ __device__ __forceinline__ void bilinear_weights(float s, float t, float w[4]) {
 // h(i, A) for a 32-bit lane mask: lane of the i-th set bit.
 __device__ __forceinline__ int nth_set_lane(uint32_t A, int i) { return (int)__fns(A, 0, i + 1); }
 
+// Programmatic dependent launch (launch_dependent, ctf_internal.h).
+// grid_wait: wait until the kernels before this one in the stream are done
+// and their writes visible (at once when it was launched without the
+// attribute); every CTA calls it, so that a kernel never ends before the ones
+// before it.  grid_trigger: the next such kernel may start; called after
+// grid_wait, so that at most one kernel waits beside a running one.
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 __device__ __forceinline__ uint32_t lanemask_lt() {
     uint32_t m;
     asm("mov.u32 %0, %%lanemask_lt;" : "=r"(m));

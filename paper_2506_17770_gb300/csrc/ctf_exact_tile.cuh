@@ -40,14 +40,24 @@ __device__ __forceinline__ void store_pixel(const ExactParams &p, uint32_t idx, 
     if (p.evals) p.evals[idx] = count;
 }
 
-// The decode tables (DecodeTables, ctf_internal.h) into this CTA's shared
-// memory, 16 bytes per thread and step; the interpolated palette entries
-// carry the offset 256 in every field of the sum.
-__device__ __forceinline__ void load_decode_tables(DecodeTables *t, const DecodeTables *g) {
-    const uint4 *src = reinterpret_cast<const uint4 *>(g);
-    uint4 *dst = reinterpret_cast<uint4 *>(t);
-    for (int i = threadIdx.x; i < (int)(sizeof(DecodeTables) / 16); i += blockDim.x) dst[i] = __ldg(src + i);
-}
+// The decode tables (DecodeTables, ctf_internal.h) into the shared memory of
+// a CTA of kThr threads, in two halves (other loads go between); the
+// interpolated palette entries carry the offset 256 in every field of the sum.
+template <int kThr>
+struct DecodeTableLoad {
+    static constexpr int kN = (int)(sizeof(DecodeTables) / 16), kPer = (kN + kThr - 1) / kThr;
+    uint4 v[kPer];
+    __device__ __forceinline__ void load(const DecodeTables *g) {
+#pragma unroll
+        for (int k = 0; k < kPer; ++k)
+            v[k] = __ldg(reinterpret_cast<const uint4 *>(g) + min((int)threadIdx.x + k * kThr, kN - 1));
+    }
+    __device__ __forceinline__ void store(DecodeTables *t) const {
+#pragma unroll
+        for (int k = 0; k < kPer; ++k)
+            if ((int)threadIdx.x + k * kThr < kN) reinterpret_cast<uint4 *>(t)[threadIdx.x + k * kThr] = v[k];
+    }
+};
 
 // RGB of texel (x, y) of a block (alpha is 1): palette c0, c1,
 // (2c0+c1+1)/3, (c0+2c1+1)/3, 2-bit index at bits 2*(4*(y&3)+(x&3)).

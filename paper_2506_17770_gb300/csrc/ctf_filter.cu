@@ -71,9 +71,14 @@ __global__ void __launch_bounds__(kThreads, kExt ? 4 : min_blocks<ALG>()) exact_
 
     bool inside = n_mine > 0 && bx < lim_x && by < lim_y;
     uint32_t idx = by * (TH * W) + bx * TW + lane_off;
+    // the decode tables are requested before the kernels before this one are
+    // done, and stored while the first tile's inputs are in flight
+    DecodeTableLoad<kThreads> tl;
+    tl.load(p.tables);
+    grid_wait();
+    grid_trigger();
     Inputs cur = load_inputs_any<kJac>(p, inside, idx);
-    // the decode tables come in while the first tile's inputs are in flight
-    load_decode_tables(&tabs, p.tables);
+    tl.store(&tabs);
     __syncthreads();
 
     for (uint32_t i = 0; i < n_mine; ++i) {
@@ -183,8 +188,7 @@ cudaError_t launch_exact_filter(const ExactParams &p, int alg, int tile_w, int m
     const long long want = (p.n_tiles + kWarps - 1) / kWarps;
     const long long cap = (long long)device_sm_count() * per_sm;
     const int grid = (int)(want < cap ? want : cap);
-    fn<<<grid, kThreads, 0, stream>>>(p);
-    return cudaGetLastError();
+    return launch_dependent(fn, grid, kThreads, 0, stream, p);
 }
 
 }  // namespace ctf

@@ -142,6 +142,9 @@ __global__ void __launch_bounds__(kPThreads, kPCtasPerSm)
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
+    // (as in the packed-group kernel)
+    grid_wait();
+    grid_trigger();
     const uint32_t tmem = *tslot;
     Counters cnt;
 #pragma unroll
@@ -331,8 +334,7 @@ cudaError_t dense_launch(const DenseArgs &a, const MlpDevice &m, const MlpEpilog
     cudaError_t e = dense_prepare(fn);
     if (e != cudaSuccess) return e;
     const long long cap = (long long)device_sm_count() * kPCtasPerSm;
-    fn<<<(int)(groups < cap ? groups : cap), kPThreads, kDBytes, stream>>>(a, m, ep);
-    return cudaGetLastError();
+    return launch_dependent(fn, (int)(groups < cap ? groups : cap), kPThreads, kDBytes, stream, a, m, ep);
 }
 
 }  // namespace

@@ -76,8 +76,7 @@ cudaError_t launch_mlp_filter_pf(const ExactParams &p, const MlpDevice &m, const
     const long long groups = (p.n_tiles + k->tiles[var] - 1) / k->tiles[var];
     const long long cap = (long long)device_sm_count() * k->ctas_per_sm;
     const int grid = (int)(groups < cap ? groups : cap);
-    fn<<<grid, k->threads, k->smem[var], stream>>>(p, m, ep, err);
-    return cudaGetLastError();
+    return launch_dependent(fn, grid, k->threads, k->smem[var], stream, p, m, ep, err);
 }
 
 int mlp_batch_pf_tiles() { return kernels_of(8)->tiles[kPfPlain]; }
@@ -118,8 +117,7 @@ cudaError_t launch_mlp_batch_pf(const BatchViewDev *views, int nviews, const int
     b.err = err;
     const long long cap = (long long)device_sm_count() * k->ctas_per_sm;
     const int grid = (int)(total_items < cap ? total_items : cap);
-    fn<<<grid, k->threads, k->batch_smem, s>>>(b, m0, ep0);
-    return cudaGetLastError();
+    return launch_dependent(fn, grid, k->threads, k->batch_smem, s, b, m0, ep0);
 }
 
 }  // namespace ctf

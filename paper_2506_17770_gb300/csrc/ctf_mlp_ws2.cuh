@@ -550,6 +550,10 @@ __global__ void __launch_bounds__(kPThreads, kPCtasPerSm)
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
+    // what comes before overlaps the end of the kernel before this one; the
+    // next kernel starts when this one has its TMEM
+    grid_wait();
+    grid_trigger();
     const uint32_t tmem = *tslot;
     const float *inv_a1 = reinterpret_cast<const float *>(sm + kImgA1);
     Counters cnt;
@@ -781,6 +785,10 @@ __global__ void __launch_bounds__(kPThreads, kPCtasPerSm)
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
+    // what comes before overlaps the end of the kernel before this one; the
+    // next kernel starts when this one has its TMEM
+    grid_wait();
+    grid_trigger();
     const uint32_t tmem = *tslot;
     Counters cnt;
 #pragma unroll

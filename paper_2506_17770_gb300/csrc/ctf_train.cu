@@ -202,12 +202,6 @@ __device__ __forceinline__ void bilinear_taps(const GradParams &g, int grid, int
 }
 
 
-// Programmatic dependent launch: wait for the kernels before this one in the
-// stream (at once when it was launched without the attribute), and let the
-// one after it start.
-__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void grid_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-
 // Texel i of the step's batch.
 __device__ __forceinline__ void sample_texel(const GradParams &g, uint32_t i, int &x, int &y) {
     const uint4 rr = philox4x32_10(make_uint4(i, g.step, 0x5A4Du, 0u), g.k0, g.k1);
@@ -986,23 +980,6 @@ GradParams grad_params(const ctf_trainer_s *t) {
     g.err = nullptr;
     device_error_word(&g.err);  // a static device word: no allocation; nullptr if it cannot be had
     return g;
-}
-
-// A launch that may begin while the kernel before it in the stream ends (that
-// kernel triggers it early, or not at all); it waits with grid_wait.
-template <typename... Params, typename... Args>
-cudaError_t launch_dependent(void (*fn)(Params...), int grid, int threads, size_t smem, cudaStream_t s, Args... args) {
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3((unsigned)threads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, fn, args...);
 }
 
 // The split of a batch over the gradient kernel's CTAs.  Two CTAs fit on an
