@@ -23,7 +23,7 @@
 // (ctf_mlp_chain.cuh, mlp_group; the persistent batch kernel runs the same
 // for every algorithm with group_dedup).  Everything else runs in kernels
 // whose warps are specialised by role, which give the same outputs:
-// ctf_mlp_ws2.cuh (STF, List Merge, Box and Mask Sampling), ctf_mlp_ws.cu (STF,
+// ctf_mlp_ws2.cu (STF, List Merge, Box and Mask Sampling), ctf_mlp_ws.cu (STF,
 // Box and Mask with group_dedup), ctf_mlp_ext.cu (combined extensions) and
 // ctf_mlp_dense.cu (per-pixel 4-tap, decode of a list).
 #include <cstdint>

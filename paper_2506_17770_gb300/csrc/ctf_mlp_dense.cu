@@ -3,7 +3,7 @@
 // decode of an explicit list of texels.
 //
 // The roles and the chain are those of the packed-group kernel
-// (ctf_mlp_ws2.cuh): per CTA (four per SM) one consumer warpgroup runs the
+// (ctf_mlp_ws2.cu): per CTA (four per SM) one consumer warpgroup runs the
 // tcgen05 MLP chains over 128-row tiles, and four producer warps compute the
 // features straight into the layer-1 operand of a stage of 256 rows, four
 // stages in rotation.  Every row is used, so a stage is exactly two chains.
@@ -25,7 +25,8 @@
 #include <set>
 #include <utility>
 
-#include "ctf_mlp_ws2.cuh"
+#define CTF_MLP_WS2_PART
+#include "ctf_mlp_ws2.cu"
 
 namespace ctf {
 namespace {

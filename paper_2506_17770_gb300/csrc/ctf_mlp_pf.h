@@ -1,6 +1,6 @@
 // ctf_mlp_pf.h -- the host's view of the packed-group kernels of
-// ctf_mlp_ws2.cuh, which are compiled in one file per tile width
-// (ctf_mlp_ws2_w8.cu, _w4.cu, _w16.cu) and launched from ctf_mlp_ws2.cu.
+// ctf_mlp_ws2.cu, which are compiled in one unit per tile width
+// (ctf_mlp_ws2.cu itself, _w4.cu, _w16.cu) and launched from ctf_mlp_pf.cu.
 #pragma once
 #include <cuda_runtime.h>
 

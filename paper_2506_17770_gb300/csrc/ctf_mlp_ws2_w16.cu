@@ -1,6 +1,7 @@
-// ctf_mlp_ws2_w16.cu -- the packed-group learned kernels (ctf_mlp_ws2.cuh)
+// ctf_mlp_ws2_w16.cu -- the packed-group learned kernels (ctf_mlp_ws2.cu)
 // for warp tiles 16 pixels wide.
-#include "ctf_mlp_ws2.cuh"
+#define CTF_MLP_WS2_PART
+#include "ctf_mlp_ws2.cu"
 
 namespace ctf {
 PfKernels pf_kernels_w16() { return pf_kernels<16>(); }
