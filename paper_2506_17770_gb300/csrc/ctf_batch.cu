@@ -533,11 +533,8 @@ cudaError_t launch_plan(const Plan &plan, const DevPlan &dp, int alg, const Reso
             e = cudaGetLastError();
             if (e != cudaSuccess) return e;
         } else {
-            int per_sm = 0;
-            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kBlockWarps * 32, 0) != cudaSuccess ||
-                per_sm < 1)
-                per_sm = 1;
-            long long grid = (long long)device_sm_count() * per_sm;
+            long long grid =
+                (long long)device_sm_count() * resident_ctas(reinterpret_cast<const void *>(fn), kBlockWarps * 32);
             const long long useful = (plan.items[k] + kBlockWarps - 1) / kBlockWarps;
             if (grid > useful) grid = useful;
             e = launch_dependent(fn, (int)grid, kBlockWarps * 32, 0, s, b);

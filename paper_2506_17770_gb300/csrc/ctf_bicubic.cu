@@ -430,11 +430,8 @@ cudaError_t launch_bicubic_filter(const ExactParams &p, int alg, int tile_w, int
     if (!fn) return cudaErrorInvalidValue;
     if (p.n_tiles == 0) return cudaSuccess;
     if (p.n_tiles > 0x7fffffffLL) return cudaErrorInvalidValue;
-    int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kThreads, 0) != cudaSuccess || per_sm < 1)
-        per_sm = 1;
     const long long want = (p.n_tiles + kWarps - 1) / kWarps;
-    const long long cap = (long long)device_sm_count() * per_sm;
+    const long long cap = (long long)device_sm_count() * resident_ctas(reinterpret_cast<const void *>(fn), kThreads);
     const int grid = (int)(want < cap ? want : cap);
     return launch_dependent(fn, grid, kThreads, 0, stream, p);
 }

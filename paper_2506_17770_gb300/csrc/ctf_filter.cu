@@ -22,6 +22,7 @@
 // box raster order and the mask bit order).
 #include <climits>
 #include <cstdint>
+#include <mutex>
 #include <cuda_runtime.h>
 
 #include "ctf_device.cuh"
@@ -169,6 +170,28 @@ int device_sm_count() {
     return cached;
 }
 
+// The answer for a kernel and device does not change, and asking the runtime
+// for it took 0.2 us of a call: kept in a bounded table (asked again for
+// kernels past its end).
+int resident_ctas(const void *fn, int threads) {
+    struct Entry {
+        const void *fn;
+        int dev, threads, ctas;
+    };
+    static Entry table[256];
+    static int used = 0;
+    static std::mutex mu;
+    int dev = 0;
+    cudaGetDevice(&dev);
+    std::lock_guard<std::mutex> lk(mu);
+    for (int i = 0; i < used; ++i)
+        if (table[i].fn == fn && table[i].dev == dev && table[i].threads == threads) return table[i].ctas;
+    int ctas = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctas, fn, threads, 0) != cudaSuccess || ctas < 1) return 1;
+    if (used < 256) table[used++] = Entry{fn, dev, threads, ctas};
+    return ctas;
+}
+
 cudaError_t launch_exact_filter(const ExactParams &p, int alg, int tile_w, int mask_dim, cudaStream_t stream) {
     KernelFn fn = nullptr;
     const bool st = p.stats != nullptr;
@@ -182,11 +205,8 @@ cudaError_t launch_exact_filter(const ExactParams &p, int alg, int tile_w, int m
     if (!fn) return cudaErrorInvalidValue;
     if (p.n_tiles == 0) return cudaSuccess;
     if (p.n_tiles > 0x7fffffffLL) return cudaErrorInvalidValue;
-    int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kThreads, 0) != cudaSuccess || per_sm < 1)
-        per_sm = 1;
     const long long want = (p.n_tiles + kWarps - 1) / kWarps;
-    const long long cap = (long long)device_sm_count() * per_sm;
+    const long long cap = (long long)device_sm_count() * resident_ctas(reinterpret_cast<const void *>(fn), kThreads);
     const int grid = (int)(want < cap ? want : cap);
     return launch_dependent(fn, grid, kThreads, 0, stream, p);
 }

@@ -111,6 +111,8 @@ cudaError_t launch_bicubic_filter(const ExactParams &p, int alg, int tile_w, int
 
 // Number of SMs of the current device (cached).
 int device_sm_count();
+// CTAs of `fn` (no dynamic shared memory) that fit on an SM of the current device, at least 1.
+int resident_ctas(const void *fn, int threads);
 
 // The current device's decode tables (made once per device; nullptr and a
 // recorded error if that failed).
