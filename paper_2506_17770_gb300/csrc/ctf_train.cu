@@ -11,9 +11,11 @@
 // products, the input-side gradients and the weight gradients, which it
 // sums over its rounds in TMEM and leaves as the CTA's partial sums; the
 // latent-grid gradients go to 64-bit fixed-point accumulators (integer
-// atomics are order-independent, so a step is deterministic).  An update
-// kernel adds the partial sums up, applies Adam to every parameter and clears
-// the accumulators it has read.
+// atomics are order-independent, so a step is deterministic).  A second kernel
+// adds the partial sums up and applies Adam to the weights and to the latent
+// cells that the next step reads; at the end of a segment of steps all other
+// cells take the steps they have missed (advance_kernel, sweep_kernel).
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 #include <cstdio>
@@ -57,7 +59,8 @@ struct GradParams {
     uint32_t k0, k1;       // Philox key
     float dscale;          // 2 / batch
     long long *grad;       // fixed-point gradient accumulators (same layout as params)
-    uint32_t *touched;     // one bit per latent cell (grid 0 cells, then grid 1) whose gradient a texel reached
+    uint32_t *seen;        // per latent cell (grid 0, then grid 1): see advance_kernel
+    uint32_t mark;         // the first step of a segment: the value its cells get there, else 0
     long long *loss;       // fixed-point sum of squared errors
     int *err;              // device error word: a wait that gave up records CTF_ERR_TIMEOUT
     unsigned char *wimg;   // the weight image of the gradient kernel (pack_kernel)
@@ -203,8 +206,8 @@ __device__ __forceinline__ void bilinear_taps(const GradParams &g, int grid, int
 
 
 // Texel i of the step's batch.
-__device__ __forceinline__ void sample_texel(const GradParams &g, uint32_t i, int &x, int &y) {
-    const uint4 rr = philox4x32_10(make_uint4(i, g.step, 0x5A4Du, 0u), g.k0, g.k1);
+__device__ __forceinline__ void sample_texel(const GradParams &g, uint32_t step, uint32_t i, int &x, int &y) {
+    const uint4 rr = philox4x32_10(make_uint4(i, step, 0x5A4Du, 0u), g.k0, g.k1);
     x = (int)(((unsigned long long)rr.x * (unsigned)g.Wt) >> 32);
     y = (int)(((unsigned long long)rr.y * (unsigned)g.Ht) >> 32);
 }
@@ -359,7 +362,7 @@ __global__ void __launch_bounds__(kT, 2) grad_kernel(const GradParams g) {
             x = min(max(c.x, 0), g.Wt - 1);
             y = min(max(c.y, 0), g.Ht - 1);
         } else {
-            sample_texel(g, (uint32_t)i, x, y);
+            sample_texel(g, g.step, (uint32_t)i, x, y);
         }
         const uint32_t px = fetch_block_texel(g.blocks, g.nbx, g.Wt, g.Ht, x, y, g.err);
 #pragma unroll
@@ -575,14 +578,14 @@ __global__ void __launch_bounds__(kT, 2) grad_kernel(const GradParams g) {
             const int n = __popc(__ballot_sync(FULL, there));  // (the warp's texels are its first n rows)
             for (int gi = g_lo; gi < g_hi; ++gi) {
                 unsigned long long *gl = reinterpret_cast<unsigned long long *>(g.grad + kOffLat + (gi ? lat1 : 0)) + ch;
-                const uint32_t bit0 = gi ? (uint32_t)(lat1 / 8) : 0u;
+                const uint32_t cell0 = gi ? (uint32_t)(lat1 / 8) : 0u;
 #pragma unroll 4
                 for (int t = 0; t < n; ++t) {
                     const unsigned char *rec = DH + kDHTaps + 32 * (2 * (row0 + t) + gi) + 4 * k;
                     const int cell = *reinterpret_cast<const int *>(rec);
                     const float w = *reinterpret_cast<const float *>(rec + 16);
                     const float df = *reinterpret_cast<const float *>(DH + 64 * (row0 + t) + 32 * gi + 4 * ch);
-                    if (ch == 0) atomicOr(g.touched + ((bit0 + (uint32_t)cell) >> 5), 1u << ((bit0 + (uint32_t)cell) & 31u));
+                    if (g.mark && ch == 0) atomicMax(g.seen + cell0 + cell, g.mark);
                     const long long v = to_fix(__fmul_rn(w, df));
                     if (v) atomicAdd(gl + (size_t)cell * 8, (unsigned long long)v);
                 }
@@ -673,21 +676,30 @@ __global__ void __launch_bounds__(kRedEntries * kRedRows) reduce_kernel(const fl
     }
 }
 
+// Steps of a segment at most (see advance_kernel): 4096^2 texture, 8,192
+// texels, 64 steps 2.72 ms with 8, 2.61 with 16, 2.59 with 32, 2.82 with 64.
+constexpr int kSegment = 16;
+
+// What a step multiplies: the learning rate over the first bias correction
+// (weights, latents) and 1 / (1 - beta2^t).
+struct AdamStep {
+    float w, lat, inv_bc2;
+};
+
 struct AdamParams {
     float *params, *m, *v;
     long long *grad;
     size_t n;
     float beta1, beta2, eps;
-    float step_w, step_lat;  // learning rate / (1 - beta1^t), weights and latents
-    float inv_bc2;           // 1 / (1 - beta2^t)
-    const uint32_t *touched;  // latent cells with a gradient this step (the others' gradients are zero)
-    uint32_t *touched_next;   // the next step's, cleared here
-    size_t words;
+    AdamStep st[kSegment];   // the segment's steps
+    int j;                   // this step's place in them
+    uint32_t base;           // steps before the segment
+    uint32_t *seen;          // per latent cell, see advance_kernel
     const float *partial;    // the gradient kernel's weight sums, `ctas` of them
     int ctas;
     double dscale;           // 2 / batch
     unsigned char *wimg;     // the weight image, kept current
-    int descending;          // walk the latents from the last one down
+    int descending;          // sweep_kernel walks the latents from the last one down
 };
 
 __device__ __forceinline__ float sqrt_approx(float x) {
@@ -699,136 +711,184 @@ __device__ __forceinline__ float sqrt_approx(float x) {
 // p -= step * m / (sqrt(v / (1 - beta2^t)) + eps) after the moment updates
 // (bias corrections folded into step and inv_bc2; approximate square root
 // and division, as an optimiser needs no correctly rounded update).
-__device__ __forceinline__ void adam_update(const AdamParams &a, long long gi, float step, float &p, float &m,
-                                            float &v) {
+__device__ __forceinline__ void adam_update(const AdamParams &a, long long gi, float step, float inv_bc2, float &p,
+                                            float &m, float &v) {
     const float gr = __ll2float_rn(gi) * 0x1p-44f;  // fixed point back to FP32 (exact scale)
     m = __fmaf_rn(a.beta1, m, (1.f - a.beta1) * gr);
     v = __fmaf_rn(a.beta2, v, (1.f - a.beta2) * (gr * gr));
-    p = __fmaf_rn(-step, __fdividef(m, sqrt_approx(v * a.inv_bc2) + a.eps), p);
+    p = __fmaf_rn(-step, __fdividef(m, sqrt_approx(v * inv_bc2) + a.eps), p);
 }
 
-__device__ __forceinline__ void adam_quad(const AdamParams &a, float step, float4 &p, float4 &m, float4 &v,
+__device__ __forceinline__ void adam_quad(const AdamParams &a, const AdamStep &st, float4 &p, float4 &m, float4 &v,
                                           longlong2 g01, longlong2 g23) {
-    adam_update(a, g01.x, step, p.x, m.x, v.x);
-    adam_update(a, g01.y, step, p.y, m.y, v.y);
-    adam_update(a, g23.x, step, p.z, m.z, v.z);
-    adam_update(a, g23.y, step, p.w, m.w, v.w);
+    adam_update(a, g01.x, st.lat, st.inv_bc2, p.x, m.x, v.x);
+    adam_update(a, g01.y, st.lat, st.inv_bc2, p.y, m.y, v.y);
+    adam_update(a, g23.x, st.lat, st.inv_bc2, p.z, m.z, v.z);
+    adam_update(a, g23.y, st.lat, st.inv_bc2, p.w, m.w, v.w);
 }
 
-// One step's update, launched as the dependent of the gradient kernel: Adam
-// on the weights (the CTAs' partial sums added in CTA order, as in
-// reduce_kernel), which also refreshes their operand image, and on the
-// latents, reading and clearing the gradients of the cells that a texel
-// reached only (every other gradient is exactly zero, so each update is bit
-// for bit the same).  Bound by the 24 bytes per parameter of parameters and
-// moments.  Each thread loads its first quads before it waits for the
-// gradients, which do not change them.
-// The latents are walked upwards in one step and downwards in the next, so
-// that a step begins with the cells that the last one left in L2 (4096^2
-// texture: 85 us a step with one direction, 71 with both).
-// A 4096^2 step of 8,192 texels took 93 us as seven launches: weight image
-// 4.4, gradients 27.3, weight sums 8.3, Adam 41.4, two memsets and the gaps.
-// Now 17 us of gradients and 47 of update.  Measured and not kept: the
-// untouched cells (nearly all) updated beside the gradient kernel (66-74 us:
-// the moment traffic slows the gradients by as much as it hides), chunks from
-// a counter (72), one, three or four quads in flight or two or four CTAs per
-// SM (70-96), parts of the state kept in L2 by eviction policy (70-73).
-constexpr int kUpThreads = 256, kUpCtasPerSm = 3, kUpQuads = 2;
-__global__ void __launch_bounds__(kUpThreads, kUpCtasPerSm) update_kernel(const AdamParams a) {
-    static_assert(kUpThreads == kRedEntries * kRedRows, "the weight sums' thread layout");
+// The weights' share of a step, 16 slots per CTA and turn for CTA `first`, +
+// `ctas`, ...: the gradient CTAs' partial sums added in CTA order (as in
+// reduce_kernel), Adam, and the operand image.
+__device__ __forceinline__ void update_weights(const AdamParams &a, const AdamStep &st, int first, int ctas) {
     __shared__ double part[kRedRows][kRedEntries];
-    float4 *__restrict__ P = reinterpret_cast<float4 *>(a.params + kOffLat);
-    float4 *__restrict__ M = reinterpret_cast<float4 *>(a.m + kOffLat);
-    float4 *__restrict__ V = reinterpret_cast<float4 *>(a.v + kOffLat);
-    longlong2 *__restrict__ G = reinterpret_cast<longlong2 *>(a.grad + kOffLat);
-    const size_t nq = (a.n - kOffLat) / 4, stride = (size_t)gridDim.x * kUpThreads;
-    const size_t t0 = blockIdx.x * (size_t)kUpThreads + threadIdx.x;
-    const longlong2 z = make_longlong2(0, 0);
-    float4 p[kUpQuads], m[kUpQuads], v[kUpQuads];
-    auto quad_at = [&](size_t i) {  // (past the end: the last quad again, not stored)
-        const size_t c = min(i, nq - 1);
-        return a.descending ? nq - 1 - c : c;
-    };
-    auto load = [&](size_t i) {
-#pragma unroll
-        for (int k = 0; k < kUpQuads; ++k) {
-            const size_t q = quad_at(i + k * stride);
-            p[k] = P[q];
-            m[k] = M[q];
-            v[k] = V[q];
-        }
-    };
-    load(t0);
-    for (size_t w = t0; w < a.words; w += stride) a.touched_next[w] = 0u;
-    // (the weights' own values too, for the CTAs that have some)
-    const int w0 = blockIdx.x * kRedEntries + threadIdx.x;
-    const bool own = threadIdx.x < kRedEntries && w0 < kWeights;
-    const int wp = own ? slot_param(w0) : 0;
-    float w_p = a.params[wp], w_m = a.m[wp], w_v = a.v[wp];
-
-    grid_wait();  // the gradients
-
-    // ---- the weights: 16 slots per CTA and turn (see reduce_kernel)
-    for (int b = blockIdx.x; b * kRedEntries < kWeights; b += gridDim.x) {
+    for (int b = first; b * kRedEntries < kWeights; b += ctas) {
         const int e = b * kRedEntries + (threadIdx.x % kRedEntries), row = threadIdx.x / kRedEntries;
+        const int w = e < kWeights ? slot_param(e) : 0;
+        float p = 0.f, m = 0.f, v = 0.f;
+        if (row == 0) {
+            p = __ldcg(a.params + w);
+            m = __ldcg(a.m + w);
+            v = __ldcg(a.v + w);
+        }
         part[row][threadIdx.x % kRedEntries] = e < kWeights ? partial_sum(a.partial, a.ctas, e, row) : 0.0;
         __syncthreads();
         if (row == 0 && e < kWeights) {
             double tot = 0.0;
             for (int r = 0; r < kRedRows; ++r) tot += part[r][threadIdx.x];
-            const int w = slot_param(e);
-            if (b != (int)blockIdx.x) {
-                w_p = a.params[w];
-                w_m = a.m[w];
-                w_v = a.v[w];
-            }
-            adam_update(a, __double2ll_rn(tot * a.dscale * kFix), a.step_w, w_p, w_m, w_v);
-            a.params[w] = w_p;
-            a.m[w] = w_m;
-            a.v[w] = w_v;
-            put_weight(a.wimg, w, w_p);
+            adam_update(a, __double2ll_rn(tot * a.dscale * kFix), st.w, st.inv_bc2, p, m, v);
+            a.params[w] = p;
+            a.m[w] = m;
+            a.v[w] = v;
+            put_weight(a.wimg, w, p);
         }
         __syncthreads();
     }
+}
 
-    // ---- the latents, kUpQuads quads (half a cell each) per iteration, whose
-    // loads are in flight together; the marks are read one iteration ahead, so
-    // that the gradients of the marked cells are too
-    uint32_t mark[kUpQuads];
-    auto load_marks = [&](size_t i) {
-#pragma unroll
-        for (int k = 0; k < kUpQuads; ++k) {
-            const size_t q = quad_at(i + k * stride);
-            mark[k] = (__ldg(a.touched + (q >> 6)) >> ((q >> 1) & 31)) & 1u;
+// A step's Adam update reaches every cell, but a cell that no texel of the
+// step reads takes it with a gradient of zero, which needs nothing but the
+// cell itself.  So the steps of a call run in segments of up to kSegment; a
+// cell stands still within a segment until a step is about to read it
+// (advance_kernel) or the segment ends (sweep_kernel), and then takes the steps
+// it has missed one after the other, the same operations in the same order.
+// The first of them is the step that read it last, whose gradient waits in the
+// accumulators; the others have none.  A segment moves the 24 bytes of a
+// parameter twice and not once a step.
+// seen[cell]: 1 + the steps that the cell had taken when it was last brought
+// up to date to be read; a value up to `base` is from before the segment.
+//
+// advance_kernel, which runs beside the gradients of step j and ends after
+// them: the cells that step j + 1 reads take their steps up to j, and the
+// weights take step j.  Two threads per cell, sixteen per texel; the first to
+// reach a cell claims it.  Only cells that step j reads too (`late`) wait for
+// its gradients; the gradient kernel neither reads nor changes the others.
+// 4096^2 texture, 8,192 texels: 34 us a step in a call of 64 (gradients and
+// advance 29, a sixteenth of a sweep 6); 67 us in calls of one step, whose
+// sweep moves every parameter, and 93 us with an Adam kernel of all cells and
+// five more launches a step.  Five CTAs per SM 36 us.
+constexpr int kAdvThreads = 256, kAdvCtasPerSm = 4;
+__global__ void __launch_bounds__(kAdvThreads, kAdvCtasPerSm) advance_kernel(const GradParams g, const AdamParams a) {
+    static_assert(kAdvThreads == kRedEntries * kRedRows, "the weight sums' thread layout");
+    float4 *__restrict__ P = reinterpret_cast<float4 *>(a.params + kOffLat);
+    float4 *__restrict__ M = reinterpret_cast<float4 *>(a.m + kOffLat);
+    float4 *__restrict__ V = reinterpret_cast<float4 *>(a.v + kOffLat);
+    longlong2 *__restrict__ G = reinterpret_cast<longlong2 *>(a.grad + kOffLat);
+    const longlong2 z = make_longlong2(0, 0);
+    const uint32_t j = (uint32_t)a.j, seen = a.base + j + 2;
+    const long long items = 16ll * g.n, stride = (long long)gridDim.x * kAdvThreads;
+    const int sub = threadIdx.x & 15, gi = sub >> 3, tap = (sub >> 1) & 3;
+    bool waited = false;
+    for (long long e = (long long)blockIdx.x * kAdvThreads + threadIdx.x; __shfl_sync(FULL, e, 0) < items; e += stride) {
+        const bool valid = e < items;  // (the threads of a texel alike)
+        int x, y, cells[4];
+        float w[4];
+        sample_texel(g, g.step + 1u, (uint32_t)(valid ? e >> 4 : 0), x, y);
+        bilinear_taps(g, gi, x, y, cells, w);
+        const int c01 = tap & 1 ? cells[1] : cells[0], c23 = tap & 1 ? cells[3] : cells[2];
+        const uint32_t cell = (uint32_t)(tap & 2 ? c23 : c01) + (gi ? (uint32_t)(g.gw[0] * g.gh[0]) : 0u);
+        const size_t q = 2 * (size_t)cell + (sub & 1);
+        uint32_t old = seen;
+        if (valid && !(sub & 1)) old = atomicMax(a.seen + cell, seen);
+        old = __shfl_sync(FULL, old, (int)(threadIdx.x & 30));
+        const bool mine = old < seen;
+        uint32_t t = max(old, a.base + 1u) - 1u - a.base;  // the first step to take
+        const bool late = mine && t == j;
+        float4 p, m, v;
+        if (mine) {
+            p = __ldcg(P + q);
+            m = __ldcg(M + q);
+            v = __ldcg(V + q);
         }
-    };
-    load_marks(t0);
-    for (size_t i = t0; i < nq; i += kUpQuads * stride) {
-        longlong2 g0[kUpQuads], g1[kUpQuads];
-#pragma unroll
-        for (int k = 0; k < kUpQuads; ++k) {
-            const size_t q = quad_at(i + k * stride);
-            g0[k] = mark[k] ? G[2 * q] : z;
-            g1[k] = mark[k] ? G[2 * q + 1] : z;
+        if (__any_sync(FULL, late) && !waited) {
+            grid_wait();  // the gradients of step j
+            waited = true;
         }
-        if (i != t0) load(i);
-        uint32_t had = 0;
-#pragma unroll
-        for (int k = 0; k < kUpQuads; ++k) had |= mark[k] << k;
-        load_marks(i + kUpQuads * stride);
-#pragma unroll
-        for (int k = 0; k < kUpQuads; ++k) {
-            if (i + k * stride >= nq) break;
-            const size_t q = quad_at(i + k * stride);
-            adam_quad(a, a.step_lat, p[k], m[k], v[k], g0[k], g1[k]);
-            if ((had >> k) & 1u) {
+        if (mine) {
+            const longlong2 g0 = __ldcg(G + 2 * q), g1 = __ldcg(G + 2 * q + 1);
+            adam_quad(a, a.st[t], p, m, v, g0, g1);
+#pragma unroll 1
+            while (++t <= j) adam_quad(a, a.st[t], p, m, v, z, z);
+            P[q] = p;
+            M[q] = m;
+            V[q] = v;
+            if (g0.x | g0.y | g1.x | g1.y) {
                 G[2 * q] = z;
                 G[2 * q + 1] = z;
             }
-            P[q] = p[k];
-            M[q] = m[k];
-            V[q] = v[k];
         }
+    }
+    grid_wait();
+    grid_trigger();
+    update_weights(a, a.st[a.j], (int)blockIdx.x, (int)gridDim.x);
+}
+
+// The segment's end, after the gradients of its last step j: every cell takes
+// the steps it has missed, and the weights step j.  Bound by the instructions
+// of the updates in long segments (94 us for 10.5 million parameters and 16
+// steps at 85% of the issue slots; 42 us would be the 24 bytes of each), by
+// those bytes in short ones, whose cells are walked up and down in turn so that
+// one starts with the cells that the last one left in L2 (one step: 85 us with
+// one direction, 71 with both).  Five or more CTAs per SM are slower by 3%.
+constexpr int kSweepThreads = 256, kSweepCtasPerSm = 4;
+__global__ void __launch_bounds__(kSweepThreads, kSweepCtasPerSm) sweep_kernel(const AdamParams a) {
+    static_assert(kSweepThreads == kRedEntries * kRedRows, "the weight sums' thread layout");
+    float4 *__restrict__ P = reinterpret_cast<float4 *>(a.params + kOffLat);
+    float4 *__restrict__ M = reinterpret_cast<float4 *>(a.m + kOffLat);
+    float4 *__restrict__ V = reinterpret_cast<float4 *>(a.v + kOffLat);
+    longlong2 *__restrict__ G = reinterpret_cast<longlong2 *>(a.grad + kOffLat);
+    const size_t nq = (a.n - kOffLat) / 4, stride = (size_t)gridDim.x * kSweepThreads;
+    const uint32_t j = (uint32_t)a.j;
+    const longlong2 z = make_longlong2(0, 0);
+    size_t i = blockIdx.x * (size_t)kSweepThreads + threadIdx.x;
+    auto quad_at = [&](size_t k) {  // (past the end: the last quad again, not used)
+        const size_t c = min(k, nq - 1);
+        return a.descending ? nq - 1 - c : c;
+    };
+    // parameters and moments do not change before the wait (of the cells that
+    // step j reads, neither does `seen`, but in a segment's first step)
+    size_t q = quad_at(i);
+    float4 p = __ldcg(P + q), m = __ldcg(M + q), v = __ldcg(V + q);
+    grid_wait();
+    grid_trigger();
+    uint32_t old = __ldcg(a.seen + (q >> 1));
+    update_weights(a, a.st[j], (int)blockIdx.x, (int)gridDim.x);
+    for (; i < nq; i += stride) {
+        const size_t qn = quad_at(i + stride);
+        const uint32_t oldn = __ldcg(a.seen + (qn >> 1));
+        const float4 pn = __ldcg(P + qn), mn = __ldcg(M + qn), vn = __ldcg(V + qn);
+        uint32_t t = 0;
+        longlong2 g0 = z, g1 = z;
+        if (old > a.base) {
+            t = old - 1u - a.base;
+            g0 = __ldcg(G + 2 * q);
+            g1 = __ldcg(G + 2 * q + 1);
+        }
+        adam_quad(a, a.st[t], p, m, v, g0, g1);
+#pragma unroll 1
+        while (++t <= j) adam_quad(a, a.st[t], p, m, v, z, z);
+        P[q] = p;
+        M[q] = m;
+        V[q] = v;
+        if (g0.x | g0.y | g1.x | g1.y) {
+            G[2 * q] = z;
+            G[2 * q + 1] = z;
+        }
+        q = qn;
+        old = oldn;
+        p = pn;
+        m = mn;
+        v = vn;
     }
 }
 
@@ -941,10 +1001,10 @@ struct ctf_trainer_s {
     size_t nparams = 0;
     float *params = nullptr, *m = nullptr, *v = nullptr;
     long long *grad = nullptr, *loss = nullptr;
-    uint32_t *touched = nullptr;  // latent cells that a step's texels reached: two bitmaps, even and odd steps
+    uint32_t *seen = nullptr;       // per latent cell, see advance_kernel
+    uint32_t seen_steps = 0;        // the steps that `seen` counts (all of them, but for an overflow)
     unsigned char *wimg = nullptr;  // FP16 weight operands of the gradient kernel
     float *partial = nullptr;       // per-CTA weight-gradient sums of the gradient kernel
-    size_t touched_words = 0;
     int64_t step = 0;
 };
 
@@ -972,7 +1032,8 @@ GradParams grad_params(const ctf_trainer_s *t) {
     g.k1 = (uint32_t)(t->desc.seed >> 32);
     g.dscale = 0.f;
     g.grad = t->grad;
-    g.touched = t->touched;
+    g.seen = t->seen;
+    g.mark = 0;
     g.loss = t->loss;
     g.per_round = kT;
     g.wimg = t->wimg;
@@ -1039,7 +1100,7 @@ void free_trainer(ctf_trainer_s *t) {
     ctf::dev_free(t->m);
     ctf::dev_free(t->v);
     ctf::dev_free(t->grad);
-    ctf::dev_free(t->touched);
+    ctf::dev_free(t->seen);
     ctf::dev_free(t->loss);
     ctf::dev_free(t->wimg);
     ctf::dev_free(t->partial);
@@ -1058,9 +1119,8 @@ int alloc_trainer(ctf_texture src, const ctf_train_desc *d, ctf_trainer_s **out)
     t->Ht = src->height;
     for (int g = 0; g < 2; ++g) t->n_lat[g] = (size_t)d->latent_w[g] * d->latent_h[g] * 8;
     t->nparams = kOffLat + t->n_lat[0] + t->n_lat[1];
-    t->touched_words = ((t->n_lat[0] + t->n_lat[1]) / 8 + 31) / 32;
     cudaError_t e = ctf::dev_malloc(&t->params, t->nparams * 4);
-    if (e == cudaSuccess) e = ctf::dev_malloc(&t->touched, 2 * t->touched_words * 4);
+    if (e == cudaSuccess) e = ctf::dev_malloc(&t->seen, (t->nparams - kOffLat) / 8 * 4);
     if (e == cudaSuccess) e = ctf::dev_malloc(&t->m, t->nparams * 4);
     if (e == cudaSuccess) e = ctf::dev_malloc(&t->v, t->nparams * 4);
     if (e == cudaSuccess) e = ctf::dev_malloc(&t->grad, t->nparams * 8);
@@ -1072,6 +1132,7 @@ int alloc_trainer(ctf_texture src, const ctf_train_desc *d, ctf_trainer_s **out)
     if (e == cudaSuccess) e = cudaMemset(t->grad, 0, t->nparams * 8);
     if (e == cudaSuccess) e = cudaMemset(t->params, 0, t->nparams * 4);
     if (e == cudaSuccess) e = cudaMemset(t->loss, 0, 8);
+    if (e == cudaSuccess) e = cudaMemset(t->seen, 0, (t->nparams - kOffLat) / 8 * 4);
     if (e != cudaSuccess) {
         free_trainer(t);
         return report_cuda(e, "trainer allocation");
@@ -1158,36 +1219,61 @@ int ctf_trainer_step(ctf_trainer t, int64_t steps, void *stream) {
     a.beta1 = t->desc.beta1;
     a.beta2 = t->desc.beta2;
     a.eps = t->desc.eps;
-    a.words = t->touched_words;
     a.partial = t->partial;
     a.ctas = ctas;
     a.dscale = (double)g.dscale;
     a.wimg = t->wimg;
-    auto bitmap = [&](int64_t st) { return t->touched + (size_t)(st & 1) * t->touched_words; };
-    if (steps > 0) {
-        cudaError_t e = cudaMemsetAsync(t->touched, 0, 2 * t->touched_words * 4, s);
-        if (e == cudaSuccess) e = launch_pack(g, s);
-        if (e != cudaSuccess) return report_cuda(e, "training step");
-    }
-    for (int64_t k = 0; k < steps; ++k) {
-        const int64_t st = t->step;
-        g.step = (uint32_t)st;
-        g.touched = bitmap(st);
-        cudaError_t e = launch_grad(g, ctas, s);
+    a.seen = t->seen;
+    auto adam_step = [&](int64_t st) {
         const double frac = std::fmin(1.0, (double)st / (double)t->desc.total_steps);
         const double sched = 1.0 - (1.0 - t->desc.lr_final_frac) * frac;
         const double bc1 = 1.0 - std::pow((double)t->desc.beta1, (double)(st + 1));
         const double bc2 = 1.0 - std::pow((double)t->desc.beta2, (double)(st + 1));
-        a.step_w = (float)(t->desc.lr_weights * sched / bc1);
-        a.step_lat = (float)(t->desc.lr_latents * sched / bc1);
-        a.inv_bc2 = (float)(1.0 / bc2);
-        a.touched = bitmap(st);
-        a.touched_next = bitmap(st + 1);
-        a.descending = (int)(st & 1);
-        if (e == cudaSuccess)
-            e = launch_dependent(update_kernel, device_sm_count() * kUpCtasPerSm, kUpThreads, 0, s, a);
+        AdamStep r;
+        r.w = (float)(t->desc.lr_weights * sched / bc1);
+        r.lat = (float)(t->desc.lr_latents * sched / bc1);
+        r.inv_bc2 = (float)(1.0 / bc2);
+        return r;
+    };
+    if (steps > 0) {
+        const cudaError_t e = launch_pack(g, s);
         if (e != cudaSuccess) return report_cuda(e, "training step");
-        t->step = st + 1;
+    }
+    // Segments of equal length, to one step; of one step where a step's texels
+    // reach more cells (eight each) than there are, since nothing stands still
+    // then: 4096^2 with 262,144 texels 281 us a step against 302 in segments,
+    // 2048^2 with 65,536 63 against 66; below the line, 4096^2 with 65,536
+    // texels, 124 against 105.
+    const int sms = device_sm_count();
+    const int64_t longest = 64ll * g.n > (int64_t)(t->nparams - kOffLat) ? 1 : kSegment;
+    for (int64_t left = (steps + longest - 1) / longest, k = 0; k < steps; --left) {
+        const int len = (int)((steps - k + left - 1) / left);
+        a.base = t->seen_steps;
+        for (int j = 0; j < len; ++j) a.st[j] = adam_step(t->step + j);
+        cudaError_t e = cudaSuccess;
+        if (a.base > 0xffffff00u) {
+            e = cudaMemsetAsync(t->seen, 0, (t->nparams - kOffLat) / 8 * 4, s);
+            a.base = 0;
+        }
+        for (int j = 0; j < len && e == cudaSuccess; ++j) {
+            g.step = (uint32_t)(t->step + j);
+            g.mark = j == 0 ? a.base + 1u : 0u;
+            a.j = j;
+            e = launch_grad(g, ctas, s);
+            if (e != cudaSuccess) break;
+            if (j + 1 < len) {
+                const long long need = (16ll * g.n + kAdvThreads - 1) / kAdvThreads, cap = 8ll * sms * kAdvCtasPerSm;
+                const long long grid = std::max<long long>(std::min(need, cap), (kWeights + kRedEntries - 1) / kRedEntries);
+                e = launch_dependent(advance_kernel, (int)grid, kAdvThreads, 0, s, g, a);
+            } else {
+                a.descending = (int)(left & 1);
+                e = launch_dependent(sweep_kernel, sms * kSweepCtasPerSm, kSweepThreads, 0, s, a);
+            }
+        }
+        if (e != cudaSuccess) return report_cuda(e, "training step");
+        t->step += len;
+        t->seen_steps = a.base + (uint32_t)len;
+        k += len;
     }
     return CTF_OK;
 }
