@@ -1,16 +1,16 @@
 // ctf_mlp_ws2.cu -- learned-decode filter for STF, Box and Mask Sampling on
-// single views: warps specialised by role, with the texel features computed
-// by the warps that select the texels.
+// single views and batches: warps specialised by role.
 //
 // A CTA of 256 threads (four per SM) takes the groups of 8 pixel tiles g0,
 // g0 + G, ... (G = gridDim.x) in turn:
 //   - warpgroup 1 (warps 4-7, the producers, two tiles of the group each)
-//     runs step 1 of the collaborative flow (Sec. 3) on its tiles, lists
+//     runs step 1 of the collaborative flow (Sec. 3) on its tiles and lists
 //     their texels in consecutive rows (a shared-memory counter gives each
-//     tile its rows), and writes the features of the rows straight into the
-//     group's layer-1 operand buffer in the tensor cores' layout;
-//   - warpgroup 0 (warps 0-3, the consumer) owns the 128 TMEM lanes and runs
-//     the tcgen05 MLP chain(s) over the group's rows: three MMA layers, the
+//     tile its rows);
+//   - warpgroup 0 (warps 0-3, the consumer) writes the features of the rows
+//     straight into the group's layer-1 operand buffer in the tensor cores'
+//     layout, owns the 128 TMEM lanes and runs the tcgen05 MLP chain(s) over
+//     the group's rows: three MMA layers, the
 //     two hidden epilogues (bias, ReLU, conversion to the next operand) and
 //     the output epilogue into the row values; then it gathers, filters and
 //     stores the group's pixels from the row values (warp w the tiles w and
@@ -25,9 +25,14 @@
 // rotate over consecutive groups, so the producers may run two groups ahead
 // of the consumer.  The producers hand a stage over with a full barrier (four
 // arrivals) and get it back with a done barrier (one arrival, after the
-// gather); a named barrier among the producers at the start of each group
-// orders their reuse of the texel list.  Every wait is bounded; a wait that
-// gives up records CTF_ERR_TIMEOUT and both roles leave.
+// gather); a row's texel waits in the row's own place in the operand buffer,
+// so the producer warps do not wait for one another.  Every wait is bounded; a
+// wait that gives up records CTF_ERR_TIMEOUT and both roles leave.
+// The roles share the work so that neither waits long: with the features on
+// the producers the consumer stood still for half of the time (4,500 of 8,600
+// clocks a group) and a 3840x2160 Mask-11 FP16 view took 198 us, now 193; in
+// the batch kernel, whose parameters are read from shared memory, the features
+// stay on the producers (256 views 473 us, on the consumer 493).
 // What bounds it: instruction issue (about 700 warp instructions a tile at
 // 60-65% of the issue slots with 32 warps on an SM), not the tensor pipe and
 // not memory.  So the rows are given out by a counter rather than found by a
@@ -81,19 +86,18 @@ constexpr int kPTmem = kPBar + 8;
 constexpr int kPHand = kPBar + 16;               // full[kPMaxStages], done[kPMaxStages]
 // producer warps x 64 rank slots (two texels per lane may rank 64 texels a tile)
 constexpr int kPRanks = kPHand + 16 * kPMaxStages;
-constexpr int kPList = kPRanks + kPProducerWarps * 64 * 4;  // the group's texels, int2 per row
-constexpr int kPListEnd = kPList + kPGroupRows * 8;         // fallback variant: the warps' texel tables; then the stages
+constexpr int kPRanksEnd = kPRanks + kPProducerWarps * 64 * 4;  // fallback variant: the warps' texel tables; then the stages
 
 // One stage of a group of at most T tiles (offsets in bytes).
 template <int T>
 struct PStage {
     static constexpr int kPix = 32 * T;              // pixels, and rows at most
-    static constexpr int kX = 0;                     // layer-1 operand, 32 B a row; the row values (16 B) overlay it
+    // layer-1 operand, 32 B a row; before it a row's texel (p_texel), after it the row values (16 B each)
+    static constexpr int kX = 0;
     static constexpr int kWord = kX + kPix * 32;     // float4 per pixel: s, t, the packed word, unused
     static constexpr int kBase = kWord + kPix * 16;  // int2 per tile: first row, first pixel
-    static constexpr int kRowsOff = kBase + T * 8;   // int: rows of the group
-    static constexpr int kAlloc = kRowsOff + 4;      // int: rows given out so far
-    static constexpr int kEnd = kRowsOff + 16;
+    static constexpr int kAlloc = kBase + T * 8;     // int: rows given out so far
+    static constexpr int kEnd = kAlloc + 16;
     static constexpr int kQ = kEnd;                  // fallback variant: int2 texel a pixel's lane produces
     static constexpr int kUL = kQ + kPix * 8;        // fallback variant: int2 upper-left texel of the footprint
     static constexpr int kFbEnd = kUL + kPix * 8;
@@ -110,10 +114,10 @@ struct PLayout {
     static_assert(!(kFb && kBatch), "batches take no fallbacks on learned views");
     using S = PStage<kPTiles>;
     static constexpr int kStages = kFb ? 2 : 3;
-    static constexpr int kStage0 = kPListEnd + (kFb ? (4 + kPProducerWarps) * (int)sizeof(FbTable) : kBatch ? 2 * kPProducerWarps * kPViewBytes : 0);
+    static constexpr int kStage0 = kPRanksEnd + (kFb ? (4 + kPProducerWarps) * (int)sizeof(FbTable) : kBatch ? 2 * kPProducerWarps * kPViewBytes : 0);
     static constexpr int kStageBytes = kFb ? S::kFbEnd : S::kEnd + (kBatch ? kPViewBytes : 0);
     static constexpr int kBytes = kStage0 + kStages * kStageBytes;
-    static_assert(kStage0 % 16 == 0 && kStageBytes % 16 == 0 && kPListEnd % 16 == 0, "16-byte operand buffers");
+    static_assert(kStage0 % 16 == 0 && kStageBytes % 16 == 0 && kPRanksEnd % 16 == 0, "16-byte operand buffers");
     // kPCtasPerSm CTAs per SM fit, and no more than four (4 x 128 TMEM columns)
     static_assert(kPCtasPerSm * (kBytes + 1024 + 128) <= 228 * 1024, "the CTAs of an SM fit in shared memory");
 };
@@ -137,7 +141,6 @@ __device__ __forceinline__ void p_arrive(uint64_t *bar) {
 // Named barriers: 1 among the 128 consumer threads, 2 among the producer
 // threads (0 stays __syncthreads).
 __device__ __forceinline__ void cons_bar() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
-__device__ __forceinline__ void prod_bar() { asm volatile("bar.sync 2, %0;" ::"n"(kPProducerThreads) : "memory"); }
 
 // Barrier `id` among n threads, returning whether any of them passed true.
 template <int id, int n>
@@ -314,6 +317,14 @@ __device__ __forceinline__ bool p_chain(unsigned char *sm, uint32_t tmem, uint64
     return true;
 }
 
+// The texel of row `row` of a stage waits in the first 16 bytes of the row's
+// place in the layer-1 operand: the thread that reads it is the one that
+// writes the row's features over it.
+template <typename S>
+__device__ __forceinline__ int2 *p_texel(unsigned char *st, int row) {
+    return reinterpret_cast<int2 *>(st + S::kX + (row >> 3) * 256 + (row & 7) * 16);
+}
+
 // n rows of the group for tile slot g whose first pixel is `pixel`; the stage
 // keeps both for the gather.  (The rows of the tiles follow one another in
 // the order in which the warps come; a row's place does not change its
@@ -377,7 +388,7 @@ __device__ __forceinline__ Inputs p_load(const ExactParams &p, const LanePlace<T
 
 template <int ALG, int TW, int MD, bool kStats, bool kFb, bool kTwo = false>
 __device__ __forceinline__ void p_step1(const ExactParams &p, const LanePlace<TW> &lp, uint32_t bx, uint32_t by,
-                                        const Inputs &in, int g, unsigned char *st, int2 *list, int lane, uint32_t lt, int *ranks,
+                                        const Inputs &in, int g, unsigned char *st, int lane, uint32_t lt, int *ranks,
                                         Counters &cnt, FbTable *fbt) {
     using S = typename PLayout<kFb>::S;
     constexpr uint32_t TH = 32 / TW;
@@ -399,7 +410,7 @@ __device__ __forceinline__ void p_step1(const ExactParams &p, const LanePlace<TW
     }
     float4 *word = reinterpret_cast<float4 *>(st + S::kWord) + 32 * g + lane;
     auto put = [&](int row, int x, int y) {
-        list[ck(row, kPGroupRows, p.err, kBndTexList)] =
+        *p_texel<S>(st, ck(row, kPGroupRows, p.err, kBndTexList)) =
             make_int2(min(max(x, 0), p.Wt - 1), min(max(y, 0), p.Ht - 1));
     };
     if (kFb && p.fallback != 0 && sel.path == PATH_FALLBACK_BUDGET) {  // warp-uniform
@@ -498,6 +509,21 @@ __device__ __forceinline__ void p_gather(const ExactParams &p, uint32_t off, int
     if (p.evals) p.evals[idx] = cv;
 }
 
+// The features of rows tid, tid + 128 of the R rows of stage st in the tensor
+// cores' operand layout, for thread tid of a role; published to the MMAs.
+static_assert(kPProducerThreads == kRows, "either role has a thread per row of a chain");
+template <typename S, bool kFp8>
+__device__ __forceinline__ void p_features(const MlpDevice &m, unsigned char *st, int R, int tid, const float *inv_a1) {
+#pragma unroll 1
+    for (int row = tid; row < R; row += kRows) {
+        const int2 t = *p_texel<S>(st, row);
+        float f[kMlpIn];
+        texel_features(m, t.x, t.y, f);
+        store_x_row_at(st + S::kX, row, f, kFp8, inv_a1);
+    }
+    tc::fence_proxy_async();  // generic-proxy writes -> the MMAs' async proxy
+}
+
 // Column and row of the tile g places after (bx, by).
 __device__ __forceinline__ void p_tile(uint32_t tiles_x, uint32_t &bx, uint32_t &by, uint32_t g) {
     bx += g;
@@ -521,7 +547,7 @@ __global__ void __launch_bounds__(kPThreads, kPCtasPerSm)
     const int lane = threadIdx.x & 31;
     const int warp = __shfl_sync(FULL, (int)(threadIdx.x >> 5), 0);  // uniform, and known to be
     // fallback variant: warp w's texel table (empty between tiles)
-    FbTable *fbt = kFb ? reinterpret_cast<FbTable *>(sm + kPListEnd) + warp : nullptr;
+    FbTable *fbt = kFb ? reinterpret_cast<FbTable *>(sm + kPRanksEnd) + warp : nullptr;
     if (kFb) fb_clear(fbt, lane);
     uint64_t *mma_bar = reinterpret_cast<uint64_t *>(sm + kPBar);
     uint32_t *tslot = reinterpret_cast<uint32_t *>(sm + kPTmem);
@@ -576,11 +602,14 @@ __global__ void __launch_bounds__(kPThreads, kPCtasPerSm)
             unsigned char *st = p_stage<kFb>(sm, s);
             bool ok = tc::mbar_wait(p_full(sm, s), par, kMaxTries);
             __syncwarp();
+            // the features of rows tid and tid + 128 in the tensor cores' operand layout
+            const int R = min(__shfl_sync(FULL, *reinterpret_cast<const int *>(st + S::kAlloc), 0), kPGroupRows);
+            if (ok) p_features<S, kFp8>(m, st, R, tid, inv_a1);
             if (bar_or<1, kRows>(!ok)) {
                 if (tid == 0) atomicExch(err, CTF_ERR_TIMEOUT);
                 break;
             }
-            const int R = __shfl_sync(FULL, *reinterpret_cast<const int *>(st + S::kRowsOff), 0);
+            if (kStats && tid == 0) cnt.v[kStatTexelEvalsUnique] += R;
             const int passes = (R + kRows - 1) / kRows;
             float4 *outrow = reinterpret_cast<float4 *>(st + S::kX);
             const uint32_t sX = tc::smem_addr(st + S::kX);
@@ -605,15 +634,16 @@ __global__ void __launch_bounds__(kPThreads, kPCtasPerSm)
             }
             __syncwarp();
             cons_bar();  // every consumer warp has read the stage
-            if (tid == 0) p_arrive(p_done(sm, s));
+            if (tid == 0) {
+                *reinterpret_cast<int *>(st + S::kAlloc) = 0;
+                p_arrive(p_done(sm, s));
+            }
         }
     } else {
         // ---------------- producers: kPSlots tile slots per warp ----------------
         const int pw = warp - 4;
         const uint32_t lt = lanemask_lt();
         int *ranks = reinterpret_cast<int *>(sm + kPRanks) + 64 * pw;
-        int2 *list = reinterpret_cast<int2 *>(sm + kPList);
-        const int pt = threadIdx.x - kRows;  // producer thread
         const LanePlace<TW> lp(p, lane);
         // the warp's tiles, advanced by the grid's stride without dividing again
         const uint32_t tiles_x = (uint32_t)p.tiles_x;
@@ -629,20 +659,12 @@ __global__ void __launch_bounds__(kPThreads, kPCtasPerSm)
             {
                 const int s = (int)(j % kPStages);
                 unsigned char *st = p_stage<kFb>(sm, s);
-                if (j >= kPStages) {
-                    // the consumer has gathered group j - kPStages from this stage
+                if (j >= kPStages) {  // the consumer has gathered group j - kPStages from this stage
                     const bool okd = tc::mbar_wait(p_done(sm, s), (uint32_t)(((j - kPStages) / kPStages) & 1), kMaxTries);
-                    __syncwarp();
-                    // (this barrier also says that every producer warp has read
-                    // the texel lists of group j - 1)
-                    if (bar_or<2, kPProducerThreads>(!okd)) {
-                        if (threadIdx.x == 128) atomicExch(err, CTF_ERR_TIMEOUT);
+                    if (!__all_sync(FULL, okd)) {
+                        if (lane == 0) atomicExch(err, CTF_ERR_TIMEOUT);
                         break;
                     }
-                } else {
-                    // every producer warp has read the texel lists of group j - 1
-                    __syncwarp();
-                    prod_bar();
                 }
 #pragma unroll 1
                 for (int k = 0; k < kSlots; ++k) {
@@ -662,32 +684,12 @@ __global__ void __launch_bounds__(kPThreads, kPCtasPerSm)
                         ny = gy;
                     }
                     const Inputs next = p_load<ALG, TW>(p, lp, nx, ny);
-                    p_step1<ALG, TW, MD, kStats, kFb, kTwo>(p, lp, bx, by, in, kSlots * pw + k, st, list, lane, lt,
+                    p_step1<ALG, TW, MD, kStats, kFb, kTwo>(p, lp, bx, by, in, kSlots * pw + k, st, lane, lt,
                                                             ranks, cnt, fbt);
                     bx = nx;
                     by = ny;
                     in = next;
                 }
-                // the next group's stage starts with no rows given out (the last
-                // group that used it has its row count in kRowsOff)
-                if (pt == 0) *reinterpret_cast<int *>(p_stage<kFb>(sm, (int)((j + 1) % kPStages)) + S::kAlloc) = 0;
-                __syncwarp();
-                prod_bar();  // every tile's texels are in the list
-                const int R = *reinterpret_cast<const int *>(st + S::kAlloc);
-                if (pt == 0) {
-                    *reinterpret_cast<int *>(st + S::kRowsOff) = R;
-                    if (kStats) cnt.v[kStatTexelEvalsUnique] += R;
-                }
-                // features of rows pt, pt + kPProducerThreads, ... in the tensor
-                // cores' operand layout
-#pragma unroll 1
-                for (int row = pt; row < R; row += kPProducerThreads) {
-                    const int2 t = list[ck(row, kPGroupRows, p.err, kBndTexList)];
-                    float f[kMlpIn];
-                    texel_features(m, t.x, t.y, f);
-                    store_x_row_at(st + S::kX, ck(row, kPGroupRows, p.err, kBndRow), f, kFp8, inv_a1);
-                }
-                tc::fence_proxy_async();  // generic-proxy writes -> the MMAs' async proxy
                 __syncwarp();
                 if (lane == 0) p_arrive(p_full(sm, s));
             }
@@ -823,7 +825,8 @@ __global__ void __launch_bounds__(kPThreads, kPCtasPerSm)
                 loaded = m.img;
             }
             const bool fp8 = __shfl_sync(FULL, m.fp8, 0) != 0;
-            const int R = __shfl_sync(FULL, *reinterpret_cast<const int *>(st + S::kRowsOff), 0);
+            const int R = min(__shfl_sync(FULL, *reinterpret_cast<const int *>(st + S::kAlloc), 0), kPGroupRows);
+            if (kStats && tid == 0) cnt.v[kStatTexelEvalsUnique] += R;
             const int passes = (R + kRows - 1) / kRows;
             float4 *outrow = reinterpret_cast<float4 *>(st + S::kX);
             const uint32_t sX = tc::smem_addr(st + S::kX);
@@ -851,17 +854,18 @@ __global__ void __launch_bounds__(kPThreads, kPCtasPerSm)
             }
             __syncwarp();
             cons_bar();  // every consumer warp has read the stage
-            if (tid == 0) p_arrive(p_done(sm, s));
+            if (tid == 0) {
+                *reinterpret_cast<int *>(st + S::kAlloc) = 0;
+                p_arrive(p_done(sm, s));
+            }
         }
     } else {
         // ---------------- producers ----------------
         const int pw = warp - 4;
         const uint32_t lt = lanemask_lt();
         int *ranks = reinterpret_cast<int *>(sm + kPRanks) + 64 * pw;
-        int2 *list = reinterpret_cast<int2 *>(sm + kPList);
-        const int pt = threadIdx.x - kRows;  // producer thread
         // this warp's copies of its current and its next group's view
-        unsigned char *own = sm + kPListEnd + 2 * pw * kPViewBytes;
+        unsigned char *own = sm + kPRanksEnd + 2 * pw * kPViewBytes;
         auto params = [&](int c) -> const ExactParams & {
             return *reinterpret_cast<const ExactParams *>(own + c * kPViewBytes);
         };
@@ -903,33 +907,19 @@ __global__ void __launch_bounds__(kPThreads, kPCtasPerSm)
                 nxt = cur ^ 1;
                 locate(next_item, at, nxt);
             }
-            if (j >= kPStages) {
-                // the consumer has gathered group j - kPStages from this stage
-                const bool okd = tc::mbar_wait(p_done(sm, s), (uint32_t)(((j - kPStages) / kPStages) & 1), kMaxTries);
-                __syncwarp();
-                // (this barrier also says that every producer warp has read
-                // the texel lists of the last group)
-                if (bar_or<2, kPProducerThreads>(!okd)) {
-                    if (threadIdx.x == 128) atomicExch(err, CTF_ERR_TIMEOUT);
-                    break;
-                }
-            } else {
-                // every producer warp has read the texel lists of the last group
-                __syncwarp();
-                prod_bar();
-            }
+            // the consumer has gathered group j - kPStages from this stage
+            bool okd = true;
+            if (j >= kPStages)
+                okd = __all_sync(FULL, tc::mbar_wait(p_done(sm, s), (uint32_t)(((j - kPStages) / kPStages) & 1), kMaxTries));
             const ExactParams &p = params(cur);
-            const MlpDevice &m = *reinterpret_cast<const MlpDevice *>(own + cur * kPViewBytes + sizeof(ExactParams));
-            if (pw == 0) {  // the view for the consumer
+            if (okd && pw == 0) {  // the view for the consumer
                 const uint4 *src = reinterpret_cast<const uint4 *>(own + cur * kPViewBytes);
                 if (lane < kPViewBytes / 16) reinterpret_cast<uint4 *>(st + kPBat)[lane] = src[lane];
             }
-            const bool fp8 = m.fp8 != 0;
-            const float *inv_a1 = reinterpret_cast<const float *>(reinterpret_cast<const unsigned char *>(m.img) + kImgA1);
             const LanePlace<TW> lp(p, lane);
             const uint32_t tiles_x = (uint32_t)p.tiles_x;
 #pragma unroll 1
-            for (int k = 0; k < kPSlots; ++k) {
+            for (int k = 0; k < kPSlots && okd; ++k) {
                 uint32_t nx = bx, ny = by;
                 Inputs next;
                 if (k + 1 < kPSlots) {
@@ -940,29 +930,26 @@ __global__ void __launch_bounds__(kPThreads, kPCtasPerSm)
                     if (more) first_tile(next_item, at, nxt, nx, ny);
                     next = p_load<ALG, TW>(params(nxt), LanePlace<TW>(params(nxt), lane), nx, ny);
                 }
-                p_step1<ALG, TW, MD, kStats, false>(p, lp, bx, by, in, kPSlots * pw + k, st, list, lane, lt, ranks,
+                p_step1<ALG, TW, MD, kStats, false>(p, lp, bx, by, in, kPSlots * pw + k, st, lane, lt, ranks,
                                                     cnt, nullptr);
                 bx = nx;
                 by = ny;
                 in = next;
             }
-            // (as in the single-view kernel)
-            if (pt == 0) *reinterpret_cast<int *>(p_stage<false, true>(sm, (int)((j + 1) % kPStages)) + S::kAlloc) = 0;
             __syncwarp();
-            prod_bar();  // every tile's texels are in the list
-            const int R = *reinterpret_cast<const int *>(st + S::kAlloc);
-            if (pt == 0) {
-                *reinterpret_cast<int *>(st + S::kRowsOff) = R;
-                if (kStats) cnt.v[kStatTexelEvalsUnique] += R;
+            // every tile's texels are listed (unless a warp gave up its wait)
+            if (bar_or<2, kPProducerThreads>(!okd)) {
+                if (threadIdx.x == kRows) atomicExch(err, CTF_ERR_TIMEOUT);
+                break;
             }
-#pragma unroll 1
-            for (int row = pt; row < R; row += kPProducerThreads) {
-                const int2 t = list[ck(row, kPGroupRows, err, kBndTexList)];
-                float f[kMlpIn];
-                texel_features(m, t.x, t.y, f);
-                store_x_row_at(st + S::kX, ck(row, kPGroupRows, err, kBndRow), f, fp8, inv_a1);
+            {
+                const MlpDevice &m = *reinterpret_cast<const MlpDevice *>(own + cur * kPViewBytes + sizeof(ExactParams));
+                const float *inv_a1 =
+                    reinterpret_cast<const float *>(reinterpret_cast<const unsigned char *>(m.img) + kImgA1);
+                const int R = *reinterpret_cast<const int *>(st + S::kAlloc), pt = (int)threadIdx.x - kRows;
+                if (m.fp8) p_features<S, true>(m, st, R, pt, inv_a1);
+                else p_features<S, false>(m, st, R, pt, inv_a1);
             }
-            tc::fence_proxy_async();  // generic-proxy writes -> the MMAs' async proxy
             __syncwarp();
             if (lane == 0) p_arrive(p_full(sm, s));
             item = next_item;
