@@ -138,7 +138,8 @@ __device__ __forceinline__ ListUnion list_union(bool active, int ulx, int uly, i
 // and the same outputs, whichever lane evaluates a texel), list_union
 // otherwise.  A hash table in shared memory for every tile, which this
 // replaces, took 486 instructions a tile and 28.6 us for a 1283x797 view
-// (now 16.4 us), and 129 us against 77 us for a 1920x1080 FP8 learned view.
+// (16.4 us with the union, 12.2 with what came after), and 129 us against 77 us
+// for a 1920x1080 FP8 learned view (60 now).
 // kTwo: the variant that may evaluate two texels per lane (p.tpl == 2); the
 // other carries no code for it.
 template <int ALG, int MD, bool kStats, bool kUnique = true, bool kTwo = false>
