@@ -438,10 +438,12 @@ int ctf_checkpoint_load(const char *path, ctf_texture *out);
  * the GPU alone); the others share two persistent launches on the stream,
  * one per kind of texel evaluation (block views first).  Block views: CTAs
  * of 8 warps, every warp takes items of 32 warp tiles from an atomic
- * counter.  Learned views: CTAs of 4 warps that keep their tensor memory
- * for the whole launch take items of 8 warp tiles (4 for per-pixel 4-tap)
- * that share MLP chains, items_per_fetch at a time.  Every view is filtered
- * exactly as ctf_filter would filter it with the same options. */
+ * counter.  Learned views: CTAs that keep their tensor memory for the whole
+ * launch take items of 8 warp tiles that share MLP chains, CTA c the items c,
+ * c + G, ... of all views; with per-pixel 4-tap (items of 4 warp tiles) or
+ * group_dedup they take items_per_fetch at a time from an atomic counter.
+ * Every view is filtered exactly as ctf_filter would filter it with the same
+ * options. */
 typedef struct {
     ctf_texture tex;            /* block or learned-decode texture */
     const float *uv, *jac;      /* device, [height][width][2] and [4] */
@@ -454,8 +456,10 @@ typedef struct {
 
 /* Launch shape of a batch; NULL means the defaults in brackets.
  *   filter           tile shape, budget, mask_dim, edge_remap (as ctf_filter)
- *   items_per_fetch  learned views: items taken per fetch, 1..64      [4]
- *   ctas_per_sm      learned views: persistent CTAs per SM, 1..4       [4]
+ *   items_per_fetch  learned views, 4-tap or group_dedup: items taken per
+ *                    fetch, 1..64                                      [4]
+ *   ctas_per_sm      learned views, 4-tap or group_dedup: persistent CTAs
+ *                    per SM, 1..4                                      [4]
  *   solo_tiles       views of at least this many warp tiles get their own
  *                    launch; 0: every view in the persistent launches [16384]
  * (the block-view launch always fills every SM to its occupancy limit). */
