@@ -155,9 +155,9 @@ inline uint64_t fnv1a(const void *data, size_t n, uint64_t h = 14695981039346656
     return h;
 }
 // The learned filters with warps specialised by role, which
-// launch_mlp_filter uses for STF, Box and Mask Sampling: the features
-// computed by the selecting warps (ctf_mlp_ws2.cu), and with group_dedup the
-// consumer merging the group's lists (ctf_mlp_ws.cu).
+// launch_mlp_filter uses for STF, Box and Mask Sampling: the packed-group
+// kernel (ctf_mlp_ws2.cu, ctf_mlp_pf.cu), and with group_dedup the consumer
+// merging the group's lists (ctf_mlp_ws.cu).
 bool mlp_filter_ws_applies(const ExactParams &p, int alg);
 // Box and Mask with fallback C / C+ and one texel per lane run the
 // fallback variant of the packed-group kernel (ctf_mlp_ws2.cu).

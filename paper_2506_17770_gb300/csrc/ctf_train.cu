@@ -764,7 +764,7 @@ __device__ __forceinline__ void update_weights(const AdamParams &a, const AdamSt
 // it has missed one after the other, the same operations in the same order.
 // The first of them is the step that read it last, whose gradient waits in the
 // accumulators; the others have none.  A segment moves the 24 bytes of a
-// parameter twice and not once a step.
+// parameter once, and once more each time its cell is read, and not once a step.
 // seen[cell]: 1 + the steps that the cell had taken when it was last brought
 // up to date to be read; a value up to `base` is from before the segment.
 //
