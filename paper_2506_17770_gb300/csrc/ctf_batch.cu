@@ -242,8 +242,8 @@ __global__ void __launch_bounds__(kRows, 4) batch_mlp_kernel(const BatchParams b
                 loaded_img = img;
                 __syncthreads();
             }
-            if (ALG == ALG_4TAP)
-                ok = mlp_warp_tile<ALG, TW, MD>(V.p, V.m, ch, local * 4 + warp, lane, lt, cnt, inv_a1, b.err);
+            if constexpr (ALG == ALG_4TAP)
+                ok = mlp_warp_tile<TW>(V.p, V.m, ch, local * 4 + warp, lane, cnt, inv_a1, b.err);
             else
                 ok = mlp_group<ALG, TW, MD>(V.p, V.m, ch, local * kGroupTiles, lane, lt, cnt, inv_a1, b.err);
         }

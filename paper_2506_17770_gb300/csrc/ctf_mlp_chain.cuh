@@ -388,14 +388,13 @@ __device__ __forceinline__ void chain_teardown(const Chain &ch) {
 }
 
 
-// One iteration of the learned-decode filter for the calling warp's pixel
-// tile `tile` of view p: step 1 of the collaborative flow, the warp's texels
-// through the MLP chain (all 4 warps of the CTA call this together), the
-// gather and filter, the store.  Returns false if the chain gave up.
-template <int ALG, int TW, int MD>
+// One iteration of the learned per-pixel 4-tap filter for the calling warp's
+// pixel tile `tile` of view p: the four taps through the MLP chain, one after
+// the other (all 4 warps of the CTA call this together), the filter, the
+// store.  Returns false if the chain gave up.
+template <int TW>
 __device__ __forceinline__ bool mlp_warp_tile(const ExactParams &p, const MlpDevice &m, Chain &ch, long long tile,
-                                              int lane, uint32_t lt, Counters &cnt,
-                                              const float *inv_a1, int *err) {
+                                              int lane, Counters &cnt, const float *inv_a1, int *err) {
     constexpr int TH = 32 / TW;
     unsigned char *sm = ch.sm;
     const int tx = lane % TW, ty = lane / TW;
@@ -410,11 +409,9 @@ __device__ __forceinline__ bool mlp_warp_tile(const ExactParams &p, const MlpDev
                             kBndPixel);
     PixelSetup ps;
     float2 uv = make_float2(0.f, 0.f);
-    float4 jac = make_float4(0.f, 0.f, 0.f, 0.f);
     bool covered = inside;
     if (inside) {
         uv = __ldcs(p.uv + idx);
-        if (ALG >= ALG_LIST) jac = __ldcs(p.jac + idx);
         if (p.cov) covered = __ldcs(p.cov + idx) != 0;
     }
     ps.active = covered;
@@ -422,107 +419,53 @@ __device__ __forceinline__ bool mlp_warp_tile(const ExactParams &p, const MlpDev
 
     float4 result = make_float4(0.f, 0.f, 0.f, 0.f);
     uint8_t count = 0;
-    if (ALG == ALG_4TAP) {
-        const uint32_t A = __ballot_sync(FULL, ps.active);
-        if (valid) {
-            cnt.v[kStatTilesTotal] += 1;
-            if (A == 0) {
-                cnt.v[kStatTilesEmpty] += 1;
-            } else {
-                cnt.v[kStatPixelsActive] += __popc(A);
-                cnt.v[kStatTilesDirect] += 1;
-                cnt.v[kStatTexelEvals] += 4 * __popc(A);
-                cnt.v[kStatTexelEvalsUnique] += 4 * __popc(A);
-            }
-        }
-        float4 tap[4];
-#pragma unroll 1
-        for (int k = 0; k < 4; ++k) {
-            if (ps.active) {
-                const int x = min(max(ps.ulx + (k & 1), 0), p.Wt - 1);
-                const int y = min(max(ps.uly + (k >> 1), 0), p.Ht - 1);
-                float f[kMlpIn];
-                texel_features(m, x, y, f);
-                store_x_row(sm, threadIdx.x, f, m.fp8, inv_a1);
-            } else {
-                store_zero_x_row(sm, threadIdx.x);
-            }
-            ok = mlp_chain(ch, m.fp8, tap[k], err);
-            if (!ok) return false;
-        }
-        if (!ok) return false;
-        if (ps.active) {
-            float w[4];
-            bilinear_weights(ps.s, ps.t, w);
-            float r = 0.f, g = 0.f, b = 0.f, a = 0.f;
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                r = __fmaf_rn(w[k], tap[k].x, r);
-                g = __fmaf_rn(w[k], tap[k].y, g);
-                b = __fmaf_rn(w[k], tap[k].z, b);
-                a = __fmaf_rn(w[k], tap[k].w, a);
-            }
-            result = make_float4(r, g, b, a);
-            count = 4;
-        }
-    } else {
-        Selection sel;
-        if (valid) {
-            sel = select_tile<ALG, MD, true>(p, ps, jac, px, py, lane, lt,
-                                          reinterpret_cast<int *>(sm + kSmRanks) + 32 * (threadIdx.x >> 5), cnt);
+    const uint32_t A = __ballot_sync(FULL, ps.active);
+    if (valid) {
+        cnt.v[kStatTilesTotal] += 1;
+        if (A == 0) {
+            cnt.v[kStatTilesEmpty] += 1;
         } else {
-            sel.path = PATH_EMPTY;
-            sel.produce = false;
-            sel.count = 0;
-#pragma unroll
-            for (int k = 0; k < 4; ++k) sel.src[k] = lane;
+            cnt.v[kStatPixelsActive] += __popc(A);
+            cnt.v[kStatTilesDirect] += 1;
+            cnt.v[kStatTexelEvals] += 4 * __popc(A);
+            cnt.v[kStatTexelEvalsUnique] += 4 * __popc(A);
         }
-        // step 2: the lane's texel goes into the lane's own row
-        if (sel.produce) {
-            const int x = min(max(sel.tx, 0), p.Wt - 1), y = min(max(sel.ty, 0), p.Ht - 1);
+    }
+    float4 tap[4];
+#pragma unroll 1
+    for (int k = 0; k < 4; ++k) {
+        if (ps.active) {
+            const int x = min(max(ps.ulx + (k & 1), 0), p.Wt - 1);
+            const int y = min(max(ps.uly + (k >> 1), 0), p.Ht - 1);
             float f[kMlpIn];
             texel_features(m, x, y, f);
             store_x_row(sm, threadIdx.x, f, m.fp8, inv_a1);
         } else {
             store_zero_x_row(sm, threadIdx.x);
         }
-        float4 val;
-        ok = mlp_chain(ch, m.fp8, val, err);
+        ok = mlp_chain(ch, m.fp8, tap[k], err);
         if (!ok) return false;
-        if (sel.path == PATH_SUCCESS) {
-            // step 3: gather the 2x2 taps from the producing lanes
-            float4 tap[4];
+    }
+    if (!ok) return false;
+    if (ps.active) {
+        float w[4];
+        bilinear_weights(ps.s, ps.t, w);
+        float r = 0.f, g = 0.f, b = 0.f, a = 0.f;
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                tap[k].x = __shfl_sync(FULL, val.x, sel.src[k]);
-                tap[k].y = __shfl_sync(FULL, val.y, sel.src[k]);
-                tap[k].z = __shfl_sync(FULL, val.z, sel.src[k]);
-                tap[k].w = __shfl_sync(FULL, val.w, sel.src[k]);
-            }
-            if (ps.active) {
-                float w[4];
-                bilinear_weights(ps.s, ps.t, w);
-                float r = 0.f, g = 0.f, b = 0.f, a = 0.f;
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    r = __fmaf_rn(w[k], tap[k].x, r);
-                    g = __fmaf_rn(w[k], tap[k].y, g);
-                    b = __fmaf_rn(w[k], tap[k].z, b);
-                    a = __fmaf_rn(w[k], tap[k].w, a);
-                }
-                result = make_float4(r, g, b, a);
-                count = sel.count;
-            }
-        } else if (ps.active) {
-            result = val;
-            count = 1;
+        for (int k = 0; k < 4; ++k) {
+            r = __fmaf_rn(w[k], tap[k].x, r);
+            g = __fmaf_rn(w[k], tap[k].y, g);
+            b = __fmaf_rn(w[k], tap[k].z, b);
+            a = __fmaf_rn(w[k], tap[k].w, a);
         }
+        result = make_float4(r, g, b, a);
+        count = 4;
     }
     if (inside) {
         __stcs(p.out + idx, result);
         if (p.evals) p.evals[idx] = count;
     }
-        return true;
+    return true;
 }
 
 // One iteration of the learned-decode filter for the collaborative
