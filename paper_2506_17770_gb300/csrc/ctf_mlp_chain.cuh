@@ -244,9 +244,14 @@ __device__ __forceinline__ void hidden_epilogue(unsigned char *sm, uint32_t tadd
 
 // The three layers for the 128 rows whose layer-1 operand is in place.
 // Every thread of the CTA calls it; returns false (for every thread alike)
-// if an MMA did not complete within the wait bound.
-__device__ __forceinline__ bool mlp_chain(Chain &ch, bool fp8, float4 &out, int *err) {
-    const int tid = threadIdx.x, warp = tid >> 5;
+// if an MMA did not complete within the wait bound.  One elected thread of
+// warp 0 issues the MMAs inside a warp-uniform branch, and a branch holds one
+// kind of them: the compiler then knows that descriptors, TMEM addresses and
+// predicates are uniform.
+template <bool kFp8>
+__device__ __forceinline__ bool mlp_chain_as(Chain &ch, float4 &out, int *err) {
+    const int tid = threadIdx.x;
+    const int warp = __shfl_sync(FULL, tid >> 5, 0);  // uniform, and known to be
     unsigned char *sm = ch.sm;
     const float *b1 = reinterpret_cast<const float *>(sm + kImgB1);
     const float *b2 = reinterpret_cast<const float *>(sm + kImgB2);
@@ -259,24 +264,22 @@ __device__ __forceinline__ bool mlp_chain(Chain &ch, bool fp8, float4 &out, int 
     const uint32_t sW1 = tc::smem_addr(sm + kImgW1), sW2 = tc::smem_addr(sm + kImgW2),
                    sW3 = tc::smem_addr(sm + kImgW3);
     // K-major no-swizzle descriptors; one MMA covers K = 16 (FP16) or 32 (E4M3)
-    const uint32_t esz = fp8 ? 1u : 2u;
-    const uint32_t kstep_bytes = 256;  // two 16-byte core-matrix columns = 32 bytes of K per row group
-    const uint32_t sboX = fp8 ? 256u : 256u;   // K = 32 B per row either way
-    const uint32_t sboH = fp8 ? 512u : 1024u;  // 64 elements per row
-    const int nk_h = fp8 ? 2 : 4;              // MMAs over K = 64
-    const uint32_t id64 = fp8 ? tc::idesc_e4m3(128, 64) : tc::idesc_f16(128, 64);
-    const uint32_t id16 = fp8 ? tc::idesc_e4m3(128, 16) : tc::idesc_f16(128, 16);
-    (void)esz;
+    constexpr uint32_t kstep_bytes = 256;  // two 16-byte core-matrix columns = 32 bytes of K per row group
+    constexpr uint32_t sboX = 256u;        // K = 32 B per row either way
+    constexpr uint32_t sboH = kFp8 ? 512u : 1024u;  // 64 elements per row
+    constexpr int nk_h = kFp8 ? 2 : 4;              // MMAs over K = 64
+    constexpr uint32_t id64 = kFp8 ? tc::idesc_e4m3(128, 64) : tc::idesc_f16(128, 64);
+    constexpr uint32_t id16 = kFp8 ? tc::idesc_e4m3(128, 16) : tc::idesc_f16(128, 16);
 
     bool timed_out = false;
     // ---- layer 1: D[0..64) = X * W1^T
     tc::fence_proxy_async();
     tc::fence_before_sync();
     __syncthreads();
-    if (tid == 0) {
+    if (warp == 0 && tc::elect_one()) {
         tc::fence_after_sync();
         const uint64_t a = tc::smem_desc(sX, 128, sboX), b = tc::smem_desc(sW1, 128, sboX);
-        if (fp8) tc::mma_e4m3(ch.tmem, a, b, id64, false);
+        if (kFp8) tc::mma_e4m3(ch.tmem, a, b, id64, false);
         else tc::mma_f16(ch.tmem, a, b, id64, false);
         tc::commit(ch.bar);
     }
@@ -284,7 +287,7 @@ __device__ __forceinline__ bool mlp_chain(Chain &ch, bool fp8, float4 &out, int 
     __syncwarp();  // the lanes may leave the wait apart; tcgen05.ld needs the whole warp
     ch.phase ^= 1u;
     tc::fence_after_sync();
-    hidden_epilogue(sm, lane_base + 0, b1, s1, fp8, tid);
+    hidden_epilogue(sm, lane_base + 0, b1, s1, kFp8, tid);
     // ---- layer 2: D[64..128) = H1 * W2^T
     tc::fence_proxy_async();
     tc::fence_before_sync();
@@ -292,12 +295,13 @@ __device__ __forceinline__ bool mlp_chain(Chain &ch, bool fp8, float4 &out, int 
         if (tid == 0) atomicExch(err, CTF_ERR_TIMEOUT);
         return false;
     }
-    if (tid == 0) {
+    if (warp == 0 && tc::elect_one()) {
         tc::fence_after_sync();
+#pragma unroll
         for (int j = 0; j < nk_h; ++j) {
             const uint64_t a = tc::smem_desc(sH + j * kstep_bytes, 128, sboH);
             const uint64_t b = tc::smem_desc(sW2 + j * kstep_bytes, 128, sboH);
-            if (fp8) tc::mma_e4m3(ch.tmem + 64, a, b, id64, j > 0);
+            if (kFp8) tc::mma_e4m3(ch.tmem + 64, a, b, id64, j > 0);
             else tc::mma_f16(ch.tmem + 64, a, b, id64, j > 0);
         }
         tc::commit(ch.bar);
@@ -307,7 +311,7 @@ __device__ __forceinline__ bool mlp_chain(Chain &ch, bool fp8, float4 &out, int 
     ch.phase ^= 1u;
     tc::fence_after_sync();
     // the layer-2 MMAs have read H1, so H2 may overwrite it
-    hidden_epilogue(sm, lane_base + 64, b2, s2, fp8, tid);
+    hidden_epilogue(sm, lane_base + 64, b2, s2, kFp8, tid);
     // ---- layer 3: D[0..16) = H2 * W3^T
     tc::fence_proxy_async();
     tc::fence_before_sync();
@@ -315,12 +319,13 @@ __device__ __forceinline__ bool mlp_chain(Chain &ch, bool fp8, float4 &out, int 
         if (tid == 0) atomicExch(err, CTF_ERR_TIMEOUT);
         return false;
     }
-    if (tid == 0) {
+    if (warp == 0 && tc::elect_one()) {
         tc::fence_after_sync();
+#pragma unroll
         for (int j = 0; j < nk_h; ++j) {
             const uint64_t a = tc::smem_desc(sH + j * kstep_bytes, 128, sboH);
             const uint64_t b = tc::smem_desc(sW3 + j * kstep_bytes, 128, sboH);
-            if (fp8) tc::mma_e4m3(ch.tmem, a, b, id16, j > 0);
+            if (kFp8) tc::mma_e4m3(ch.tmem, a, b, id16, j > 0);
             else tc::mma_f16(ch.tmem, a, b, id16, j > 0);
         }
         tc::commit(ch.bar);
@@ -336,7 +341,7 @@ __device__ __forceinline__ bool mlp_chain(Chain &ch, bool fp8, float4 &out, int 
     float o[4];
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
-        const float v = fp8 ? __fmaf_rn(d[c], s3[c], b3[c]) : __fadd_rn(d[c], b3[c]);
+        const float v = kFp8 ? __fmaf_rn(d[c], s3[c], b3[c]) : __fadd_rn(d[c], b3[c]);
         o[c] = fminf(fmaxf(v, 0.f), 1.f);
     }
     out = make_float4(o[0], o[1], o[2], o[3]);
@@ -346,6 +351,11 @@ __device__ __forceinline__ bool mlp_chain(Chain &ch, bool fp8, float4 &out, int 
         return false;
     }
     return true;
+}
+
+// The same for a network known at run time (fp8 is the same for every thread).
+__device__ __forceinline__ bool mlp_chain(Chain &ch, bool fp8, float4 &out, int *err) {
+    return __shfl_sync(FULL, (int)fp8, 0) ? mlp_chain_as<true>(ch, out, err) : mlp_chain_as<false>(ch, out, err);
 }
 
 // CTA set-up shared by both kernels: operand image into shared memory,
@@ -365,6 +375,7 @@ __device__ __forceinline__ void chain_setup(Chain &ch, unsigned char *sm, const 
         tc::fence_mbar_init();
     }
     if ((threadIdx.x >> 5) == 0) {
+        __syncwarp();  // tcgen05.alloc needs the whole warp
         tc::tmem_alloc(tslot, kTmemCols);
         tc::tmem_relinquish();
     }

@@ -145,11 +145,13 @@ __device__ __forceinline__ void ws_hidden_epilogue(unsigned char *sm, uint32_t t
 }
 
 // The three layers for the 128 rows whose layer-1 operand the consumer
-// threads have written; mlp_chain with the consumer barrier in place of the
-// CTA barrier.  Returns false (for every consumer thread alike) if an MMA
+// threads have written; mlp_chain_as with the consumer barrier in place of
+// the CTA barrier.  Returns false (for every consumer thread alike) if an MMA
 // did not complete within the wait bound.
-__device__ __forceinline__ bool ws_chain(Chain &ch, bool fp8, float4 &out, int *err) {
-    const int tid = threadIdx.x, warp = tid >> 5;
+template <bool kFp8>
+__device__ __forceinline__ bool ws_chain(Chain &ch, float4 &out, int *err) {
+    const int tid = threadIdx.x;
+    const int warp = __shfl_sync(FULL, tid >> 5, 0);  // uniform, and known to be
     unsigned char *sm = ch.sm;
     const float *b1 = reinterpret_cast<const float *>(sm + kImgB1);
     const float *b2 = reinterpret_cast<const float *>(sm + kImgB2);
@@ -161,22 +163,22 @@ __device__ __forceinline__ bool ws_chain(Chain &ch, bool fp8, float4 &out, int *
     const uint32_t sX = tc::smem_addr(sm + kSmX), sH = tc::smem_addr(sm + kSmH);
     const uint32_t sW1 = tc::smem_addr(sm + kImgW1), sW2 = tc::smem_addr(sm + kImgW2),
                    sW3 = tc::smem_addr(sm + kImgW3);
-    const uint32_t kstep_bytes = 256;
-    const uint32_t sboX = 256u;
-    const uint32_t sboH = fp8 ? 512u : 1024u;
-    const int nk_h = fp8 ? 2 : 4;
-    const uint32_t id64 = fp8 ? tc::idesc_e4m3(128, 64) : tc::idesc_f16(128, 64);
-    const uint32_t id16 = fp8 ? tc::idesc_e4m3(128, 16) : tc::idesc_f16(128, 16);
+    constexpr uint32_t kstep_bytes = 256;
+    constexpr uint32_t sboX = 256u;
+    constexpr uint32_t sboH = kFp8 ? 512u : 1024u;
+    constexpr int nk_h = kFp8 ? 2 : 4;
+    constexpr uint32_t id64 = kFp8 ? tc::idesc_e4m3(128, 64) : tc::idesc_f16(128, 64);
+    constexpr uint32_t id16 = kFp8 ? tc::idesc_e4m3(128, 16) : tc::idesc_f16(128, 16);
 
     bool timed_out = false;
     // ---- layer 1: D[0..64) = X * W1^T
     tc::fence_proxy_async();
     tc::fence_before_sync();
     cons_sync();
-    if (tid == 0) {
+    if (warp == 0 && tc::elect_one()) {
         tc::fence_after_sync();
         const uint64_t a = tc::smem_desc(sX, 128, sboX), b = tc::smem_desc(sW1, 128, sboX);
-        if (fp8) tc::mma_e4m3(ch.tmem, a, b, id64, false);
+        if (kFp8) tc::mma_e4m3(ch.tmem, a, b, id64, false);
         else tc::mma_f16(ch.tmem, a, b, id64, false);
         tc::commit(ch.bar);
     }
@@ -184,7 +186,7 @@ __device__ __forceinline__ bool ws_chain(Chain &ch, bool fp8, float4 &out, int *
     __syncwarp();
     ch.phase ^= 1u;
     tc::fence_after_sync();
-    ws_hidden_epilogue(sm, lane_base + 0, b1, s1, fp8, tid);
+    ws_hidden_epilogue(sm, lane_base + 0, b1, s1, kFp8, tid);
     // ---- layer 2: D[64..128) = H1 * W2^T
     tc::fence_proxy_async();
     tc::fence_before_sync();
@@ -192,12 +194,13 @@ __device__ __forceinline__ bool ws_chain(Chain &ch, bool fp8, float4 &out, int *
         if (tid == 0) atomicExch(err, CTF_ERR_TIMEOUT);
         return false;
     }
-    if (tid == 0) {
+    if (warp == 0 && tc::elect_one()) {
         tc::fence_after_sync();
+#pragma unroll
         for (int j = 0; j < nk_h; ++j) {
             const uint64_t a = tc::smem_desc(sH + j * kstep_bytes, 128, sboH);
             const uint64_t b = tc::smem_desc(sW2 + j * kstep_bytes, 128, sboH);
-            if (fp8) tc::mma_e4m3(ch.tmem + 64, a, b, id64, j > 0);
+            if (kFp8) tc::mma_e4m3(ch.tmem + 64, a, b, id64, j > 0);
             else tc::mma_f16(ch.tmem + 64, a, b, id64, j > 0);
         }
         tc::commit(ch.bar);
@@ -207,7 +210,7 @@ __device__ __forceinline__ bool ws_chain(Chain &ch, bool fp8, float4 &out, int *
     ch.phase ^= 1u;
     tc::fence_after_sync();
     // the layer-2 MMAs have read H1, so H2 may overwrite it
-    ws_hidden_epilogue(sm, lane_base + 64, b2, s2, fp8, tid);
+    ws_hidden_epilogue(sm, lane_base + 64, b2, s2, kFp8, tid);
     // ---- layer 3: D[0..16) = H2 * W3^T
     tc::fence_proxy_async();
     tc::fence_before_sync();
@@ -215,12 +218,13 @@ __device__ __forceinline__ bool ws_chain(Chain &ch, bool fp8, float4 &out, int *
         if (tid == 0) atomicExch(err, CTF_ERR_TIMEOUT);
         return false;
     }
-    if (tid == 0) {
+    if (warp == 0 && tc::elect_one()) {
         tc::fence_after_sync();
+#pragma unroll
         for (int j = 0; j < nk_h; ++j) {
             const uint64_t a = tc::smem_desc(sH + j * kstep_bytes, 128, sboH);
             const uint64_t b = tc::smem_desc(sW3 + j * kstep_bytes, 128, sboH);
-            if (fp8) tc::mma_e4m3(ch.tmem, a, b, id16, j > 0);
+            if (kFp8) tc::mma_e4m3(ch.tmem, a, b, id16, j > 0);
             else tc::mma_f16(ch.tmem, a, b, id16, j > 0);
         }
         tc::commit(ch.bar);
@@ -236,7 +240,7 @@ __device__ __forceinline__ bool ws_chain(Chain &ch, bool fp8, float4 &out, int *
     float o[4];
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
-        const float v = fp8 ? __fmaf_rn(d[c], s3[c], b3[c]) : __fadd_rn(d[c], b3[c]);
+        const float v = kFp8 ? __fmaf_rn(d[c], s3[c], b3[c]) : __fadd_rn(d[c], b3[c]);
         o[c] = fminf(fmaxf(v, 0.f), 1.f);
     }
     out = make_float4(o[0], o[1], o[2], o[3]);
@@ -353,8 +357,9 @@ __device__ __forceinline__ void ws_gather(const ExactParams &p, long long first,
     if (p.evals) p.evals[idx] = cv;
 }
 
-// kDedup: group_dedup (the variant without it carries no code for it).
-template <int ALG, int TW, int MD, bool kDedup>
+// kDedup: group_dedup (the variant without it carries no code for it).  kFp8:
+// an E4M3 network (one kind of MMA in a kernel).
+template <int ALG, int TW, int MD, bool kDedup, bool kFp8>
 __global__ void __launch_bounds__(kWsThreads, 4) mlp_filter_ws_kernel(const ExactParams p, const MlpDevice m,
                                                                       int *err) {
     extern __shared__ __align__(1024) unsigned char sm[];
@@ -390,14 +395,18 @@ __global__ void __launch_bounds__(kWsThreads, 4) mlp_filter_ws_kernel(const Exac
             const int s = (int)(j & 1);
             const uint32_t par = (uint32_t)((j >> 1) & 1);
             unsigned char *st = ws_stage(sm, s);
-            if (cons_or(!tc::mbar_wait(ws_bar(sm, kBarFull, s), par, kMaxTries))) {
+            const bool full = tc::mbar_wait(ws_bar(sm, kBarFull, s), par, kMaxTries);
+            __syncwarp();  // the lanes may leave the wait apart; bar.red is for whole warps
+            if (cons_or(!full)) {
                 if (tid == 0) atomicExch(err, CTF_ERR_TIMEOUT);
                 break;
             }
             // the row values and row map of this stage are free once the
             // gather of group j - 2 is done (it always is by now: each
             // producer warp gathers group j - 2 before its step 1 of group j)
-            if (j >= 2 && cons_or(!tc::mbar_wait(ws_bar(sm, kBarGathered, s), par ^ 1u, kMaxTries))) {
+            const bool gathered = j < 2 || tc::mbar_wait(ws_bar(sm, kBarGathered, s), par ^ 1u, kMaxTries);
+            __syncwarp();
+            if (cons_or(!gathered)) {
                 if (tid == 0) atomicExch(err, CTF_ERR_TIMEOUT);
                 break;
             }
@@ -498,12 +507,12 @@ __global__ void __launch_bounds__(kWsThreads, 4) mlp_filter_ws_kernel(const Exac
                     const int2 t = c == 0 ? xy[0] : xy[1];
                     float f[kMlpIn];
                     texel_features(m, t.x, t.y, f);
-                    store_x_row(sm, tid, f, m.fp8, inv_a1);
+                    store_x_row(sm, tid, f, kFp8, inv_a1);
                 } else {
                     store_zero_x_row(sm, tid);
                 }
                 float4 v;
-                ok = ws_chain(ch, m.fp8, v, err);
+                ok = ws_chain<kFp8>(ch, v, err);
                 if (ok) outrow[ck(row, 2 * kRows, p.err, kBndRow)] = v;
             }
             if (!ok) break;
@@ -564,13 +573,14 @@ __global__ void __launch_bounds__(kWsThreads, 4) mlp_filter_ws_kernel(const Exac
 
 using WsFn = void (*)(const ExactParams, const MlpDevice, int *);
 
-template <int TW, bool kDedup>
+template <int TW, bool kDedup, bool kFp8>
 WsFn ws_pick(int alg, int md) {
     switch (alg) {
-    case ALG_STF: return mlp_filter_ws_kernel<ALG_STF, TW, 16, kDedup>;
-    case ALG_BOX: return mlp_filter_ws_kernel<ALG_BOX, TW, 16, kDedup>;
+    case ALG_STF: return mlp_filter_ws_kernel<ALG_STF, TW, 16, kDedup, kFp8>;
+    case ALG_BOX: return mlp_filter_ws_kernel<ALG_BOX, TW, 16, kDedup, kFp8>;
     case ALG_MASK:
-        return md == 11 ? mlp_filter_ws_kernel<ALG_MASK, TW, 11, kDedup> : mlp_filter_ws_kernel<ALG_MASK, TW, 16, kDedup>;
+        return md == 11 ? mlp_filter_ws_kernel<ALG_MASK, TW, 11, kDedup, kFp8>
+                        : mlp_filter_ws_kernel<ALG_MASK, TW, 16, kDedup, kFp8>;
     default: return nullptr;
     }
 }
@@ -596,12 +606,12 @@ cudaError_t ws_prepare(WsFn fn) {
 
 // Only the group_dedup variant is launched: without the option the
 // producers compute the features themselves (ctf_mlp_ws2.cu).
-WsFn ws_kernel(int alg, int tile_w, int mask_dim, bool dedup) {
+WsFn ws_kernel(int alg, int tile_w, int mask_dim, bool dedup, bool fp8) {
     if (!dedup) return nullptr;
     switch (tile_w) {
-    case 8: return ws_pick<8, true>(alg, mask_dim);
-    case 4: return ws_pick<4, true>(alg, mask_dim);
-    case 16: return ws_pick<16, true>(alg, mask_dim);
+    case 8: return fp8 ? ws_pick<8, true, true>(alg, mask_dim) : ws_pick<8, true, false>(alg, mask_dim);
+    case 4: return fp8 ? ws_pick<4, true, true>(alg, mask_dim) : ws_pick<4, true, false>(alg, mask_dim);
+    case 16: return fp8 ? ws_pick<16, true, true>(alg, mask_dim) : ws_pick<16, true, false>(alg, mask_dim);
     default: return nullptr;
     }
 }
@@ -613,13 +623,17 @@ bool mlp_filter_ws_applies(const ExactParams &, int alg) {
 }
 
 cudaError_t prepare_mlp_filter_ws(int alg, int tile_w, int mask_dim) {
-    WsFn fn = ws_kernel(alg, tile_w, mask_dim, true);
-    return fn ? ws_prepare(fn) : cudaErrorInvalidValue;
+    for (int fp8 = 0; fp8 < 2; ++fp8) {
+        WsFn fn = ws_kernel(alg, tile_w, mask_dim, true, fp8 != 0);
+        const cudaError_t e = fn ? ws_prepare(fn) : cudaErrorInvalidValue;
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 cudaError_t launch_mlp_filter_ws(const ExactParams &p, const MlpDevice &m, int alg, int tile_w, int mask_dim,
                                  int *err, cudaStream_t stream) {
-    WsFn fn = ws_kernel(alg, tile_w, mask_dim, p.group_dedup != 0);
+    WsFn fn = ws_kernel(alg, tile_w, mask_dim, p.group_dedup != 0, m.fp8 != 0);
     if (!fn) return cudaErrorInvalidValue;
     if (p.n_tiles == 0) return cudaSuccess;
     if (p.n_tiles > 0x7fffffffLL) return cudaErrorInvalidValue;  // tile positions use 32-bit arithmetic
