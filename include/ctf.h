@@ -307,6 +307,13 @@ int64_t ctf_debug_device_allocations(void);
 int64_t ctf_debug_live_allocations(void);
 int ctf_debug_fail_allocations(int skip, int n);
 
+/* The same for kernel launches: ctf_debug_fail_launches(skip, n) lets the
+ * library's next `skip` launches through and asks for a block of 2,048
+ * threads in the n after them, which the runtime refuses on the host (nothing
+ * runs): the entry point returns CTF_ERR_CUDA and the CUDA context stays
+ * usable.  n = 0 disarms it; negative arguments return CTF_ERR_ARG. */
+int ctf_debug_fail_launches(int skip, int n);
+
 /* Debug build.  The library also builds as libctf_debug.so (compiled with
  * -DCTF_DEBUG): the same entry points and results, and every data-dependent
  * index its kernels use to reach a texel (block or latent cell), a pixel of

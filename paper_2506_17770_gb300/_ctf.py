@@ -132,6 +132,7 @@ def _bind_optional(lib):
         "ctf_debug_device_allocations": ([], ctypes.c_int64),
         "ctf_debug_live_allocations": ([], ctypes.c_int64),
         "ctf_debug_fail_allocations": ([I, I], I),
+        "ctf_debug_fail_launches": ([I, I], I),
         "ctf_debug_build": ([], I),
         "ctf_debug_selftest_bounds": ([I, P], I),
     }
@@ -362,6 +363,12 @@ def ctf_debug_fail_allocations(n, skip=0):
     """Let the library's next `skip` device allocations through, then make
     the n after them fail (CTF_ERR_OOM); n = 0 disarms."""
     _check(load().ctf_debug_fail_allocations(int(skip), int(n)))
+
+
+def ctf_debug_fail_launches(n, skip=0):
+    """Let the library's next `skip` kernel launches through, then have the
+    runtime refuse the n after them (CTF_ERR_CUDA); n = 0 disarms."""
+    _check(load().ctf_debug_fail_launches(int(skip), int(n)))
 
 
 def ctf_debug_build() -> bool:

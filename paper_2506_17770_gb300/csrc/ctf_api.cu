@@ -359,8 +359,7 @@ __global__ void bounds_selftest_kernel(int index, int *err) {
 }  // namespace
 
 cudaError_t launch_bounds_selftest(int index, int *err, cudaStream_t stream) {
-    bounds_selftest_kernel<<<1, 32, 0, stream>>>(index, err);
-    return cudaGetLastError();
+    return launch_plain(bounds_selftest_kernel, 1, 32, 0, stream, index, err);
 }
 
 std::mutex g_alloc_mutex;
@@ -398,6 +397,24 @@ void dev_free(void *p) {
     cudaFree(p);
     std::lock_guard<std::mutex> lk(g_alloc_mutex);
     --g_alloc_live;
+}
+
+// Launches that a test has refused.  (The flag keeps the mutex out of calls
+// that no test armed.)
+static std::atomic<bool> g_launch_armed{false};
+static std::mutex g_launch_mutex;
+static int g_launch_skip = 0, g_launch_fail = 0;
+
+bool refuse_launch() {
+    if (!g_launch_armed.load(std::memory_order_relaxed)) return false;
+    std::lock_guard<std::mutex> lk(g_launch_mutex);
+    if (g_launch_fail <= 0) return false;
+    if (g_launch_skip > 0) {
+        --g_launch_skip;
+        return false;
+    }
+    if (--g_launch_fail == 0) g_launch_armed.store(false);
+    return true;
 }
 
 }  // namespace ctf
@@ -512,6 +529,16 @@ int ctf_debug_fail_allocations(int skip, int n) {
     std::lock_guard<std::mutex> lk(ctf::g_alloc_mutex);
     ctf::g_alloc_skip = skip;
     ctf::g_alloc_fail = n;
+    return CTF_OK;
+}
+
+int ctf_debug_fail_launches(int skip, int n) {
+    g_last_error.clear();
+    if (skip < 0 || n < 0) return fail(CTF_ERR_ARG, "skip = %d and n = %d must not be negative", skip, n);
+    std::lock_guard<std::mutex> lk(ctf::g_launch_mutex);
+    ctf::g_launch_skip = skip;
+    ctf::g_launch_fail = n;
+    ctf::g_launch_armed.store(n > 0);
     return CTF_OK;
 }
 

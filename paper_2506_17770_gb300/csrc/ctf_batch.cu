@@ -529,8 +529,7 @@ cudaError_t launch_plan(const Plan &plan, const DevPlan &dp, int alg, const Reso
             long long grid = (long long)device_sm_count() * r.ctas_per_sm;
             const long long useful = (plan.items[k] + r.items_per_fetch - 1) / r.items_per_fetch;
             if (grid > useful) grid = useful;
-            fn<<<(int)grid, kRows, kSmRequest, s>>>(b);
-            e = cudaGetLastError();
+            e = launch_plain(fn, (int)grid, kRows, kSmRequest, s, b);
             if (e != cudaSuccess) return e;
         } else {
             long long grid =

@@ -187,7 +187,10 @@ int resident_ctas(const void *fn, int threads) {
     for (int i = 0; i < used; ++i)
         if (table[i].fn == fn && table[i].dev == dev && table[i].threads == threads) return table[i].ctas;
     int ctas = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctas, fn, threads, 0) != cudaSuccess || ctas < 1) return 1;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctas, fn, threads, 0) != cudaSuccess || ctas < 1) {
+        cudaGetLastError();  // (the launch that follows answers for itself)
+        return 1;
+    }
     if (used < 256) table[used++] = Entry{fn, dev, threads, ctas};
     return ctas;
 }

@@ -208,6 +208,31 @@ void clear_error();
 // allocates.
 int device_error_word(int **out);
 
+// Whether a test has asked for this launch to be refused
+// (ctf_debug_fail_launches, ctf_api.cu).
+bool refuse_launch();
+
+// Every kernel of the library is launched here.  The answer is the launch's
+// own: what an earlier call left as the runtime's last error is not taken for
+// it, and a refused launch leaves none for the next.
+template <typename... Params, typename... Args>
+cudaError_t launch_with(void (*fn)(Params...), bool dependent, int grid, int threads, size_t smem, cudaStream_t s,
+                        const Args &...args) {
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)(refuse_launch() ? 2048 : threads));
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &attr;
+    cfg.numAttrs = dependent ? 1 : 0;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, fn, args...);
+    if (e != cudaSuccess) cudaGetLastError();
+    return e;
+}
+
 // A launch that may begin while the kernel before it in the stream runs or
 // ends: fn sets itself up, calls grid_wait (ctf_device.cuh) before it touches
 // anything that a kernel or copy before it may write or read, and grid_trigger
@@ -220,17 +245,14 @@ int device_error_word(int **out);
 template <typename... Params, typename... Args>
 cudaError_t launch_dependent(void (*fn)(Params...), int grid, int threads, size_t smem, cudaStream_t s,
                              const Args &...args) {
-    cudaLaunchAttribute attr{};
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3((unsigned)threads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, fn, args...);
+    return launch_with(fn, true, grid, threads, smem, s, args...);
+}
+
+// A launch that begins when everything before it in the stream is done.
+template <typename... Params, typename... Args>
+cudaError_t launch_plain(void (*fn)(Params...), int grid, int threads, size_t smem, cudaStream_t s,
+                         const Args &...args) {
+    return launch_with(fn, false, grid, threads, smem, s, args...);
 }
 
 // Every device allocation of the library goes through here (ctf_api.cu): it

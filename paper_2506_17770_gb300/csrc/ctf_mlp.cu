@@ -137,8 +137,7 @@ cudaError_t prepare_mlp_filter(int alg, int tile_w, int mask_dim) {
 }
 
 cudaError_t launch_bounded_wait_selftest(uint32_t polls, int *err, cudaStream_t stream) {
-    bounded_wait_selftest_kernel<<<1, kRows, 0, stream>>>(polls, err);
-    return cudaGetLastError();
+    return launch_plain(bounded_wait_selftest_kernel, 1, kRows, 0, stream, polls, err);
 }
 
 cudaError_t launch_mlp_filter(const ExactParams &p, const MlpDevice &m, const MlpEpilogue &ep, int alg, int tile_w,
@@ -163,8 +162,7 @@ cudaError_t launch_mlp_filter(const ExactParams &p, const MlpDevice &m, const Ml
     const long long iters = (p.n_tiles + mlp_group_tiles(alg) - 1) / mlp_group_tiles(alg);
     const long long cap = (long long)device_sm_count() * 4;
     const int grid = (int)(iters < cap ? iters : cap);
-    fn<<<grid, kRows, kSmRequest, stream>>>(p, m, err);
-    return cudaGetLastError();
+    return launch_plain(fn, grid, kRows, kSmRequest, stream, p, m, err);
 }
 
 }  // namespace ctf

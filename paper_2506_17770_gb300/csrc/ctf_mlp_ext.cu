@@ -253,8 +253,7 @@ cudaError_t launch_mlp_filter_ext(const ExactParams &p, const MlpDevice &m, int 
     const long long iters = (p.n_tiles + 3) / 4;
     const long long cap = (long long)device_sm_count() * 4;
     const int grid = (int)(iters < cap ? iters : cap);
-    fn<<<grid, kRows, kSmRequest, stream>>>(p, m, err);
-    return cudaGetLastError();
+    return launch_plain(fn, grid, kRows, kSmRequest, stream, p, m, err);
 }
 
 }  // namespace ctf

@@ -642,8 +642,7 @@ cudaError_t launch_mlp_filter_ws(const ExactParams &p, const MlpDevice &m, int a
     const long long groups = (p.n_tiles + kGroupTiles - 1) / kGroupTiles;
     const long long cap = (long long)device_sm_count() * 4;
     const int grid = (int)(groups < cap ? groups : cap);
-    fn<<<grid, kWsThreads, kWsBytes, stream>>>(p, m, err);
-    return cudaGetLastError();
+    return launch_plain(fn, grid, kWsThreads, kWsBytes, stream, p, m, err);
 }
 
 }  // namespace ctf

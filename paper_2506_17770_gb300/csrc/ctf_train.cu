@@ -1077,8 +1077,7 @@ cudaError_t launch_grad(const GradParams &g, int ctas, cudaStream_t s) {
 }
 
 cudaError_t launch_pack(const GradParams &g, cudaStream_t s) {
-    pack_kernel<<<(kPackThreads + 255) / 256, 256, 0, s>>>(g.params, g.wimg);
-    return cudaGetLastError();
+    return launch_plain(pack_kernel, (kPackThreads + 255) / 256, 256, 0, s, g.params, g.wimg);
 }
 
 int check_desc(const ctf_train_desc *d) {
@@ -1178,8 +1177,8 @@ int ctf_trainer_create(ctf_texture exact_src, const ctf_train_desc *desc, ctf_tr
     ctf_trainer_s *t = nullptr;
     int rc = alloc_trainer(exact_src, desc, &t);
     if (rc) return rc;
-    init_kernel<<<1024, 256>>>(t->params, t->nparams, (uint32_t)(desc->seed & 0xffffffffu), (uint32_t)(desc->seed >> 32));
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_plain(init_kernel, 1024, 256, 0, nullptr, t->params, t->nparams,
+                                 (uint32_t)(desc->seed & 0xffffffffu), (uint32_t)(desc->seed >> 32));
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e != cudaSuccess) {
         free_trainer(t);
@@ -1295,9 +1294,8 @@ int ctf_trainer_gradients(ctf_trainer t, const int32_t *xy, int n, double *loss,
     if (e == cudaSuccess) e = launch_pack(g, s);
     if (e == cudaSuccess) e = launch_grad(g, ctas, s);
     if (e == cudaSuccess) {
-        reduce_kernel<<<(kWeights + kRedEntries - 1) / kRedEntries, kRedEntries * kRedRows, 0, s>>>(
-            g.partial, ctas, (double)g.dscale, g.grad);
-        e = cudaGetLastError();
+        e = launch_plain(reduce_kernel, (kWeights + kRedEntries - 1) / kRedEntries, kRedEntries * kRedRows, 0, s,
+                         g.partial, ctas, (double)g.dscale, g.grad);
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return report_cuda(e, "gradient kernel");
@@ -1382,8 +1380,7 @@ int ctf_trainer_export(ctf_trainer t, ctf_eval_mode mode, ctf_texture *out) {
         if (e == cudaSuccess) e = cudaMemset(dmax, 0, 144 * 4);
         if (e == cudaSuccess) {
             GradParams g = grad_params(t);
-            actstats_kernel<<<device_sm_count() * 4, kThreads>>>(g, dmax);
-            e = cudaGetLastError();
+            e = launch_plain(actstats_kernel, device_sm_count() * 4, kThreads, 0, nullptr, g, dmax);
         }
         if (e == cudaSuccess) e = cudaMemcpy(amax.data(), dmax, 144 * 4, cudaMemcpyDeviceToHost);
         ctf::dev_free(dmax);
@@ -1517,13 +1514,11 @@ int ctf_texture_compare(ctf_texture ref, ctf_texture learned, double *mse_rgb, d
     const MlpDevice m = mlp_device_view(learned);
     for (long long st = 0; st < total && e == cudaSuccess; st += chunk) {
         const int n = (int)std::min<long long>(chunk, total - st);
-        linear_xy_kernel<<<1024, 256, 0, s>>>(xy, st, n, ref->width);
-        e = cudaGetLastError();
+        e = launch_plain(linear_xy_kernel, 1024, 256, 0, s, xy, st, n, ref->width);
         if (e == cudaSuccess) e = launch_mlp_decode(m, learned->epi, learned->width, learned->height, xy, n, dec, err, s);
         if (e == cudaSuccess) {
-            compare_kernel<<<1024, 256, 0, s>>>(static_cast<const uint2 *>(ref->blocks), ref->width / 4, ref->width,
-                                                ref->height, dec, st, n, sse, mx);
-            e = cudaGetLastError();
+            e = launch_plain(compare_kernel, 1024, 256, 0, s, static_cast<const uint2 *>(ref->blocks), ref->width / 4,
+                             ref->width, ref->height, dec, st, n, sse, mx);
         }
     }
     double h_sse = 0.0;
