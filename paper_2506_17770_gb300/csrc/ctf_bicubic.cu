@@ -64,38 +64,6 @@ __device__ __forceinline__ int pick_tap(const float w[4], float xi, float &g) {
     return i;
 }
 
-// List Merge of a tile whose bounding box is larger than 16 x 16 texels:
-// list_union of ctf_select.cuh for the 16 taps of the 4x4 footprint at
-// (ox, oy).  Returns the number of distinct texels (budget + 1 when there are
-// more); byte c of src[r] is the list index of tap (c, r), (qx, qy) texel
-// `lane` of the list.
-__device__ __forceinline__ int list_union16(bool active, int ox, int oy, int budget, int lane, uint32_t src[4], int &qx,
-                                            int &qy) {
-    uint32_t left = active ? 0xFFFFu : 0u;
-    int n = 0;
-#pragma unroll
-    for (int r = 0; r < 4; ++r) src[r] = 0;
-    while (true) {  // at most budget + 1 <= 33 iterations
-        const uint32_t any = __ballot_sync(FULL, left != 0);
-        if (any == 0) return n;
-        if (n == budget) return budget + 1;
-        const int from = __ffs(any) - 1, k = __ffs(left) - 1;
-        const int x = __shfl_sync(FULL, ox + (k & 3), from), y = __shfl_sync(FULL, oy + ((k >> 2) & 3), from);
-#pragma unroll
-        for (int t = 0; t < 16; ++t) {
-            if (((left >> t) & 1u) && ox + (t & 3) == x && oy + (t >> 2) == y) {
-                src[t >> 2] |= (uint32_t)n << (8 * (t & 3));
-                left &= ~(1u << t);
-            }
-        }
-        if (lane == n) {
-            qx = x;
-            qy = y;
-        }
-        ++n;
-    }
-}
-
 // What bounds it: instructions issued.  A 1920x1080 Mask view with Catmull-Rom,
 // magnified 1 to 32 times: 46.4 us with a 64-bit division a tile, the inputs
 // loaded when they are needed, a rank per tap and a mask word per footprint
@@ -205,8 +173,8 @@ __global__ void __launch_bounds__(kThreads, 4) bicubic_filter_kernel(const Exact
         int n = 0, minx = 0, miny = 0, bw = 0, bh = 0, mcls = 0;
         uint32_t word = 0;            // a mask of one word (mcls 1); else lane w holds word w
         int before = 0;               // and the number of bits in the words before it
-        uint32_t lsrc[4];             // List Merge with a larger box: list indices of the taps,
-        int qlx = 0, qly = 0;         // texel `lane`
+        ListUnion<4> lu;              // List Merge with a larger box (mcls 4)
+        uint32_t lsrc[4];             // List Merge: list indices of the taps, four a word
         if (ALG >= ALG_LIST) {
             mini = __any_sync(FULL, ps.active && is_minified(in.jac, fW, fH));
             if (!mini) {
@@ -255,7 +223,10 @@ __global__ void __launch_bounds__(kThreads, 4) bicubic_filter_kernel(const Exact
                         fits = n <= p.budget;
                     } else if (ALG == ALG_LIST) {
                         mcls = 4;
-                        n = list_union16(ps.active, ox, oy, p.budget, lane, lsrc, qlx, qly);
+                        lu = list_union<4, false>(ps.active, ox, oy, p.budget, lane, lt, ranks, p.err);
+                        n = lu.n;
+#pragma unroll
+                        for (int r = 0; r < 4; ++r) lsrc[r] = lu.idx[r];
                         fits = n <= p.budget;
                     }
                 }
@@ -345,8 +316,8 @@ __global__ void __launch_bounds__(kThreads, 4) bicubic_filter_kernel(const Exact
             }
             __syncwarp();
         } else if (lane < n) {  // the list's order
-            qx = qlx;
-            qy = qly;
+            qx = lu.tx;
+            qy = lu.ty;
         }
         if (ALG == ALG_LIST && mcls != 4) {
 #pragma unroll

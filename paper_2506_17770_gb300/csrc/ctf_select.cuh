@@ -82,51 +82,88 @@ struct Selection {
 };
 
 // List Merge of a tile whose bounding box is wider or higher than 16 texels
-// (it spans an edge between surfaces; a magnified tile of one surface stays
-// below 14): the exact union, one distinct texel per iteration.  The lowest
-// lane with a tap left offers its first one, every lane marks its equal taps
-// with the texel's index n, and lane n mod 32 keeps the texel.
+// (it spans edges between surfaces; a magnified tile of one surface stays
+// below 14): the exact union by classes.  A footprint of kSide x kSide texels
+// holds one texel of each class of coordinates modulo kSide, so the distinct
+// texels are those of every class together, and within a class the pixels
+// that share a texel find one another by __match_any_sync.  The first of them
+// stands for the texel in the list.  A tile leaves with the class that takes
+// it over budget.
+// 1920x1080 block views whose tiles see 2 to 32 spots, us: 37 to 62, with two
+// texels per lane 44 to 91, with Catmull-Rom 43 to 65 (16 texels a pixel).
+// One texel a turn took 94 to 120, 115 to 243 and 457, a hash table in shared
+// memory 60 to 75, 66 to 103 and 66 to 104; cells of 8 x 4 texels in turn 52
+// to 83, 59 to 120 and 44 to 51.
+template <int kSide>
 struct ListUnion {
-    int n;                   // distinct texels, or budget + 1 when there are more
-    uint32_t idx;            // list index of tap k in byte k
-    int tx, ty, tx2, ty2;    // texels lane and lane + 32 of the list
+    int n;                            // distinct texels, or budget + 1 when there are more
+    uint32_t idx[kSide * kSide / 4];  // list index of tap k in byte k & 3 of word k >> 2
+    int tx, ty, tx2, ty2;             // texels lane and (kTwo) lane + 32 of the list
 };
 
-__device__ __forceinline__ ListUnion list_union(bool active, int ulx, int uly, int budget, int lane) {
-    ListUnion u;
-    u.n = 0;
-    u.idx = 0;
-    u.tx = u.tx2 = ulx;
-    u.ty = u.ty2 = uly;
-    uint32_t left = active ? 15u : 0u;  // taps without an index yet
-    while (true) {                      // at most budget + 1 <= 65 iterations
-        const uint32_t any = __ballot_sync(FULL, left != 0);
-        if (any == 0) return u;
-        if (u.n == budget) {
-            u.n = budget + 1;
-            return u;
-        }
-        const int src = __ffs(any) - 1, k = __ffs(left) - 1;
-        const int qx = __shfl_sync(FULL, ulx + (k & 1), src), qy = __shfl_sync(FULL, uly + ((k >> 1) & 1), src);
-        const int ex = qx - ulx, ey = qy - uly;
-        if (((ex | ey) & ~1) == 0) {  // both 0 or 1: one of this lane's taps
-            const int t = ex + 2 * ey;
-            if ((left >> t) & 1u) {
-                u.idx |= (uint32_t)u.n << (8 * t);
-                left &= ~(1u << t);
+template <int kSide, bool kTwo>
+__device__ __forceinline__ ListUnion<kSide> list_union(bool active, int ox, int oy, int budget, int lane, uint32_t lt,
+                                                       int *ranks, int *err) {
+    constexpr int kRanksN = kTwo ? 64 : 32;  // rank slots the caller provides
+    constexpr int kWords = kSide * kSide / 4;
+    static_assert(kSide == 2 || kSide == 4, "classes by the low bits of a coordinate");
+    ListUnion<kSide> u;
+    uint32_t by_class[kWords];  // list index of the pixel's texel of class (cx, cy) in byte cx + kSide * cy
+#pragma unroll
+    for (int w = 0; w < kWords; ++w) u.idx[w] = by_class[w] = 0;
+    u.tx = u.tx2 = ox;
+    u.ty = u.ty2 = oy;
+    int n = 0;
+#pragma unroll
+    for (int cy = 0; cy < kSide; ++cy) {
+        const int y = oy + ((cy - oy) & (kSide - 1));
+#pragma unroll 1
+        for (int cx = 0; cx < kSide; ++cx) {
+            const int x = ox + ((cx - ox) & (kSide - 1));
+            // (an active pixel's key never has all bits set: |x| is below 2^23)
+            const unsigned long long key =
+                active ? ((unsigned long long)(uint32_t)y << 32) | (uint32_t)(x ^ INT_MIN) : ~0ull;
+            const uint32_t same = __match_any_sync(FULL, key);
+            const bool first = active && (same & lt) == 0;
+            const uint32_t firsts = __ballot_sync(FULL, first);
+            // the firsts before this pixel's first
+            const int i = n + __popc(firsts & ((same & (0u - same)) - 1u));
+            n += __popc(firsts);
+            if (n > budget) {
+                u.n = budget + 1;
+                return u;
             }
+            const int c = cx + kSide * cy;
+            by_class[c >> 2] |= (uint32_t)i << (8 * (c & 3));
+            if (first) ranks[ck(i, kRanksN, err, kBndRanks)] = 32 * c + lane;
         }
-        if (lane == (u.n & 31)) {
-            if (u.n < 32) {
-                u.tx = qx;
-                u.ty = qy;
-            } else {
-                u.tx2 = qx;
-                u.ty2 = qy;
-            }
-        }
-        ++u.n;
     }
+    u.n = n;
+    __syncwarp();
+    // from classes to taps: byte c of a row of taps is class (ox + c) mod kSide
+    if (kSide == 2) {
+        u.idx[0] = __byte_perm(by_class[0], 0u, 0x3210u ^ ((ox & 1) ? 0x1111u : 0u) ^ ((oy & 1) ? 0x2222u : 0u));
+    } else {
+#pragma unroll
+        for (int r = 0; r < kSide; ++r) {
+            const int cy = (oy + r) & 3;
+            const uint32_t w = cy < 2 ? (cy == 0 ? by_class[0] : by_class[1 % kWords])
+                                      : (cy == 2 ? by_class[2 % kWords] : by_class[3 % kWords]);
+            u.idx[r % kWords] = __byte_perm(w, 0u, 0x32103210u >> (4 * (ox & 3)));
+        }
+    }
+    // the texel of list index i: class and first pixel are filed there
+    auto texel = [&](int i, int &x, int &y) {
+        const int f = i < n ? ranks[ck(i, kRanksN, err, kBndRanks)] : lane;
+        x = __shfl_sync(FULL, ox, f & 31);
+        y = __shfl_sync(FULL, oy, f & 31);
+        x += ((f >> 5) - x) & (kSide - 1);
+        y += ((f >> 5) / kSide - y) & (kSide - 1);
+    };
+    texel(lane, u.tx, u.ty);
+    if (kTwo) texel(lane + 32, u.tx2, u.ty2);
+    __syncwarp();  // rank slots free again
+    return u;
 }
 
 // Step 1 for the collaborative algorithms (ALG >= ALG_LIST) and the STF
@@ -176,7 +213,7 @@ __device__ __forceinline__ Selection select_tile(const ExactParams &p, const Pix
     int n = 0, minx = 0, miny = 0, bw = 0, mcls = 0;
     uint32_t Bw[NW];  // mask words and their prefix popcounts, set (and read) per size class
     int pre[NW];
-    ListUnion lu;     // List Merge with a larger box (mcls 4)
+    ListUnion<2> lu;  // List Merge with a larger box (mcls 4)
     if (ALG >= ALG_LIST) {
         mini = __any_sync(FULL, ps.active && is_minified(jac, fW, fH));
         if (!mini) {
@@ -223,7 +260,7 @@ __device__ __forceinline__ Selection select_tile(const ExactParams &p, const Pix
                     fits = n <= p.budget;
                 } else if (ALG == ALG_LIST) {
                     mcls = 4;
-                    lu = list_union(ps.active, ps.ulx, ps.uly, p.budget, lane);
+                    lu = list_union<2, kTwo>(ps.active, ps.ulx, ps.uly, p.budget, lane, lt, ranks, p.err);
                     n = lu.n;
                     fits = n <= p.budget;
                 }
@@ -319,7 +356,7 @@ __device__ __forceinline__ Selection select_tile(const ExactParams &p, const Pix
                 __syncwarp();
             } else {  // the list's order
 #pragma unroll
-                for (int k = 0; k < 4; ++k) j[k] = (int)((lu.idx >> (8 * k)) & 63u);
+                for (int k = 0; k < 4; ++k) j[k] = (int)((lu.idx[0] >> (8 * k)) & 63u);
                 sel.produce = lane < n;
                 sel.produce2 = lane + 32 < n;
                 sel.tx = lu.tx;
@@ -425,7 +462,7 @@ __device__ __forceinline__ Selection select_tile(const ExactParams &p, const Pix
                 __syncwarp();
             } else {
 #pragma unroll
-                for (int k = 0; k < 4; ++k) j[k] = (int)((lu.idx >> (8 * k)) & 31u);
+                for (int k = 0; k < 4; ++k) j[k] = (int)((lu.idx[0] >> (8 * k)) & 31u);
                 lu.tx = __shfl_sync(FULL, lu.tx, my_i & 31);  // texel my_i of the list
                 lu.ty = __shfl_sync(FULL, lu.ty, my_i & 31);
             }
