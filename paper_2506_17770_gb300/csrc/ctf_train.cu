@@ -1234,8 +1234,18 @@ int ctf_trainer_step(ctf_trainer t, int64_t steps, void *stream) {
         r.inv_bc2 = (float)(1.0 / bc2);
         return r;
     };
+    // A captured call runs whenever its graph does, after other replays and
+    // calls: its segments count from zero in cells that it clears itself.
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    uint32_t seen_steps = t->seen_steps;
     if (steps > 0) {
-        const cudaError_t e = launch_pack(g, s);
+        cudaError_t e = cudaStreamIsCapturing(s, &capture);
+        if (e != cudaSuccess) cudaGetLastError();
+        if (e == cudaSuccess && capture != cudaStreamCaptureStatusNone) {
+            seen_steps = 0;
+            e = cudaMemsetAsync(t->seen, 0, (t->nparams - kOffLat) / 8 * 4, s);
+        }
+        if (e == cudaSuccess) e = launch_pack(g, s);
         if (e != cudaSuccess) return report_cuda(e, "training step");
     }
     // Segments of equal length, to one step; of one step where a step's texels
@@ -1247,7 +1257,7 @@ int ctf_trainer_step(ctf_trainer t, int64_t steps, void *stream) {
     const int64_t longest = 64ll * g.n > (int64_t)(t->nparams - kOffLat) ? 1 : kSegment;
     for (int64_t left = (steps + longest - 1) / longest, k = 0; k < steps; --left) {
         const int len = (int)((steps - k + left - 1) / left);
-        a.base = t->seen_steps;
+        a.base = seen_steps;
         for (int j = 0; j < len; ++j) a.st[j] = adam_step(t->step + j);
         cudaError_t e = cudaSuccess;
         if (a.base > 0xffffff00u) {
@@ -1271,7 +1281,9 @@ int ctf_trainer_step(ctf_trainer t, int64_t steps, void *stream) {
         }
         if (e != cudaSuccess) return report_cuda(e, "training step");
         t->step += len;
-        t->seen_steps = a.base + (uint32_t)len;
+        seen_steps = a.base + (uint32_t)len;
+        // (the marks that a captured call leaves lie below either count)
+        t->seen_steps = capture == cudaStreamCaptureStatusNone ? seen_steps : std::max(t->seen_steps, seen_steps);
         k += len;
     }
     return CTF_OK;
