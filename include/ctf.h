@@ -365,7 +365,11 @@ typedef struct ctf_trainer_s *ctf_trainer;
 int ctf_trainer_create(ctf_texture exact_src, const ctf_train_desc *desc, ctf_trainer *out);
 int ctf_trainer_destroy(ctf_trainer tr);
 
-/* Run `steps` optimisation steps on the stream (asynchronous). */
+/* Run `steps` optimisation steps on the stream (asynchronous).  A launch that
+ * the runtime refuses ends the call with CTF_ERR_CUDA; a step that was begun
+ * by then is completed, and counted with those before it, by the next call
+ * that reads or changes the trainer.  Captured into a graph, every replay takes
+ * the captured steps again. */
 int ctf_trainer_step(ctf_trainer tr, int64_t steps, void *stream);
 
 /* Steps taken so far. */

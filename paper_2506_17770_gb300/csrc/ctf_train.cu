@@ -1006,6 +1006,11 @@ struct ctf_trainer_s {
     unsigned char *wimg = nullptr;  // FP16 weight operands of the gradient kernel
     float *partial = nullptr;       // per-CTA weight-gradient sums of the gradient kernel
     int64_t step = 0;
+    // a segment that a refused launch cut short (finish_segment): its step whose
+    // launches are not all queued, or -1; whether the gradients are; its base
+    int open = -1;
+    bool open_grad = false;
+    uint32_t open_base = 0;
 };
 
 namespace ctf {
@@ -1078,6 +1083,75 @@ cudaError_t launch_grad(const GradParams &g, int ctas, cudaStream_t s) {
 
 cudaError_t launch_pack(const GradParams &g, cudaStream_t s) {
     return launch_plain(pack_kernel, (kPackThreads + 255) / 256, 256, 0, s, g.params, g.wimg);
+}
+
+// A step's gradients, and their split over CTAs.
+GradParams step_grad_params(const ctf_trainer_s *t, int &ctas) {
+    GradParams g = grad_params(t);
+    g.n = t->desc.batch;
+    g.dscale = 2.0f / (float)t->desc.batch;
+    ctas = split_batch(g);
+    return g;
+}
+
+AdamParams adam_params(const ctf_trainer_s *t, const GradParams &g, int ctas) {
+    AdamParams a;
+    a.params = t->params;
+    a.m = t->m;
+    a.v = t->v;
+    a.grad = t->grad;
+    a.n = t->nparams;
+    a.beta1 = t->desc.beta1;
+    a.beta2 = t->desc.beta2;
+    a.eps = t->desc.eps;
+    a.partial = t->partial;
+    a.ctas = ctas;
+    a.dscale = (double)g.dscale;
+    a.wimg = t->wimg;
+    a.seen = t->seen;
+    return a;
+}
+
+AdamStep adam_step(const ctf_trainer_s *t, int64_t st) {
+    const double frac = std::fmin(1.0, (double)st / (double)t->desc.total_steps);
+    const double sched = 1.0 - (1.0 - t->desc.lr_final_frac) * frac;
+    const double bc1 = 1.0 - std::pow((double)t->desc.beta1, (double)(st + 1));
+    const double bc2 = 1.0 - std::pow((double)t->desc.beta2, (double)(st + 1));
+    AdamStep r;
+    r.w = (float)(t->desc.lr_weights * sched / bc1);
+    r.lat = (float)(t->desc.lr_latents * sched / bc1);
+    r.inv_bc2 = (float)(1.0 / bc2);
+    return r;
+}
+
+// A launch refused inside a segment leaves the weights and some cells steps
+// ahead of the others.  Every call that reads or changes the trainer first ends
+// such a segment with the step that was refused: its gradients, if they are
+// not queued yet, and a sweep.  The steps count from then on.  If that is refused
+// too, the trainer stays as it was.
+int finish_segment(ctf_trainer_s *t, cudaStream_t s) {
+    if (t->open < 0) return CTF_OK;
+    int ctas = 0;
+    GradParams g = step_grad_params(t, ctas);
+    AdamParams a = adam_params(t, g, ctas);
+    a.base = t->open_base;
+    a.j = t->open;
+    for (int j = 0; j <= t->open; ++j) a.st[j] = adam_step(t, t->step + j);
+    a.descending = 0;
+    g.step = (uint32_t)(t->step + t->open);
+    cudaError_t e = cudaSuccess;
+    if (!t->open_grad) {  // (after a plain launch, so after everything before it)
+        e = launch_pack(g, s);
+        if (e == cudaSuccess) e = launch_grad(g, ctas, s);
+        t->open_grad = e == cudaSuccess;
+    }
+    if (e == cudaSuccess)
+        e = launch_plain(sweep_kernel, device_sm_count() * kSweepCtasPerSm, kSweepThreads, 0, s, a);
+    if (e != cudaSuccess) return report_cuda(e, "finishing a training segment");
+    t->step += t->open + 1;
+    t->seen_steps = t->open_base + (uint32_t)t->open + 1;
+    t->open = -1;
+    return CTF_OK;
 }
 
 int check_desc(const ctf_train_desc *d) {
@@ -1205,35 +1279,9 @@ int ctf_trainer_step(ctf_trainer t, int64_t steps, void *stream) {
     if (!t) return report(CTF_ERR_ARG, "trainer is NULL");
     if (steps < 0) return report(CTF_ERR_ARG, "negative step count");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    GradParams g = grad_params(t);
-    g.n = t->desc.batch;
-    g.dscale = 2.0f / (float)t->desc.batch;
-    const int ctas = split_batch(g);
-    AdamParams a;
-    a.params = t->params;
-    a.m = t->m;
-    a.v = t->v;
-    a.grad = t->grad;
-    a.n = t->nparams;
-    a.beta1 = t->desc.beta1;
-    a.beta2 = t->desc.beta2;
-    a.eps = t->desc.eps;
-    a.partial = t->partial;
-    a.ctas = ctas;
-    a.dscale = (double)g.dscale;
-    a.wimg = t->wimg;
-    a.seen = t->seen;
-    auto adam_step = [&](int64_t st) {
-        const double frac = std::fmin(1.0, (double)st / (double)t->desc.total_steps);
-        const double sched = 1.0 - (1.0 - t->desc.lr_final_frac) * frac;
-        const double bc1 = 1.0 - std::pow((double)t->desc.beta1, (double)(st + 1));
-        const double bc2 = 1.0 - std::pow((double)t->desc.beta2, (double)(st + 1));
-        AdamStep r;
-        r.w = (float)(t->desc.lr_weights * sched / bc1);
-        r.lat = (float)(t->desc.lr_latents * sched / bc1);
-        r.inv_bc2 = (float)(1.0 / bc2);
-        return r;
-    };
+    int ctas = 0;
+    GradParams g = step_grad_params(t, ctas);
+    AdamParams a = adam_params(t, g, ctas);
     // A captured call runs whenever its graph does, after other replays and
     // calls: its segments count from zero in cells that it clears itself.
     cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
@@ -1242,8 +1290,15 @@ int ctf_trainer_step(ctf_trainer t, int64_t steps, void *stream) {
         cudaError_t e = cudaStreamIsCapturing(s, &capture);
         if (e != cudaSuccess) cudaGetLastError();
         if (e == cudaSuccess && capture != cudaStreamCaptureStatusNone) {
+            if (t->open >= 0)
+                return report(CTF_ERR_UNSUPPORTED, "steps cut short by a refused launch are finished outside a capture");
             seen_steps = 0;
             e = cudaMemsetAsync(t->seen, 0, (t->nparams - kOffLat) / 8 * 4, s);
+        }
+        if (e == cudaSuccess && t->open >= 0) {
+            const int rc = finish_segment(t, s);
+            if (rc) return rc;
+            seen_steps = t->seen_steps;
         }
         if (e == cudaSuccess) e = launch_pack(g, s);
         if (e != cudaSuccess) return report_cuda(e, "training step");
@@ -1258,7 +1313,7 @@ int ctf_trainer_step(ctf_trainer t, int64_t steps, void *stream) {
     for (int64_t left = (steps + longest - 1) / longest, k = 0; k < steps; --left) {
         const int len = (int)((steps - k + left - 1) / left);
         a.base = seen_steps;
-        for (int j = 0; j < len; ++j) a.st[j] = adam_step(t->step + j);
+        for (int j = 0; j < len; ++j) a.st[j] = adam_step(t, t->step + j);
         cudaError_t e = cudaSuccess;
         if (a.base > 0xffffff00u) {
             e = cudaMemsetAsync(t->seen, 0, (t->nparams - kOffLat) / 8 * 4, s);
@@ -1269,14 +1324,20 @@ int ctf_trainer_step(ctf_trainer t, int64_t steps, void *stream) {
             g.mark = j == 0 ? a.base + 1u : 0u;
             a.j = j;
             e = launch_grad(g, ctas, s);
-            if (e != cudaSuccess) break;
-            if (j + 1 < len) {
+            const bool grad = e == cudaSuccess;
+            if (grad && j + 1 < len) {
                 const long long need = (16ll * g.n + kAdvThreads - 1) / kAdvThreads, cap = 8ll * sms * kAdvCtasPerSm;
                 const long long grid = std::max<long long>(std::min(need, cap), (kWeights + kRedEntries - 1) / kRedEntries);
                 e = launch_dependent(advance_kernel, (int)grid, kAdvThreads, 0, s, g, a);
-            } else {
+            } else if (grad) {
                 a.descending = (int)(left & 1);
                 e = launch_dependent(sweep_kernel, sms * kSweepCtasPerSm, kSweepThreads, 0, s, a);
+            }
+            // (of a capture that fails nothing will run)
+            if (e != cudaSuccess && (grad || j > 0) && capture == cudaStreamCaptureStatusNone) {
+                t->open = j;
+                t->open_grad = grad;
+                t->open_base = a.base;
             }
         }
         if (e != cudaSuccess) return report_cuda(e, "training step");
@@ -1296,6 +1357,8 @@ int ctf_trainer_gradients(ctf_trainer t, const int32_t *xy, int n, double *loss,
     if (!t) return report(CTF_ERR_ARG, "trainer is NULL");
     if (n < 1 || !xy) return report(CTF_ERR_ARG, "need n >= 1 texels");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
+    const int rc = finish_segment(t, s);
+    if (rc) return rc;
     GradParams g = grad_params(t);
     g.xy = reinterpret_cast<const int2 *>(xy);
     g.n = n;
@@ -1339,6 +1402,8 @@ int ctf_trainer_get_params(ctf_trainer t, const ctf_mlp_arrays *out) {
     layout(t, off, cnt);
     arrays_of(out, p);
     cudaDeviceSynchronize();
+    const int rc = finish_segment(t, nullptr);
+    if (rc) return rc;
     for (int i = 0; i < 8; ++i)
         if (p[i]) {
             cudaError_t e = cudaMemcpy(p[i], t->params + off[i], cnt[i] * 4, cudaMemcpyDefault);
@@ -1356,6 +1421,8 @@ int ctf_trainer_set_params(ctf_trainer t, const ctf_mlp_arrays *in) {
     layout(t, off, cnt);
     arrays_of(in, p);
     cudaDeviceSynchronize();
+    const int rc = finish_segment(t, nullptr);
+    if (rc) return rc;
     for (int i = 0; i < 8; ++i)
         if (p[i]) {
             cudaError_t e = cudaMemcpy(t->params + off[i], p[i], cnt[i] * 4, cudaMemcpyDefault);
@@ -1368,6 +1435,11 @@ int ctf_trainer_export(ctf_trainer t, ctf_eval_mode mode, ctf_texture *out) {
     using namespace ctf;
     clear_error();
     if (!t || !out) return report(CTF_ERR_ARG, "trainer and out must not be NULL");
+    if (t->open >= 0) {
+        cudaDeviceSynchronize();
+        const int rc = finish_segment(t, nullptr);
+        if (rc) return rc;
+    }
     ctf_mlp_desc d;
     std::memset(&d, 0, sizeof(d));
     d.width = t->Wt;
@@ -1411,6 +1483,8 @@ int ctf_trainer_save(ctf_trainer t, const char *path) {
     clear_error();
     if (!t || !path) return report(CTF_ERR_ARG, "trainer and path must not be NULL");
     cudaDeviceSynchronize();
+    const int rc = finish_segment(t, nullptr);
+    if (rc) return rc;
     std::vector<float> buf(3 * t->nparams);
     cudaError_t e = cudaMemcpy(buf.data(), t->params, t->nparams * 4, cudaMemcpyDeviceToHost);
     if (e == cudaSuccess) e = cudaMemcpy(buf.data() + t->nparams, t->m, t->nparams * 4, cudaMemcpyDeviceToHost);

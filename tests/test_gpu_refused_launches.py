@@ -94,3 +94,50 @@ def test_hook_arguments_are_checked():
         with pytest.raises(_ctf.CtfError) as ei:
             _ctf.ctf_debug_fail_launches(n, skip=skip)
         assert ei.value.status == _ctf.CTF_ERR_ARG
+
+
+def _params(tr, desc):
+    p = _ctf.ctf_trainer_get_params(tr, desc)
+    return np.concatenate([np.asarray(p[k], np.float32).ravel() for k in sorted(p)]).view(np.uint32)
+
+
+@pytest.mark.parametrize("after", ["params", "step", "save", "gradients", "twice"])
+def test_training_goes_on_after_a_refused_launch(textures, after, tmp_path):
+    """One launch of a call of 20 steps (two segments; a pack, then gradients
+    and an update a step) refused, for every launch: the trainer then stands at
+    the number of steps that it reports, bit for bit, and goes on from there."""
+    desc = _ctf.train_desc(((16, 16), (8, 8)), batch=30, total_steps=60)
+    tr = _ctf.ctf_trainer_create(textures[0], desc)
+    want = [_params(tr, desc)]
+    for _ in range(30):
+        _ctf.ctf_trainer_step(tr, 1)
+        want.append(_params(tr, desc))
+    _ctf.ctf_trainer_destroy(tr)
+    xy = torch.zeros((4, 2), dtype=torch.int32, device="cuda")
+    try:
+        for skip in range(41):
+            tr = _ctf.ctf_trainer_create(textures[0], desc)
+            _ctf.ctf_trainer_step(tr, 3)
+            _ctf.ctf_debug_fail_launches(2 if after == "twice" else 1, skip=skip)
+            with pytest.raises(_ctf.CtfError) as ei:
+                _ctf.ctf_trainer_step(tr, 20)
+            assert ei.value.status == _ctf.CTF_ERR_CUDA
+            if after == "twice" and skip % 20 > 1:  # (elsewhere nothing of a segment is begun)
+                with pytest.raises(_ctf.CtfError):
+                    _params(tr, desc)
+            _ctf.ctf_debug_fail_launches(0)
+            if after == "step":
+                _ctf.ctf_trainer_step(tr, 2)
+            elif after == "save":
+                _ctf.ctf_trainer_save(tr, str(tmp_path / "t"))
+                _ctf.ctf_trainer_destroy(tr)
+                tr = _ctf.ctf_trainer_load(textures[0], str(tmp_path / "t"))
+            elif after == "gradients":
+                _ctf.ctf_trainer_gradients(tr, desc, xy, 4)
+            assert np.array_equal(_params(tr, desc), want[_ctf.ctf_trainer_steps_done(tr)]), skip
+            assert _ctf.ctf_trainer_steps_done(tr) >= 3 + max(0, (skip - 1) // 2)
+            _ctf.ctf_trainer_step(tr, 4)
+            assert np.array_equal(_params(tr, desc), want[_ctf.ctf_trainer_steps_done(tr)]), skip
+            _ctf.ctf_trainer_destroy(tr)
+    finally:
+        _ctf.ctf_debug_fail_launches(0)
