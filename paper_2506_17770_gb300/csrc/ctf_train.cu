@@ -774,7 +774,7 @@ __device__ __forceinline__ void update_weights(const AdamParams &a, const AdamSt
 // reach a cell claims it.  Only cells that step j reads too (`late`) wait for
 // its gradients; the gradient kernel neither reads nor changes the others.
 // 4096^2 texture, 8,192 texels: 34 us a step in a call of 64 (gradients and
-// advance 29, a sixteenth of a sweep 6); 67 us in calls of one step, whose
+// advance 29, a sixteenth of a sweep 6); 66 us in calls of one step, whose
 // sweep moves every parameter, and 93 us with an Adam kernel of all cells and
 // five more launches a step.  Five CTAs per SM 36 us.
 constexpr int kAdvThreads = 256, kAdvCtasPerSm = 4;
@@ -838,8 +838,9 @@ __global__ void __launch_bounds__(kAdvThreads, kAdvCtasPerSm) advance_kernel(con
 // of the updates in long segments (94 us for 10.5 million parameters and 16
 // steps at 85% of the issue slots; 42 us would be the 24 bytes of each), by
 // those bytes in short ones, whose cells are walked up and down in turn so that
-// one starts with the cells that the last one left in L2 (one step: 85 us with
-// one direction, 71 with both).  Five or more CTAs per SM are slower by 3%.
+// a sweep starts with the cells that the last one left in L2 (4096^2 texture,
+// 8,192 texels, calls of one step: 78 us a step with one direction, 66 with
+// both).  Five or more CTAs per SM are slower by 3%.
 constexpr int kSweepThreads = 256, kSweepCtasPerSm = 4;
 __global__ void __launch_bounds__(kSweepThreads, kSweepCtasPerSm) sweep_kernel(const AdamParams a) {
     static_assert(kSweepThreads == kRedEntries * kRedRows, "the weight sums' thread layout");
@@ -1006,6 +1007,7 @@ struct ctf_trainer_s {
     unsigned char *wimg = nullptr;  // FP16 weight operands of the gradient kernel
     float *partial = nullptr;       // per-CTA weight-gradient sums of the gradient kernel
     int64_t step = 0;
+    uint32_t sweeps = 0;            // sweeps so far: every other one walks down
     // a segment that a refused launch cut short (finish_segment): its step whose
     // launches are not all queued, or -1; whether the gradients are; its base
     int open = -1;
@@ -1137,7 +1139,7 @@ int finish_segment(ctf_trainer_s *t, cudaStream_t s) {
     a.base = t->open_base;
     a.j = t->open;
     for (int j = 0; j <= t->open; ++j) a.st[j] = adam_step(t, t->step + j);
-    a.descending = 0;
+    a.descending = (int)(t->sweeps & 1u);
     g.step = (uint32_t)(t->step + t->open);
     cudaError_t e = cudaSuccess;
     if (!t->open_grad) {  // (after a plain launch, so after everything before it)
@@ -1148,6 +1150,7 @@ int finish_segment(ctf_trainer_s *t, cudaStream_t s) {
     if (e == cudaSuccess)
         e = launch_plain(sweep_kernel, device_sm_count() * kSweepCtasPerSm, kSweepThreads, 0, s, a);
     if (e != cudaSuccess) return report_cuda(e, "finishing a training segment");
+    ++t->sweeps;
     t->step += t->open + 1;
     t->seen_steps = t->open_base + (uint32_t)t->open + 1;
     t->open = -1;
@@ -1330,8 +1333,9 @@ int ctf_trainer_step(ctf_trainer t, int64_t steps, void *stream) {
                 const long long grid = std::max<long long>(std::min(need, cap), (kWeights + kRedEntries - 1) / kRedEntries);
                 e = launch_dependent(advance_kernel, (int)grid, kAdvThreads, 0, s, g, a);
             } else if (grad) {
-                a.descending = (int)(left & 1);
+                a.descending = (int)(t->sweeps & 1u);
                 e = launch_dependent(sweep_kernel, sms * kSweepCtasPerSm, kSweepThreads, 0, s, a);
+                if (e == cudaSuccess) ++t->sweeps;
             }
             // (of a capture that fails nothing will run)
             if (e != cudaSuccess && (grad || j > 0) && capture == cudaStreamCaptureStatusNone) {
