@@ -343,6 +343,7 @@ const char *bounds_site_name(int site) {
     case kBndLane: return "a shuffle's source lane";
     case kBndBatch: return "a batch plan";
     case kBndTrain: return "the trainer's buffers";
+    case kBndDecodeList: return "a list of texels to decode";
     case kBndSelfTest: return "the self-test";
     default: return "an unknown site";
     }

@@ -30,6 +30,7 @@ enum BoundsSite {
     kBndLane,          // a source lane of a shuffle (n = 32)
     kBndBatch,         // a view or tile of a batch plan
     kBndTrain,         // a texel, cell or partial sum of the trainer
+    kBndDecodeList,    // the texel list and the outputs of ctf_mlp_decode
     kBndSelfTest,      // ctf_debug_selftest_bounds
     kBndNumSites
 };

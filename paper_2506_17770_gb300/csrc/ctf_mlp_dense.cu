@@ -181,10 +181,10 @@ __global__ void __launch_bounds__(kPThreads, kPCtasPerSm)
                 if (!ok) break;
                 if (kTap) {
                     // (chain c's values overlay operand rows of chain 0, which has been read)
-                    outrow[kRows * c + tid] = v;
+                    outrow[ck(kRows * c + tid, kDRows, a.err, kBndRow)] = v;
                 } else {
                     const long long row = grp * kDRows + kRows * c + tid;
-                    if (row < a.n) a.out[row] = v;
+                    if (row < a.n) a.out[ck(row, a.n, a.err, kBndDecodeList)] = v;
                 }
                 ok = !bar_or<1, kRows>(bad);
                 if (!ok && tid == 0) atomicExch(a.err, CTF_ERR_TIMEOUT);
@@ -203,7 +203,7 @@ __global__ void __launch_bounds__(kPThreads, kPCtasPerSm)
                         float2 rg = make_float2(0.f, 0.f), ba = make_float2(0.f, 0.f);
 #pragma unroll
                         for (int k = 0; k < 4; ++k) {
-                            const float4 t = outrow[kRows * warp + 32 * k + lane];
+                            const float4 t = outrow[ck(kRows * warp + 32 * k + lane, kDRows, a.err, kBndRow)];
                             const float2 wk = make_float2(w[k], w[k]);
                             rg = __ffma2_rn(wk, make_float2(t.x, t.y), rg);
                             ba = __ffma2_rn(wk, make_float2(t.z, t.w), ba);
@@ -269,7 +269,7 @@ __global__ void __launch_bounds__(kPThreads, kPCtasPerSm)
                     const int r = kRows * c + 32 * pw + lane;
                     const long long i = grp * kDRows + r;
                     if (i >= a.n) break;
-                    const int2 t = a.xy[i];
+                    const int2 t = a.xy[ck(i, a.n, a.err, kBndDecodeList)];
                     float f[kMlpIn];
                     texel_features(m, min(max(t.x, 0), a.Wt - 1), min(max(t.y, 0), a.Ht - 1), f);
                     store_x_row_at(st + kDX, r, f, kFp8, inv_a1);

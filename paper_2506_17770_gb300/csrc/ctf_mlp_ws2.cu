@@ -493,7 +493,8 @@ __device__ __forceinline__ void p_gather(const ExactParams &p, uint32_t off, int
             for (int k = 0; k < 4; ++k) {
                 // (paired taps: the odd one is the next row)
                 const bool next = p_tap_pairs<ALG>() && (k & 1);
-                const float4 t = outrow[row_of((info >> (kIdxBits * (next ? k - 1 : k))) & kIdxMask) + (next ? 1 : 0)];
+                const float4 t = outrow[ck(row_of((info >> (kIdxBits * (next ? k - 1 : k))) & kIdxMask) + (next ? 1 : 0),
+                                           kPGroupRows, p.err, kBndRow)];
                 const float2 wk = make_float2(w[k], w[k]);
                 rg = __ffma2_rn(wk, make_float2(t.x, t.y), rg);
                 ba = __ffma2_rn(wk, make_float2(t.z, t.w), ba);
