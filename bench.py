@@ -167,7 +167,7 @@ def kernel_source_hash(files):
 
 EXACT_SOURCES = ("ctf_filter.cu", "ctf_device.cuh", "ctf_exact_tile.cuh", "ctf_select.cuh")
 LEARNED_SOURCES = ("ctf_mlp_ws2.cu", "ctf_mlp_chain.cuh", "ctf_mlp.cuh", "ctf_device.cuh", "ctf_select.cuh",
-                   "tc_ops.cuh")
+                   "ctf_exact_tile.cuh", "tc_ops.cuh")
 
 
 def ncu_traffic(key: str, sources):
