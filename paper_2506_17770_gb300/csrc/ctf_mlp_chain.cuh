@@ -479,14 +479,14 @@ __device__ __forceinline__ bool mlp_warp_tile(const ExactParams &p, const MlpDev
     return true;
 }
 
-// One iteration of the learned-decode filter for the collaborative
-// algorithms and STF.  The CTA's 4 warps run step 1 on two pixel tiles each
-// (slots g = warp and g = 4 + warp of the group of 8 tiles from `first`); the
-// texel lists of the 8 tiles are packed into consecutive rows in slot order
-// and decoded by as few 128-row chains as they fill (none for an empty
-// group), and every pixel then gathers its taps from the rows.  Which thread
-// computes a texel does not change its value: the rows of an MMA are
-// independent.  Returns false (for every thread alike) if a chain gave up.
+// One iteration of the learned-decode filter with group_dedup.  The CTA's 4
+// warps run step 1 on two pixel tiles each (slots g = warp and g = 4 + warp of
+// the group of 8 tiles from `first`); the distinct texels of the 8 tiles are
+// packed into consecutive rows and decoded by as few 128-row chains as they
+// fill (none for an empty group), and every pixel then gathers its taps from
+// the rows.  Which thread computes a texel does not change its value: the rows
+// of an MMA are independent.  Returns false (for every thread alike) if a chain
+// gave up.
 template <int ALG, int TW, int MD>
 __device__ __forceinline__ bool mlp_group(const ExactParams &p, const MlpDevice &m, Chain &ch, long long first,
                                           int lane, uint32_t lt, Counters &cnt, const float *inv_a1,
@@ -556,96 +556,67 @@ __device__ __forceinline__ bool mlp_group(const ExactParams &p, const MlpDevice 
     }
     __syncthreads();
 
-    // ---- rows.  Without group_dedup slot g owns rows [base_g, base_g +
-    // count[g]) in slot order.  With it, the distinct texels of the group
-    // get rows in the order their first lists entries win a shared hash
-    // table, and rowmap sends every list entry to its texel's row.  Every
-    // thread then reads the texels of its rows (threadIdx.x and 128 +
-    // threadIdx.x) before the first chain overwrites the X buffer that holds
-    // the lists.
+    // ---- rows: the distinct texels of the group get rows in the order their
+    // first list entries win a shared hash table, and rowmap sends every list
+    // entry to its texel's row.  Every thread then reads the texels of its rows
+    // (threadIdx.x and 128 + threadIdx.x) before the first chain overwrites the
+    // X buffer that holds the lists.
     int cnts[kGroupTiles];
 #pragma unroll
     for (int g = 0; g < kGroupTiles; ++g) cnts[g] = count[g];
-    int R = 0, my_base[2] = {0, 0};
     int2 xy[2] = {make_int2(0, 0), make_int2(0, 0)};
     unsigned char *rowmap = sm + kSmRowMap;
-    if (p.group_dedup) {  // CTA-uniform
-        unsigned long long *hkey = reinterpret_cast<unsigned long long *>(sm + kSmHashKey);
-        unsigned char *hrow = sm + kSmHashRow;
-        int *nuniq = reinterpret_cast<int *>(sm + kSmNUnique);
-        for (int i = threadIdx.x; i < 512; i += kRows) hkey[i] = ~0ull;
-        if (threadIdx.x == 0) *nuniq = 0;
-        __syncthreads();
-        int slot[2] = {0, 0};
-        bool has[2] = {false, false}, won[2] = {false, false};
-        int2 t2[2] = {make_int2(0, 0), make_int2(0, 0)};
+    unsigned long long *hkey = reinterpret_cast<unsigned long long *>(sm + kSmHashKey);
+    unsigned char *hrow = sm + kSmHashRow;
+    int *nuniq = reinterpret_cast<int *>(sm + kSmNUnique);
+    for (int i = threadIdx.x; i < 512; i += kRows) hkey[i] = ~0ull;
+    if (threadIdx.x == 0) *nuniq = 0;
+    __syncthreads();
+    int slot[2] = {0, 0};
+    bool has[2] = {false, false}, won[2] = {false, false};
+    int2 t2[2] = {make_int2(0, 0), make_int2(0, 0)};
 #pragma unroll
-        for (int c = 0; c < 2; ++c) {
-            const int e = (int)threadIdx.x + kRows * c, g = e >> 5;
-            int n_g = cnts[0];
+    for (int c = 0; c < 2; ++c) {
+        const int e = (int)threadIdx.x + kRows * c, g = e >> 5;
+        int n_g = cnts[0];
 #pragma unroll
-            for (int k = 1; k < kGroupTiles; ++k) n_g = g == k ? cnts[k] : n_g;
-            if ((e & 31) < n_g) {
-                has[c] = true;
-                t2[c] = texlist[e];
-                const unsigned long long key = ((unsigned long long)(uint32_t)t2[c].y << 32) | (uint32_t)t2[c].x;
-                unsigned h = (((uint32_t)t2[c].x * 0x9E3779B1u) ^ ((uint32_t)t2[c].y * 0x85EBCA77u)) >> 23;
-                // at most 256 keys in 512 slots: the probe always ends
-                for (int probe = 0; probe < 512; ++probe) {
-                    const unsigned long long old = atomicCAS(&hkey[h], ~0ull, key);
-                    if (old == ~0ull || old == key) {
-                        won[c] = old == ~0ull;
-                        slot[c] = (int)h;
-                        break;
-                    }
-                    h = (h + 1) & 511u;
+        for (int k = 1; k < kGroupTiles; ++k) n_g = g == k ? cnts[k] : n_g;
+        if ((e & 31) < n_g) {
+            has[c] = true;
+            t2[c] = texlist[e];
+            const unsigned long long key = ((unsigned long long)(uint32_t)t2[c].y << 32) | (uint32_t)t2[c].x;
+            unsigned h = (((uint32_t)t2[c].x * 0x9E3779B1u) ^ ((uint32_t)t2[c].y * 0x85EBCA77u)) >> 23;
+            // at most 256 keys in 512 slots: the probe always ends
+            for (int probe = 0; probe < 512; ++probe) {
+                const unsigned long long old = atomicCAS(&hkey[h], ~0ull, key);
+                if (old == ~0ull || old == key) {
+                    won[c] = old == ~0ull;
+                    slot[c] = (int)h;
+                    break;
                 }
+                h = (h + 1) & 511u;
             }
         }
-        __syncthreads();
-        int2 *uxy = texlist;  // the lists have been read: the distinct texels reuse the space
+    }
+    __syncthreads();
+    int2 *uxy = texlist;  // the lists have been read: the distinct texels reuse the space
 #pragma unroll
-        for (int c = 0; c < 2; ++c) {
-            if (won[c]) {
-                const int row = ck(atomicAdd(nuniq, 1), 2 * kRows, p.err, kBndRow);
-                hrow[slot[c]] = (unsigned char)row;
-                uxy[row] = t2[c];
-            }
+    for (int c = 0; c < 2; ++c) {
+        if (won[c]) {
+            const int row = ck(atomicAdd(nuniq, 1), 2 * kRows, p.err, kBndRow);
+            hrow[slot[c]] = (unsigned char)row;
+            uxy[row] = t2[c];
         }
-        __syncthreads();
+    }
+    __syncthreads();
 #pragma unroll
-        for (int c = 0; c < 2; ++c)
-            if (has[c]) rowmap[threadIdx.x + kRows * c] = hrow[slot[c]];
-        R = *nuniq;
+    for (int c = 0; c < 2; ++c)
+        if (has[c]) rowmap[threadIdx.x + kRows * c] = hrow[slot[c]];
+    const int R = *nuniq;
 #pragma unroll
-        for (int c = 0; c < 2; ++c) {
-            const int row = kRows * c + (int)threadIdx.x;
-            if (row < R) xy[c] = uxy[row];
-        }
-    } else {
-        int start[kGroupTiles];
-#pragma unroll
-        for (int g = 0; g < kGroupTiles; ++g) {
-            start[g] = R;
-            if (g == warp) my_base[0] = R;
-            if (g == 4 + warp) my_base[1] = R;
-            R += cnts[g];
-        }
-#pragma unroll
-        for (int c = 0; c < 2; ++c) {
-            const int row = kRows * c + (int)threadIdx.x;
-            if (row < R) {
-                int g = 0, b = 0;
-#pragma unroll
-                for (int k = 1; k < kGroupTiles; ++k) {
-                    if (row >= start[k]) {
-                        g = k;
-                        b = start[k];
-                    }
-                }
-                xy[c] = texlist[32 * g + ck(row - b, 32, p.err, kBndTexList)];
-            }
-        }
+    for (int c = 0; c < 2; ++c) {
+        const int row = kRows * c + (int)threadIdx.x;
+        if (row < R) xy[c] = uxy[row];
     }
     if (threadIdx.x == 0) cnt.v[kStatTexelEvalsUnique] += R;
     __syncthreads();
@@ -679,12 +650,8 @@ __device__ __forceinline__ bool mlp_group(const ExactParams &p, const MlpDevice 
         tile_pos(tp, g, bx, by);
         const uint32_t idx =
             ck((uint32_t)(by * TH + ty) * (uint32_t)p.W + (uint32_t)(bx * TW + tx), view_pixels(p), p.err, kBndPixel);
-        const int b = h == 0 ? my_base[0] : my_base[1];
-        const bool dedup = p.group_dedup != 0;
         // row of list entry i of this tile
-        auto row_of = [&](uint32_t i) {
-            return ck(dedup ? (int)rowmap[32 * g + (int)i] : b + (int)i, 2 * kRows, p.err, kBndRow);
-        };
+        auto row_of = [&](uint32_t i) { return ck((int)rowmap[32 * g + (int)i], 2 * kRows, p.err, kBndRow); };
         float4 result = make_float4(0.f, 0.f, 0.f, 0.f);
         uint8_t cv = 0;
         if ((info >> 23) & 1u) {

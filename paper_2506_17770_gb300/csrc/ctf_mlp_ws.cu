@@ -1,12 +1,12 @@
 // ctf_mlp_ws.cu -- learned-decode filter with warps specialised by role, for
-// STF, Box and Mask Sampling on single views (with or without group_dedup).
+// STF, Box and Mask Sampling on single views with group_dedup.
 //
 // A CTA of 256 threads (four per SM) takes the groups of 8 pixel tiles g0,
 // g0 + G, ... (G = gridDim.x) in turn:
 //   - warpgroup 0 (warps 0-3, the consumer, 80 registers) owns the 128 TMEM
-//     lanes: for each group it packs the texel lists of the 8 tiles into
-//     rows, computes their features and runs the tcgen05 MLP chain(s) into a
-//     row-value buffer;
+//     lanes: for each group it merges the texel lists of the 8 tiles in a hash
+//     table, so that each distinct texel takes one row, computes the rows'
+//     features and runs the tcgen05 MLP chain(s) into a row-value buffer;
 //   - warpgroup 1 (warps 4-7, the producers, 48 registers, two tiles of the
 //     group each) runs step 1 of the collaborative flow for the next group
 //     while the consumer's MMAs execute, and gathers, filters and stores the
@@ -19,10 +19,12 @@
 // hand them over: full (step 1 done), empty (lists read), done (row values
 // written), gathered (row values read).  Every wait is bounded; a wait that
 // gives up records CTF_ERR_TIMEOUT and the waiting role stops, so the kernel
-// always ends.  Each group gets the same rows, texel values, image and counts
-// as mlp_group in ctf_mlp_chain.cuh; with group_dedup the consumer merges
-// the group's lists in a hash table first, so that each distinct texel takes
-// one row, and a per-stage row map sends every list entry to its row.
+// always ends.  A per-stage row map sends every list entry to its texel's row;
+// each group gets the same texel values, image and counts as mlp_group in
+// ctf_mlp_chain.cuh.
+// Launched plainly (here and in ctf_mlp_ext.cu, ctf_mlp.cu and the batch kernel
+// of ctf_batch.cu that shares the chain): the kernels of options off the main
+// path, whose gain from an early start was not measured.
 #include <cstdint>
 #include <mutex>
 #include <set>
@@ -57,9 +59,8 @@ constexpr int kWsTex = 0;                                    // 256 x int2 texel
 constexpr int kWsST = kWsTex + 256 * 8;                      // 256 x float2 (s, t)
 constexpr int kWsInfo = kWsST + 256 * 8;                     // 256 x uint32 per-pixel words
 constexpr int kWsCount = kWsInfo + 256 * 4;                  // 8 x int texels per tile (producers)
-constexpr int kWsBase = kWsCount + 32;                       // 8 x int first row per tile (consumer)
-constexpr int kWsOut = kWsBase + 32;                         // 256 x float4 row values
-constexpr int kWsRowMap = kWsOut + 256 * 16;                 // 256 x u8 list entry -> row (group_dedup)
+constexpr int kWsOut = kWsCount + 32;                        // 256 x float4 row values
+constexpr int kWsRowMap = kWsOut + 256 * 16;                 // 256 x u8 list entry -> row
 constexpr int kWsStageBytes = kWsRowMap + 256;
 constexpr int kWsBars = kWsStage0 + 2 * kWsStageBytes;       // full[2], empty[2], done[2], gathered[2]
 constexpr int kWsBytes = kWsBars + 8 * 8;
@@ -314,7 +315,7 @@ __device__ __forceinline__ void ws_step1(const ExactParams &p, long long first, 
 // (its row values written by the consumer): gather, filter, store.
 template <int TW>
 __device__ __forceinline__ void ws_gather(const ExactParams &p, long long first, int g, const unsigned char *st,
-                                          int lane, bool dedup) {
+                                          int lane) {
     constexpr int TH = 32 / TW;
     const int tx = lane % TW, ty = lane / TW;
     const float2 *pix_st = reinterpret_cast<const float2 *>(st + kWsST);
@@ -322,11 +323,8 @@ __device__ __forceinline__ void ws_gather(const ExactParams &p, long long first,
     const float4 *outrow = reinterpret_cast<const float4 *>(st + kWsOut);
     const uint32_t info = pix_info[32 * g + lane];
     if (!((info >> 24) & 1u)) return;  // outside the frame (or no tile)
-    // the slot's first row, from the consumer (the other slots' counts may
-    // already belong to a later group)
-    const int base = reinterpret_cast<const int *>(st + kWsBase)[g];
     const unsigned char *rowmap = st + kWsRowMap + 32 * g;
-    auto row_of = [&](uint32_t i) { return ck(dedup ? (int)rowmap[i] : base + (int)i, 2 * kRows, p.err, kBndRow); };
+    auto row_of = [&](uint32_t i) { return ck((int)rowmap[i], 2 * kRows, p.err, kBndRow); };
     int bx, by;
     tile_pos(tile_pos0(p, first), g, bx, by);
     const uint32_t idx =
@@ -357,9 +355,8 @@ __device__ __forceinline__ void ws_gather(const ExactParams &p, long long first,
     if (p.evals) p.evals[idx] = cv;
 }
 
-// kDedup: group_dedup (the variant without it carries no code for it).  kFp8:
-// an E4M3 network (one kind of MMA in a kernel).
-template <int ALG, int TW, int MD, bool kDedup, bool kFp8>
+// kFp8: an E4M3 network (one kind of MMA in a kernel).
+template <int ALG, int TW, int MD, bool kFp8>
 __global__ void __launch_bounds__(kWsThreads, 4) mlp_filter_ws_kernel(const ExactParams p, const MlpDevice m,
                                                                       int *err) {
     extern __shared__ __align__(1024) unsigned char sm[];
@@ -383,7 +380,6 @@ __global__ void __launch_bounds__(kWsThreads, 4) mlp_filter_ws_kernel(const Exac
     for (int i = 0; i < kNumStats; ++i) cnt.v[i] = 0;
     const long long n_groups = (p.n_tiles + kGroupTiles - 1) / kGroupTiles;
     const long long G = gridDim.x;
-    constexpr bool dedup = kDedup;
 
     if (warp < 4) {
         // ---------------- consumer ----------------
@@ -412,88 +408,63 @@ __global__ void __launch_bounds__(kWsThreads, 4) mlp_filter_ws_kernel(const Exac
             }
             const int *count = reinterpret_cast<const int *>(st + kWsCount);
             int2 *texlist = reinterpret_cast<int2 *>(st + kWsTex);
-            int R = 0;
             int2 xy[2] = {make_int2(0, 0), make_int2(0, 0)};
-            if (dedup) {
-                // the distinct texels of the group get rows in the order their
-                // first list entries win a 512-slot hash table (in H, which no
-                // MMA reads between chains); the row map sends every list
-                // entry to its texel's row
-                unsigned long long *hkey = reinterpret_cast<unsigned long long *>(sm + kSmH);
-                unsigned char *hrow = sm + kSmH + 512 * 8;
-                int *nuniq = reinterpret_cast<int *>(sm + kSmH + 512 * 8 + 512);
-                for (int i = tid; i < 512; i += kRows) hkey[i] = ~0ull;
-                if (tid == 0) *nuniq = 0;
-                cons_sync();
-                int slot[2] = {0, 0};
-                bool has[2] = {false, false}, won[2] = {false, false};
-                int2 t2[2] = {make_int2(0, 0), make_int2(0, 0)};
+            // the distinct texels of the group get rows in the order their
+            // first list entries win a 512-slot hash table (in H, which no
+            // MMA reads between chains); the row map sends every list
+            // entry to its texel's row
+            unsigned long long *hkey = reinterpret_cast<unsigned long long *>(sm + kSmH);
+            unsigned char *hrow = sm + kSmH + 512 * 8;
+            int *nuniq = reinterpret_cast<int *>(sm + kSmH + 512 * 8 + 512);
+            for (int i = tid; i < 512; i += kRows) hkey[i] = ~0ull;
+            if (tid == 0) *nuniq = 0;
+            cons_sync();
+            int slot[2] = {0, 0};
+            bool has[2] = {false, false}, won[2] = {false, false};
+            int2 t2[2] = {make_int2(0, 0), make_int2(0, 0)};
 #pragma unroll
-                for (int c = 0; c < 2; ++c) {
-                    const int e = tid + kRows * c, g = e >> 5;
-                    int n_g = count[0];
+            for (int c = 0; c < 2; ++c) {
+                const int e = tid + kRows * c, g = e >> 5;
+                int n_g = count[0];
 #pragma unroll
-                    for (int k = 1; k < kGroupTiles; ++k) n_g = g == k ? count[k] : n_g;
-                    if ((e & 31) < n_g) {
-                        has[c] = true;
-                        t2[c] = texlist[e];
-                        const unsigned long long key =
-                            ((unsigned long long)(uint32_t)t2[c].y << 32) | (uint32_t)t2[c].x;
-                        unsigned h = (((uint32_t)t2[c].x * 0x9E3779B1u) ^ ((uint32_t)t2[c].y * 0x85EBCA77u)) >> 23;
-                        // at most 256 keys in 512 slots: the probe always ends
-                        for (int probe = 0; probe < 512; ++probe) {
-                            const unsigned long long old = atomicCAS(&hkey[h], ~0ull, key);
-                            if (old == ~0ull || old == key) {
-                                won[c] = old == ~0ull;
-                                slot[c] = (int)h;
-                                break;
-                            }
-                            h = (h + 1) & 511u;
+                for (int k = 1; k < kGroupTiles; ++k) n_g = g == k ? count[k] : n_g;
+                if ((e & 31) < n_g) {
+                    has[c] = true;
+                    t2[c] = texlist[e];
+                    const unsigned long long key =
+                        ((unsigned long long)(uint32_t)t2[c].y << 32) | (uint32_t)t2[c].x;
+                    unsigned h = (((uint32_t)t2[c].x * 0x9E3779B1u) ^ ((uint32_t)t2[c].y * 0x85EBCA77u)) >> 23;
+                    // at most 256 keys in 512 slots: the probe always ends
+                    for (int probe = 0; probe < 512; ++probe) {
+                        const unsigned long long old = atomicCAS(&hkey[h], ~0ull, key);
+                        if (old == ~0ull || old == key) {
+                            won[c] = old == ~0ull;
+                            slot[c] = (int)h;
+                            break;
                         }
+                        h = (h + 1) & 511u;
                     }
                 }
-                cons_sync();  // every list entry is in the table; the lists have been read
+            }
+            cons_sync();  // every list entry is in the table; the lists have been read
 #pragma unroll
-                for (int c = 0; c < 2; ++c) {
-                    if (won[c]) {
-                        const int row = ck(atomicAdd(nuniq, 1), 2 * kRows, p.err, kBndRow);
-                        hrow[slot[c]] = (unsigned char)row;
-                        texlist[row] = t2[c];  // the distinct texels reuse the list space
-                    }
+            for (int c = 0; c < 2; ++c) {
+                if (won[c]) {
+                    const int row = ck(atomicAdd(nuniq, 1), 2 * kRows, p.err, kBndRow);
+                    hrow[slot[c]] = (unsigned char)row;
+                    texlist[row] = t2[c];  // the distinct texels reuse the list space
                 }
-                cons_sync();
-                unsigned char *rowmap = st + kWsRowMap;
+            }
+            cons_sync();
+            unsigned char *rowmap = st + kWsRowMap;
 #pragma unroll
-                for (int c = 0; c < 2; ++c)
-                    if (has[c]) rowmap[tid + kRows * c] = hrow[slot[c]];
-                R = *nuniq;
+            for (int c = 0; c < 2; ++c)
+                if (has[c]) rowmap[tid + kRows * c] = hrow[slot[c]];
+            const int R = *nuniq;
 #pragma unroll
-                for (int c = 0; c < 2; ++c) {
-                    const int row = kRows * c + tid;
-                    if (row < R) xy[c] = texlist[row];
-                }
-            } else {
-                // slot g owns rows [base_g, base_g + count[g]) in slot order
-                int start[kGroupTiles];
-#pragma unroll
-                for (int g = 0; g < kGroupTiles; ++g) {
-                    start[g] = R;
-                    R += count[g];
-                }
-#pragma unroll
-                for (int c = 0; c < 2; ++c) {
-                    const int row = kRows * c + tid;
-                    if (row < R) {
-                        int g = 0;
-#pragma unroll
-                        for (int k = 1; k < kGroupTiles; ++k) g = row >= start[k] ? k : g;
-                        int b = start[0];
-#pragma unroll
-                        for (int k = 1; k < kGroupTiles; ++k) b = k == g ? start[k] : b;
-                        xy[c] = texlist[32 * g + ck(row - b, 32, p.err, kBndTexList)];
-                    }
-                }
-                if (tid < kGroupTiles) reinterpret_cast<int *>(st + kWsBase)[tid] = start[tid];
+            for (int c = 0; c < 2; ++c) {
+                const int row = kRows * c + tid;
+                if (row < R) xy[c] = texlist[row];
             }
             if (tid == 0) cnt.v[kStatTexelEvalsUnique] += R;
             cons_sync();  // every consumer thread has read the lists, counts and distinct texels
@@ -552,8 +523,7 @@ __global__ void __launch_bounds__(kWsThreads, 4) mlp_filter_ws_kernel(const Exac
                 }
 #pragma unroll 1
                 for (int k = 0; k < kWsSlotsPerProducer; ++k)
-                    ws_gather<TW>(p, (grp - G) * kGroupTiles, kWsSlotsPerProducer * pw + k, ws_stage(sm, s1), lane,
-                                  dedup);
+                    ws_gather<TW>(p, (grp - G) * kGroupTiles, kWsSlotsPerProducer * pw + k, ws_stage(sm, s1), lane);
                 __syncwarp();
                 if (lane == 0) mbar_arrive(ws_bar(sm, kBarGathered, s1));
             }
@@ -573,14 +543,14 @@ __global__ void __launch_bounds__(kWsThreads, 4) mlp_filter_ws_kernel(const Exac
 
 using WsFn = void (*)(const ExactParams, const MlpDevice, int *);
 
-template <int TW, bool kDedup, bool kFp8>
+template <int TW, bool kFp8>
 WsFn ws_pick(int alg, int md) {
     switch (alg) {
-    case ALG_STF: return mlp_filter_ws_kernel<ALG_STF, TW, 16, kDedup, kFp8>;
-    case ALG_BOX: return mlp_filter_ws_kernel<ALG_BOX, TW, 16, kDedup, kFp8>;
+    case ALG_STF: return mlp_filter_ws_kernel<ALG_STF, TW, 16, kFp8>;
+    case ALG_BOX: return mlp_filter_ws_kernel<ALG_BOX, TW, 16, kFp8>;
     case ALG_MASK:
-        return md == 11 ? mlp_filter_ws_kernel<ALG_MASK, TW, 11, kDedup, kFp8>
-                        : mlp_filter_ws_kernel<ALG_MASK, TW, 16, kDedup, kFp8>;
+        return md == 11 ? mlp_filter_ws_kernel<ALG_MASK, TW, 11, kFp8>
+                        : mlp_filter_ws_kernel<ALG_MASK, TW, 16, kFp8>;
     default: return nullptr;
     }
 }
@@ -604,14 +574,11 @@ cudaError_t ws_prepare(WsFn fn) {
     return e;
 }
 
-// Only the group_dedup variant is launched: without the option the
-// producers compute the features themselves (ctf_mlp_ws2.cu).
-WsFn ws_kernel(int alg, int tile_w, int mask_dim, bool dedup, bool fp8) {
-    if (!dedup) return nullptr;
+WsFn ws_kernel(int alg, int tile_w, int mask_dim, bool fp8) {
     switch (tile_w) {
-    case 8: return fp8 ? ws_pick<8, true, true>(alg, mask_dim) : ws_pick<8, true, false>(alg, mask_dim);
-    case 4: return fp8 ? ws_pick<4, true, true>(alg, mask_dim) : ws_pick<4, true, false>(alg, mask_dim);
-    case 16: return fp8 ? ws_pick<16, true, true>(alg, mask_dim) : ws_pick<16, true, false>(alg, mask_dim);
+    case 8: return fp8 ? ws_pick<8, true>(alg, mask_dim) : ws_pick<8, false>(alg, mask_dim);
+    case 4: return fp8 ? ws_pick<4, true>(alg, mask_dim) : ws_pick<4, false>(alg, mask_dim);
+    case 16: return fp8 ? ws_pick<16, true>(alg, mask_dim) : ws_pick<16, false>(alg, mask_dim);
     default: return nullptr;
     }
 }
@@ -624,7 +591,7 @@ bool mlp_filter_ws_applies(const ExactParams &, int alg) {
 
 cudaError_t prepare_mlp_filter_ws(int alg, int tile_w, int mask_dim) {
     for (int fp8 = 0; fp8 < 2; ++fp8) {
-        WsFn fn = ws_kernel(alg, tile_w, mask_dim, true, fp8 != 0);
+        WsFn fn = ws_kernel(alg, tile_w, mask_dim, fp8 != 0);
         const cudaError_t e = fn ? ws_prepare(fn) : cudaErrorInvalidValue;
         if (e != cudaSuccess) return e;
     }
@@ -633,7 +600,7 @@ cudaError_t prepare_mlp_filter_ws(int alg, int tile_w, int mask_dim) {
 
 cudaError_t launch_mlp_filter_ws(const ExactParams &p, const MlpDevice &m, int alg, int tile_w, int mask_dim,
                                  int *err, cudaStream_t stream) {
-    WsFn fn = ws_kernel(alg, tile_w, mask_dim, p.group_dedup != 0, m.fp8 != 0);
+    WsFn fn = ws_kernel(alg, tile_w, mask_dim, m.fp8 != 0);
     if (!fn) return cudaErrorInvalidValue;
     if (p.n_tiles == 0) return cudaSuccess;
     if (p.n_tiles > 0x7fffffffLL) return cudaErrorInvalidValue;  // tile positions use 32-bit arithmetic
