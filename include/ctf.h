@@ -318,10 +318,10 @@ int ctf_debug_fail_launches(int skip, int n);
  * -DCTF_DEBUG): the same entry points and results, and every data-dependent
  * index its kernels use to reach a texel (block or latent cell), a pixel of
  * the view, or an entry of a shared-memory table (decode tables, rank
- * slots, List Merge and fallback tables, texel lists, chain rows, per-pixel
- * words) is checked against its buffer first.  An index outside it is
- * recorded in the device error word and replaced by 0, so the access stays
- * inside the buffer and the kernel runs on to its end (no trap); the next
+ * slots, fallback tables, texel lists, chain rows, per-pixel words) is
+ * checked against its buffer first.  An index outside it is recorded in the
+ * device error word and replaced by 0, so the access stays inside the buffer
+ * and the kernel runs on to its end (no trap); the next
  * ctf_sync_check returns CTF_ERR_BOUNDS, and ctf_last_error names the site,
  * the index and the bound of the first record.
  * ctf_debug_build returns 1 in that library and 0 in the release one.

@@ -8,13 +8,16 @@
 // Block views: persistent CTAs of 8 warps, like the per-view exact kernel;
 // every warp takes items of 32 consecutive warp tiles of one view from an
 // atomic counter (lane 0 fetches the next item while the current one runs)
-// and walks them with the next tile's inputs prefetched.  Learned views:
-// persistent CTAs of 4 warps that hold 128 TMEM columns for the whole launch;
-// the CTA takes items of 8 warp tiles (two per warp, their texel lists packed
-// into shared MLP chains; 4 tiles, one per warp, for per-pixel 4-tap),
-// `items_per_fetch` at a time.  A prefix over each kind's per-view item
-// counts maps an item to its view; the prefixes of up to 1024 block views
-// (256 learned views) are cached in shared memory.
+// and walks them with the next tile's inputs prefetched.  Learned views run on
+// the packed-group kernel made persistent (mlp_batch_pf_kernel,
+// ctf_mlp_ws2.cu), CTA c the items c, c + G, ... of 8 warp tiles; those with
+// per-pixel 4-tap or group_dedup on the kernel here, persistent CTAs of 4 warps
+// that hold 128 TMEM columns for the whole launch and take items of 8 warp
+// tiles (two per warp, their texel lists packed into shared MLP chains; 4
+// tiles, one per warp, for per-pixel 4-tap), `items_per_fetch` at a time.  A
+// prefix over each kind's per-view item counts maps an item to its view; the
+// prefixes of up to 1024 block views (256 learned views of the kernel here) are
+// cached in shared memory.
 // Fetching is a plain fetch-and-add: no thread ever waits on another CTA.
 #include <algorithm>
 #include <cstdint>
@@ -84,9 +87,10 @@ constexpr int batch_min_blocks() {
     return ALG >= ALG_LIST ? 4 : 1;
 }
 
-// kStats: the variant that keeps the outcome counters (its registers spill;
-// 256 views of 64..512^2, half of them blocks: 163 us with, for every call
-// before, see below for without).
+// kStats: the variant that keeps the outcome counters (its registers spill; the
+// block half of 256 views of 64..512^2 took 163 us when every call kept them,
+// 131 now).
+// The variant with fallbacks exists with counters only.
 template <int ALG, int TW, int MD, bool kFb, bool kStats>
 __global__ void __launch_bounds__(kBlockWarps * 32, batch_min_blocks<ALG>()) batch_block_kernel(const BatchParams b) {
     constexpr int TH = 32 / TW;
@@ -180,7 +184,9 @@ __global__ void __launch_bounds__(kBlockWarps * 32, batch_min_blocks<ALG>()) bat
 }
 
 // ---------------------------------------------------------------------------
-// Learned views: the 4 warps of a CTA share an MLP chain.
+// Learned views with per-pixel 4-tap or group_dedup: the 4 warps of a CTA share
+// an MLP chain.  (Single views of per-pixel 4-tap have a kernel with roles,
+// ctf_mlp_dense.cu, 1.8 times as fast; it has not been made persistent.)
 // ---------------------------------------------------------------------------
 template <int ALG, int TW, int MD>
 __global__ void __launch_bounds__(kRows, 4) batch_mlp_kernel(const BatchParams b) {
@@ -516,7 +522,7 @@ cudaError_t launch_plan(const Plan &plan, const DevPlan &dp, int alg, const Reso
         b.err = err;
         b.tables = k == 0 ? plan.views[plan.index[0][0]].p.tables : nullptr;
         if (k == 1 && mlp_batch_pf_applies(alg, r.group_dedup)) {
-            // learned views on the packed-group kernel (one group per fetch)
+            // learned views on the packed-group kernel
             e = launch_mlp_batch_pf(dp.views, (int)plan.views.size(), dp.index[1], dp.begin[1], b.nkind, b.total_items, stats,
                                     err, plan.views[plan.index[1][0]].m, *plan.epi[plan.index[1][0]], alg, r.tile_w,
                                     r.mask_dim, s);

@@ -196,7 +196,8 @@ bool mlp_batch_pf_applies(int alg, int group_dedup);
 int mlp_batch_pf_tiles();  // tiles of an item
 cudaError_t prepare_mlp_batch_pf(int alg, int tile_w, int mask_dim);
 cudaError_t launch_mlp_batch_pf(const BatchViewDev *views, int nviews, const int *index, const long long *item_begin,
-                                int nkind, long long total_items, unsigned long long *stats, int *err, const MlpDevice &m0, const MlpEpilogue &ep0, int alg, int tile_w, int mask_dim,
+                                int nkind, long long total_items, unsigned long long *stats, int *err,
+                                const MlpDevice &m0, const MlpEpilogue &ep0, int alg, int tile_w, int mask_dim,
                                 cudaStream_t s);
 
 // Error reporting shared by the C ABI translation units (ctf_api.cu).
@@ -237,7 +238,8 @@ cudaError_t launch_with(void (*fn)(Params...), bool dependent, int grid, int thr
 // ends: fn sets itself up, calls grid_wait (ctf_device.cuh) before it touches
 // anything that a kernel or copy before it may write or read, and grid_trigger
 // to let the next such kernel begin.  Before grid_wait it may read only what
-// stays the same while its texture exists (decode tables, operand images).
+// stays the same while its texture exists (decode tables, operand images);
+// the trainer's updates read more, and say what they rely on (advance_kernel).
 // After anything but such a kernel it starts like any other launch.
 // Back-to-back calls, us each, without and with: 1080p Mask-11 block view 22.6
 // and 20.8, with fallback C 29.5 and 26.2, with Catmull-Rom 51.0 and 46.4;

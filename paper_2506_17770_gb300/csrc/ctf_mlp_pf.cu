@@ -98,7 +98,8 @@ cudaError_t prepare_mlp_batch_pf(int alg, int tile_w, int mask_dim) {
 }
 
 cudaError_t launch_mlp_batch_pf(const BatchViewDev *views, int nviews, const int *index, const long long *item_begin,
-                                int nkind, long long total_items, unsigned long long *stats, int *err, const MlpDevice &m0, const MlpEpilogue &ep0, int alg, int tile_w, int mask_dim,
+                                int nkind, long long total_items, unsigned long long *stats, int *err,
+                                const MlpDevice &m0, const MlpEpilogue &ep0, int alg, int tile_w, int mask_dim,
                                 cudaStream_t s) {
     const PfKernels *k = kernels_of(tile_w);
     BatchPfFn fn = k ? k->batch(alg, mask_dim, stats != nullptr) : nullptr;

@@ -30,12 +30,15 @@
 // wait that gives up records CTF_ERR_TIMEOUT and both roles leave.
 // The roles share the work so that neither waits long: with the features on
 // the producers the consumer stood still for half of the time (4,500 of 8,600
-// clocks a group) and a 3840x2160 Mask-11 FP16 view took 198 us, now 193; in
+// clocks a group) and a 3840x2160 Mask-11 FP16 view took 198 us, now 193, with
+// the consumer the longer role: of 6,500 clocks a group it waits 460, and
+// spends 2,100 on features, 2,950 in its 1.23 chains and 950 on the gather; a
+// producer warp waits 2,900 and takes 3,450 for step 1 of its two tiles.  In
 // the batch kernel, whose parameters are read from shared memory, the features
 // stay on the producers (256 views 473 us, on the consumer 493).
-// What bounds it: instruction issue (about 700 warp instructions a tile at
-// 60-65% of the issue slots with 32 warps on an SM), not the tensor pipe and
-// not memory.  So the rows are given out by a counter rather than found by a
+// What bounds it: instruction issue (573 warp instructions a tile at 66% of the
+// issue slots with 32 warps on an SM) and the latency of the consumer's chain,
+// not the tensor pipe and not memory.  So the rows are given out by a counter rather than found by a
 // scan, a lane's place in a tile and the tile walk are computed once, FP8 is a
 // template parameter, and both roles run in the 64 registers of the launch
 // (no register split).  3840x2160 Mask-11 FP16: 276 us with the scan, 72/56
@@ -360,6 +363,16 @@ struct LanePlace {
 template <int ALG>
 constexpr bool p_tap_pairs() { return ALG == ALG_BOX || ALG == ALG_MASK; }
 
+// The inputs of the lane's pixel of the tile at (bx, by).  Every lane loads
+// (lanes outside the frame pixel 0, which exists), so that the loads carry no
+// predicates.
+template <int ALG, int TW>
+__device__ __forceinline__ Inputs p_load(const ExactParams &p, const LanePlace<TW> &lp, uint32_t bx, uint32_t by) {
+    constexpr uint32_t TH = 32 / TW;
+    return load_inputs_any<(ALG >= ALG_LIST)>(p, bx < lp.lim_x && by < lp.lim_y,
+                                              by * (TH * (uint32_t)p.W) + bx * TW + lp.off);
+}
+
 // Producer: step 1 on the tile at (bx, by), slot g of the group, into stage
 // st: per pixel (s, t) and a packed word (bits 0-19 the list indices of its 4
 // taps on success, else of its own texel; 20-22 its count; 23 active; 24
@@ -376,16 +389,6 @@ constexpr bool p_tap_pairs() { return ALG == ALG_BOX || ALG == ALG_MASK; }
 // texels): the pixel's word holds the 6-bit list indices of its taps (bits
 // 0-23, or of its own texel), its count (24-25), active (26), inside (27)
 // and success (28).
-// The inputs of the lane's pixel of the tile at (bx, by).  Every lane loads
-// (lanes outside the frame pixel 0, which exists), so that the loads carry no
-// predicates.
-template <int ALG, int TW>
-__device__ __forceinline__ Inputs p_load(const ExactParams &p, const LanePlace<TW> &lp, uint32_t bx, uint32_t by) {
-    constexpr uint32_t TH = 32 / TW;
-    return load_inputs_any<(ALG >= ALG_LIST)>(p, bx < lp.lim_x && by < lp.lim_y,
-                                              by * (TH * (uint32_t)p.W) + bx * TW + lp.off);
-}
-
 template <int ALG, int TW, int MD, bool kStats, bool kFb, bool kTwo = false>
 __device__ __forceinline__ void p_step1(const ExactParams &p, const LanePlace<TW> &lp, uint32_t bx, uint32_t by,
                                         const Inputs &in, int g, unsigned char *st, int lane, uint32_t lt, int *ranks,
@@ -670,7 +673,7 @@ __global__ void __launch_bounds__(kPThreads, kPCtasPerSm)
 #pragma unroll 1
                 for (int k = 0; k < kSlots; ++k) {
                     // the inputs of the warp's next tile come in while this one
-                    // is in step 1 (or the group's features are computed)
+                    // is in step 1 (or the warp waits for its next stage)
                     uint32_t nx = bx, ny = by;
                     if (k + 1 < kSlots) {
                         p_tile(tiles_x, nx, ny, 1u);

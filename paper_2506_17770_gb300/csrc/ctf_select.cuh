@@ -174,9 +174,9 @@ __device__ __forceinline__ ListUnion<kSide> list_union(bool active, int ox, int 
 // bounding box when the box is at most 16 x 16 (the same set, so the same n
 // and the same outputs, whichever lane evaluates a texel), list_union
 // otherwise.  A hash table in shared memory for every tile, which this
-// replaces, took 486 instructions a tile and 28.6 us for a 1283x797 view
-// (16.4 us with the union, 12.2 with what came after), and 129 us against 77 us
-// for a 1920x1080 FP8 learned view (60 now).
+// replaces, took 486 instructions a tile and 28.6 us for a 1283x797 view of
+// smooth tiles (16.4 us with the masks, 12.2 with what came after), and 129 us
+// against 77 us for a 1920x1080 FP8 learned view (60 now).
 // kTwo: the variant that may evaluate two texels per lane (p.tpl == 2); the
 // other carries no code for it.
 template <int ALG, int MD, bool kStats, bool kUnique = true, bool kTwo = false>

@@ -64,7 +64,7 @@ struct GradParams {
     long long *loss;       // fixed-point sum of squared errors
     int *err;              // device error word: a wait that gave up records CTF_ERR_TIMEOUT
     unsigned char *wimg;   // the weight image of the gradient kernel (pack_kernel)
-    float *partial;        // per-CTA weight-gradient sums [CTA][kWeights] (reduce_kernel adds them up)
+    float *partial;        // per-CTA weight-gradient sums [CTA][kWeights], added up in CTA order
 };
 
 // v * 2^44 is exact in FP32 (a power-of-two scale), so this rounds the same
@@ -595,8 +595,8 @@ __global__ void __launch_bounds__(kT, 2) grad_kernel(const GradParams g) {
     }
     if (ok) ok = !__syncthreads_or(bad);
     // ---- the CTA's weight-gradient sums, row m = tid of the two products,
-    // stored as this CTA's partial sums (reduce_kernel adds the CTAs' up in
-    // CTA order: no atomics on the few thousand weight entries)
+    // stored as this CTA's partial sums (added up in CTA order: no atomics on
+    // the few thousand weight entries)
     if (ok) {
         float *W = g.partial + (size_t)ck((int)blockIdx.x, kMaxGradCtas, g.err, kBndTrain) * kWeights;
         const int m = tid;
@@ -640,8 +640,9 @@ __global__ void __launch_bounds__(kT, 2) grad_kernel(const GradParams g) {
     }
 }
 
-// The weight gradients: the CTAs' partial sums added up in CTA order (FP64),
-// times 2 / batch, into the fixed-point accumulators.  A block takes 16
+// The weight gradients (ctf_trainer_gradients; a step's update adds them up the
+// same way itself): the CTAs' partial sums added up in CTA order (FP64), times
+// 2 / batch, into the fixed-point accumulators.  A block takes 16
 // entries; its 16 thread rows each add every 16th CTA in order (loads
 // issued 8 at a time), and the 16 row sums are added in row order, so the
 // result does not depend on timing.
@@ -773,6 +774,12 @@ __device__ __forceinline__ void update_weights(const AdamParams &a, const AdamSt
 // weights take step j.  Two threads per cell, sixteen per texel; the first to
 // reach a cell claims it.  Only cells that step j reads too (`late`) wait for
 // its gradients; the gradient kernel neither reads nor changes the others.
+// What it reads and claims before that wait (`seen`, parameters, moments,
+// accumulators) the update before wrote.  griddepcontrol.wait would order only
+// what the gradient kernel wrote; that the update before is over rests on the
+// gradient kernel, which lets this one begin only after its own wait for it, and
+// that its results are seen on the loads (__ldcg), stores and atomics, which
+// meet in L2 and leave no line of these arrays in an SM's L1.
 // 4096^2 texture, 8,192 texels: 34 us a step in a call of 64 (gradients and
 // advance 29, a sixteenth of a sweep 6); 66 us in calls of one step, whose
 // sweep moves every parameter, and 93 us with an Adam kernel of all cells and
@@ -857,7 +864,8 @@ __global__ void __launch_bounds__(kSweepThreads, kSweepCtasPerSm) sweep_kernel(c
         return a.descending ? nq - 1 - c : c;
     };
     // parameters and moments do not change before the wait (of the cells that
-    // step j reads, neither does `seen`, but in a segment's first step)
+    // step j reads, neither does `seen`, but in a segment's first step); the
+    // update before is over by now, as in advance_kernel
     size_t q = quad_at(i);
     float4 p = __ldcg(P + q), m = __ldcg(M + q), v = __ldcg(V + q);
     grid_wait();
