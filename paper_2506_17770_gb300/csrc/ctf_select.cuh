@@ -90,7 +90,7 @@ struct Selection {
 // stands for the texel in the list.  A tile leaves with the class that takes
 // it over budget.
 // 1920x1080 block views whose tiles see 2 to 32 spots, us: 37 to 62, with two
-// texels per lane 44 to 91, with Catmull-Rom 43 to 65 (16 texels a pixel).
+// texels per lane 45 to 93, with Catmull-Rom 43 to 65 (16 texels a pixel).
 // One texel a turn took 94 to 120, 115 to 243 and 457, a hash table in shared
 // memory 60 to 75, 66 to 103 and 66 to 104; cells of 8 x 4 texels in turn 52
 // to 83, 59 to 120 and 44 to 51.
@@ -114,7 +114,10 @@ __device__ __forceinline__ ListUnion<kSide> list_union(bool active, int ox, int 
     u.tx = u.tx2 = ox;
     u.ty = u.ty2 = oy;
     int n = 0;
-#pragma unroll
+    // (by_class by constant indices; with the four classes of 2 x 2 unrolled too
+    // the packed-group kernel, which is short of instruction cache, is 0.4% slower)
+    constexpr int kUnroll = kSide == 2 ? 1 : kSide;
+#pragma unroll kUnroll
     for (int cy = 0; cy < kSide; ++cy) {
         const int y = oy + ((cy - oy) & (kSide - 1));
 #pragma unroll 1
@@ -134,7 +137,7 @@ __device__ __forceinline__ ListUnion<kSide> list_union(bool active, int ox, int 
                 return u;
             }
             const int c = cx + kSide * cy;
-            by_class[c >> 2] |= (uint32_t)i << (8 * (c & 3));
+            by_class[kSide == 2 ? 0 : cy] |= (uint32_t)i << (8 * (c & 3));
             if (first) ranks[ck(i, kRanksN, err, kBndRanks)] = 32 * c + lane;
         }
     }
